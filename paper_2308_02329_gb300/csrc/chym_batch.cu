@@ -52,52 +52,6 @@ struct chym_batch {
   double part_units[9] = {};
 };
 
-namespace chym {
-namespace {
-
-struct PlanJob {
-  int desc, n_runs;
-};
-
-// Split the runs of `jobs` (all of one dimension) over P CTAs in near-equal chunk
-// counts; items never cross a context and hold at most `per_item` runs.
-void plan_dimension(const std::vector<PlanJob>& jobs, int CH, int per_item, int P,
-                    std::vector<unsigned char>& items, std::vector<int>& cta_begin) {
-  long long C = 0;
-  for (const auto& j : jobs) C += (j.n_runs + CH - 1) / CH;
-  if (P > C) P = (int)std::max(1LL, C);
-  const size_t ib = tc_item_bytes();
-  cta_begin.assign(1, 0);
-  int cta = 0;
-  long long acc = 0;
-  auto bound = [&](int b) { return (long long)llround((double)(b + 1) * (double)C / P); };
-  int n_items = 0;
-  for (const auto& j : jobs) {
-    int run = 0;
-    while (run < j.n_runs) {
-      long long cap = bound(cta) - acc;
-      if (cap <= 0 && cta + 1 < P) {
-        cta_begin.push_back(n_items);
-        ++cta;
-        continue;
-      }
-      if (cap <= 0) cap = (j.n_runs - run + CH - 1) / CH;  // last CTA takes the rest
-      const int left_chunks = (j.n_runs - run + CH - 1) / CH;
-      const int take = (int)std::min<long long>({cap, (long long)(per_item / CH), (long long)left_chunks});
-      const int runs = std::min(take * CH, j.n_runs - run);
-      items.resize(items.size() + ib);
-      tc_fill_item(items.data() + items.size() - ib, j.desc, run, runs);
-      ++n_items;
-      run += runs;
-      acc += take;
-    }
-  }
-  while ((int)cta_begin.size() < P + 1) cta_begin.push_back(n_items);
-}
-
-}  // namespace
-}  // namespace chym
-
 using namespace chym;
 
 extern "C" {
@@ -224,7 +178,7 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
       desc_of[i] = n_desc++;
     }
   struct DimLaunch {
-    int D, P, kp_max, terms_max;
+    int D, P, kp_max, terms_max, chunk;
     size_t items_off, cta_off;
     bool stall;
   };
@@ -240,7 +194,7 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     P = std::max(P, 1);
     sms_left -= P;
     --dims_left;
-    std::vector<PlanJob> jobs;
+    std::vector<TcJob> jobs;
     int kp_max = 16, terms_max = 1;
     bool stall = false;
     for (int i : by_dim[D]) {
@@ -251,8 +205,11 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     }
     std::vector<unsigned char> items;
     std::vector<int> cta;
-    plan_dimension(jobs, tc_chunk_runs(D), tc_runs_per_item(D), P, items, cta);
-    DimLaunch L{D, (int)cta.size() - 1, kp_max, terms_max, 0, 0, stall};
+    long long runs = 0;
+    for (const auto& j : jobs) runs += j.n_runs;
+    const int chunk = b->shapes.ch[D] ? b->shapes.ch[D] : tc_pick_chunk(D, runs, P);
+    tc_plan_items(jobs, chunk, tc_runs_per_item(D), P, items, cta);
+    DimLaunch L{D, (int)cta.size() - 1, kp_max, terms_max, chunk, 0, 0, stall};
     b->part_ctas[D] = L.P;
     b->part_units[D] = 0.0;
     for (const auto& jj : jobs) b->part_units[D] += (double)((jj.n_runs + tc_chunk_runs(D) - 1) / tc_chunk_runs(D));
@@ -286,7 +243,7 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     if (b->timing) CHYM_CUDA_TRY(cudaEventRecord(b->t_begin[L.D], s));
     CHYM_CUDA_TRY(launch_tc_items(L.D, base, base + L.items_off, (const int*)(base + L.cta_off), L.P,
                                   steps, L.kp_max, L.terms_max, b->d_status, s, L.stall,
-                                  b->shapes.ch[L.D]));
+                                  L.chunk));
     if (b->timing) {
       CHYM_CUDA_TRY(cudaEventRecord(b->t_end[L.D], s));
       b->timed[L.D] = true;

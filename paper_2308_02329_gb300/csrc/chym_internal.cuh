@@ -266,7 +266,17 @@ int tc_groups(int D);  // warpgroups of a CTA: the chunks it advances side by si
 size_t tc_desc_bytes();
 size_t tc_item_bytes();
 void tc_fill_desc(const chym_ctx* c, const StepConsts& sc, void* out);
-void tc_fill_item(void* out, int desc, int run_begin, int run_count);
+// Runs of one context of a plan: index of its descriptor and run count.
+struct TcJob {
+  int desc, n_runs;
+};
+// runs per epilogue chunk for `runs` runs of dimension D on P CTAs
+int tc_pick_chunk(int D, long long runs, int P);
+// Split the runs of `jobs` (all of one dimension) over at most P CTAs in near-equal
+// numbers of `chunk`-run chunks; items never cross a context and hold at most `per_item`
+// runs.  items: packed TcItem records; cta_begin: first item of each CTA, and the end.
+void tc_plan_items(const std::vector<TcJob>& jobs, int chunk, int per_item, int P,
+                   std::vector<unsigned char>& items, std::vector<int>& cta_begin);
 cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, const int* d_cta_begin,
                             int n_cta, int64_t steps, int kp_max, int terms_max, unsigned* status,
                             cudaStream_t st, bool test_stall = false, int chunk = 0);

@@ -1,0 +1,34 @@
+"""Small-N tensor-core path: a run's trajectory does not depend on how the runs of its
+context are spread over the SMs (chunk length, items per CTA, runs per group)."""
+import numpy as np
+import pytest
+
+from paper_2308_02329_gb300 import chym, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,D", [(20, 1), (100, 2), (33, 3), (128, 4), (17, 5), (64, 8)])
+@pytest.mark.parametrize("R", [1, 3, 609, 2432, 2433, 10007])
+def test_spread_of_the_runs_leaves_states_unchanged(N, D, R):
+    J = inputs.gaussian(N, 3) if D == 3 else inputs.sk_pm1(N, 3)
+    ctx = chym.Context(J, D, chym.J_REAL if D == 3 else chym.J_PM1)
+    prm = chym.Params(eps=0.25 if D == 3 else 0.25 / np.sqrt(N), prec=chym.PREC_BF16X2)
+    sched = chym.Schedule(1, 3, 9)
+    seeds = inputs.run_seeds(21, R)
+    ctx.run(prm, np.array([0.8]), seeds, 7, sched)
+    X, k = ctx.get_state()
+    assert k == 7
+    # the last runs again, alone: 5 runs take other CTAs, groups and chunks
+    few = min(R, 5)
+    ctx.run(prm, np.array([0.8]), seeds[R - few:], 7, sched)
+    Y, _ = ctx.get_state()
+    assert np.array_equal(X[R - few:], Y)
+    # and all of them as a batch
+    ctx.run(prm, np.array([0.8]), seeds, 0, sched)
+    b = chym.Batch([ctx])
+    b.run([prm], [sched], 7)
+    b.status()
+    assert np.array_equal(ctx.get_state()[0], X)
+    b.close()
+    ctx.close()
