@@ -276,6 +276,7 @@ chym_status chym_create(const double* J, int N, int D, chym_jkind kind, chym_ctx
       e = cudaMemcpy(c->d_Jbits, planes.data(), planes.size() * sizeof(uint64_t), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_jdeg, deg.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice);
   }
+  if (e == cudaSuccess && kind == CHYM_J_REAL) e = prepare_energy_digits(c);  // for the Ising energy
   // sparse J: compressed rows for the CUDA-core product
   size_t nz = 0;
   for (size_t i = 0; i < nn; ++i) nz += J[i] != 0.0;
@@ -328,6 +329,8 @@ chym_status chym_destroy(chym_ctx* c) {
   free_dev(c->d_J8);
   free_dev(c->d_Jbits);
   free_dev(c->d_jdeg);
+  free_dev(c->d_Jdig);
+  free_dev(c->d_Jexp);
   free_dev(c->d_Jbf16);
   free_dev(c->d_X);
   free_dev(c->d_h);

@@ -184,6 +184,10 @@ struct chym_ctx {
   // plane 1: J = -1; word w holds columns 64 w .. 64 w + 63), and per row (#+1) - (#-1)
   uint64_t* d_Jbits = nullptr;
   int32_t* d_jdeg = nullptr;
+  // real couplings: J in fixed point for the Ising energy, row p scaled by 2^d_Jexp[p], as
+  // FP16 digit planes in tensor-core fragments
+  void* d_Jdig = nullptr;
+  int32_t* d_Jexp = nullptr;
   // J in compressed rows when it is sparse (at most N^2 / 16 nonzeros): the coupling
   // product then runs on the CUDA cores over the nonzeros only
   bool sparse = false;
@@ -291,6 +295,7 @@ struct TileShapes {
 inline bool k2_rt_valid(int D, int rt) {
   return rt >= 32 && rt % 32 == 0 && D * rt <= 256 && (D * rt) % 16 == 0;
 }
+cudaError_t prepare_energy_digits(chym_ctx* c);
 cudaError_t launch_energy(chym_ctx* c, double* d_E, uint64_t* d_spins, cudaStream_t st);
 cudaError_t launch_energy_segments(chym_ctx* c, const SegTable& t, double* d_E, cudaStream_t st);
 cudaError_t launch_stats(chym_ctx* c, const double* d_E, double E_gs, double tol, double bin_w,
