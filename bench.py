@@ -1007,15 +1007,14 @@ def measure(args, w, sim_steps, rank, world, local, warm_steps=None, replay=Fals
         # statistics per context (a pack of graphs: pump indices, init and one segment
         # energy launch, its statistics are host-side); one persistent launch per
         # dimension for the small-N contexts; the large-N path adds 3 layout kernels per
-        # context, one grouped GEMM launch per dimension and integration step, and one
-        # step-counter kernel per 16-step graph; FP32/FP64 contexts and sparse ones take
-        # one persistent SIMT launch each
+        # context and one persistent launch per dimension and 1024 integration steps; FP32/FP64
+        # contexts and sparse ones take one persistent SIMT launch each
         bf16 = prec in (chym.PREC_BF16X2, chym.PREC_FP8)
         small = [j for j in jobs if j["N"] <= 128 and bf16]
         large = [j for j in jobs if j["N"] > 128 and bf16 and not j["ctx"].uses_csr(prec)]
         sparse = [j for j in jobs if j["ctx"].uses_csr(prec)]
         per_step = sum(3 if "seg" in j else 4 for j in jobs) + len({j["D"] for j in small}) + \
-            3 * len(large) + (sim_steps * len({j["D"] for j in large}) + sim_steps // 16 if large else 0) + (
+            3 * len(large) + -(-sim_steps // 1024) * len({j["D"] for j in large}) + (
                 len(sparse) if bf16 else len(jobs))
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
                 "steps": args.steps, "warmup": args.warmup,

@@ -6,8 +6,7 @@
 // dimension's runs over its CTAs in near-equal numbers of 8-run chunks, so no SM
 // idles while another finishes a whole extra item.  The SMs are shared between the
 // dimensions in proportion to their estimated cost.  Contexts on the large-N path
-// run their per-step GEMM launches on forked streams, captured once into a CUDA graph
-// per chunk of steps and replayed.  Contexts in FP32/FP64 run the SIMT kernels on
+// run in one persistent launch of their own on the remaining SMs, whatever their D.  Contexts in FP32/FP64 run the SIMT kernels on
 // forked streams.
 #include <math.h>
 
@@ -251,37 +250,43 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     CHYM_CUDA_TRY(cudaEventRecord(b->joins[si], s));
     used[si++] = true;
   }
-  // ---- large-N tensor-core contexts: grouped per-step launches, graph replay ----
+  // ---- large-N tensor-core contexts: one persistent launch over all of them ----
   {
     std::vector<unsigned char> descs;
     std::vector<int> dims, idx;
     const size_t kb = k2_desc_bytes();
     const int sidx = si < n ? si++ : 0;
     cudaStream_t s = b->streams[sidx];
+    // the persistent large-N grid takes the SMs the small-N CTAs leave free
+    int small_ctas = 0;
+    for (const auto& L : dl) small_ctas += L.P;
+    const int ctas = std::max(1, b->sms - small_ctas);
+    std::vector<K2Shape> k2_shapes;
     for (int i = 0; i < n; ++i) {
-      chym_ctx* c = b->ctxs[i];
+      const chym_ctx* c = b->ctxs[i];
       if (desc_of[i] >= 0 || !is_tc_prec(params[i].prec) || uses_csr(c, params[i].prec)) continue;
-      if (idx.empty()) CHYM_CUDA_TRY(cudaStreamWaitEvent(s, b->fork, 0));
-      c->prec = params[i].prec;
+      idx.push_back(i);
+      k2_shapes.push_back(k2_shape(c, params[i].prec == CHYM_PREC_FP8, c->n_runs, b->shapes.rt[c->D]));
+    }
+    const std::vector<int> rt = k2_pick_rt(k2_shapes, ctas);
+    for (size_t t = 0; t < idx.size(); ++t) {
+      chym_ctx* c = b->ctxs[idx[t]];
+      if (t == 0) CHYM_CUDA_TRY(cudaStreamWaitEvent(s, b->fork, 0));
+      c->prec = params[idx[t]].prec;
       descs.resize(descs.size() + kb);
-      const StepConsts sc = make_step_consts(c, &params[i], &schedules[i], c->k, steps);
-      cudaError_t e = k2_prepare(c, sc, s, descs.data() + descs.size() - kb, b->shapes.rt[c->D]);
+      const StepConsts sc = make_step_consts(c, &params[idx[t]], &schedules[idx[t]], c->k, steps);
+      cudaError_t e = k2_prepare(c, sc, s, descs.data() + descs.size() - kb, rt[t]);
       if (e != cudaSuccess) return cuda_fail(e, "large-N preparation");
       dims.push_back(c->D);
-      idx.push_back(i);
     }
     if (!idx.empty()) {
-      // the persistent large-N grid takes the SMs the small-N CTAs leave free
-      int small_ctas = 0;
-      for (const auto& L : dl) small_ctas += L.P;
-      const int cap = small_ctas > 0 ? std::max(1, b->sms - small_ctas) : 0;
-      b->part_ctas[0] = cap > 0 ? cap : b->sms;
+      b->part_ctas[0] = ctas;
       b->part_units[0] = 0.0;
       for (int i : idx)
         b->part_units[0] += (double)k2_work_units(b->ctxs[i]->N, b->ctxs[i]->D, b->ctxs[i]->n_runs,
                                                   b->shapes.rt[b->ctxs[i]->D]);
       if (b->timing) CHYM_CUDA_TRY(cudaEventRecord(b->t_begin[0], s));
-      cudaError_t e = k2_integrate(b->k2, descs, dims, steps, b->d_status, s, cap, b->shapes.stages);
+      cudaError_t e = k2_integrate(b->k2, descs, dims, steps, b->d_status, s, ctas, b->shapes.stages);
       if (b->timing && e == cudaSuccess) {
         CHYM_CUDA_TRY(cudaEventRecord(b->t_end[0], s));
         b->timed[0] = true;

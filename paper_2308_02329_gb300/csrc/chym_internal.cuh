@@ -151,20 +151,14 @@ struct TraceRange {
 }  // namespace chym
 
 namespace chym {
-// Launch state of the large-N path: device tables, a private capture stream and the
-// CUDA graph of a chunk of steps (re-captured when the tile table changes shape).
+// Device block of the large-N path (counters, descriptors, tile lists) and the streams of
+// the launches beside the first, kept between calls.
 struct K2Runner {
   void* d_buf = nullptr;
   size_t bytes = 0;
-  cudaStream_t stream = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  size_t sig_tiles = 0;
-  std::vector<int> sig_dims;
-  void* sig_buf = nullptr;
-  int sig_cap = 0;
-  bool sig_stall = false;
-  std::vector<int> sig_stages;
-  int sms = 0;
+  cudaEvent_t fork = nullptr;
+  cudaStream_t streams[8] = {};
+  cudaEvent_t joins[8] = {};
 };
 }  // namespace chym
 
@@ -248,7 +242,17 @@ cudaError_t launch_step_simt(chym_ctx* c, const StepConsts& sc, int32_t prec, cu
 cudaError_t launch_step_tc(chym_ctx* c, const StepConsts& sc, cudaStream_t st);
 cudaError_t launch_step_k2(chym_ctx* c, const StepConsts& sc, cudaStream_t st);
 // large-N path over several contexts (chym_k2.cu)
-cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void* desc_out, int rt = 0);
+// rt: runs per column tile (k2_pick_rt)
+cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void* desc_out, int rt);
+// What decides the runs per column tile of a context; want: a chosen value (0: none)
+struct K2Shape {
+  int N, D, n_runs, a_terms, lo8, want;
+};
+inline K2Shape k2_shape(const chym_ctx* c, int fp8, int n_runs, int want) {
+  const bool pm1 = c->kind == CHYM_J_PM1;
+  return K2Shape{c->N, c->D, n_runs, pm1 ? 1 : 2, fp8 && pm1 ? 1 : 0, want};
+}
+std::vector<int> k2_pick_rt(const std::vector<K2Shape>& shapes, int ctas);
 // most ring stages of the large-N kernel for a context of dimension D with rt runs per
 // column tile (0: the default), real J (terms 2) or FP8 lo, within its shared memory
 int k2_max_stages(int D, int rt, int n_runs, int a_terms, int lo8);
@@ -256,11 +260,9 @@ size_t k2_desc_bytes();
 // tiles x K chunks of one step of a large-N context (the planner's work unit)
 long long k2_work_units(int N, int D, int n_runs, int rt = 0);
 cudaError_t k2_finish(chym_ctx* c, const void* desc, cudaStream_t st);
-// max_ctas > 0 caps the persistent grid (the SMs left to the large-N path when the
-// small-N kernels of a batch occupy the others).
-cudaError_t k2_integrate(K2Runner& R, const std::vector<unsigned char>& descs,
-                         const std::vector<int>& dims, int64_t steps, unsigned* status,
-                         cudaStream_t st, int max_ctas = 0, const int* stages = nullptr);
+// ctas: the SMs of the persistent grid (those the small-N kernels of a batch leave free)
+cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const std::vector<int>& dims,
+                         int64_t steps, unsigned* status, cudaStream_t st, int ctas, const int* stages);
 void k2_runner_release(K2Runner& R);
 // small-N tensor-core kernel over an item plan (chym_tc.cu)
 cudaError_t prepare_tc_operand(chym_ctx* c);

@@ -26,30 +26,45 @@
 // that x_lo S sits in the normal range of e4m3 (|x_lo| <= 2^-9 |x|); the hi and lo
 // products add into one FP32 accumulator holding S y, and the epilogue folds 1/S
 // into dt eps.  x_lo then keeps 4 significant bits: x = hi + lo within 2^-13 |x|.
-// One launch covers a table of tiles (context, M tile mt, column tile ct) that may
-// span many contexts of the same D, ordered with mt fastest so that the CTAs that
-// run at the same time share their column tile's B blocks in L2.  The grid is
-// persistent, one CTA per SM; CTA b takes tiles b, b + grid, ...:
-//   warp 0  producer: TMA bulk copies of the A / B_hi / B_lo blocks of each K
-//           chunk into a ring of up to 8 stages (mbarrier expect_tx);
+// One launch advances every context of a call (any mix of D) by all its steps.  Work is a
+// table of tiles (context, M tile mt, column tile ct), given to the CTAs once per call in
+// lists of near-equal cost (longest tile first, mt fastest so that the CTAs that run at the
+// same time share their column tile's B blocks in L2); a CTA, one per SM, walks its list
+// once per step, and its three roles walk it independently:
+//   warp 0  producer: waits until all MT tiles of the column tile have finished the previous
+//           step (a counter per column tile in global memory), then fills a ring of up to
+//           8 stages with TMA bulk copies of the A / B_hi / B_lo blocks of each K chunk
+//           (mbarrier expect_tx);
 //   warp 1  MMA issuer: tcgen05.mma (M = 128, N = n, K = 16), J_hi X_hi +
 //           J_hi X_lo (+ J_lo X_hi), FP32 accumulators in TMEM, two of them so
 //           that the next tile's products run while the epilogue drains the last;
-//   warps 2-9  epilogue: thread = spin (TMEM lane) x half of the tile's runs; it
+//   warps 2-17 epilogue: thread = spin (TMEM lane) x a quarter of the tile's runs; it
 //           loads its runs' x (global) before the accumulator is ready, then reads
 //           Y (tcgen05.ld), applies drift, loss, annealing and Philox noise (text
 //           after Eq. 1 and after Fig. 2), writes x back and the new BF16 hi/lo
 //           straight into the other buffer (the next step's B blocks).  Per-run
-//           quantities (key, local step, annealing scale) are staged per warp in
-//           shared memory once per tile.
-// The step index comes from a device counter plus a per-launch offset, so a chunk
-// of steps is captured once as a CUDA graph and replayed.  All waits are bounded;
-// on a timeout the CTA raises the status word, drains its own tensor-core and
-// copy work with bounded waits, frees TMEM and returns.
+//           quantities (round keys, the rounds of Philox that depend on the run and step
+//           only, annealing scale) are staged per warp in shared memory;
+//   warp 18 publisher: once the tile's stores (generic proxy) are issued, fences towards the
+//           async proxy of the other SMs' TMA and adds 1 to the column tile's counter.
+// A column tile depends on its own tiles of the previous step only, so there is no barrier
+// over a step: tiles of other column tiles and contexts fill the time of its hand-over.
+// (One launch per step and D, graph-replayed, measured: 32 uneven instances 187 us a step,
+// N = 250 with 1024 runs 18.5 us; every step paid the launch, the ring's fill, the last
+// tile's epilogue, and one D after the other left most SMs idle.)
+// The CTAs wait for one another, so only CTAs known to be resident take part: each counts
+// itself in; once all have, or 100 us after the first, the first one freezes the count P,
+// CTAs that start later exit, and the P present ones share the lists of the absent ones.
+// All waits are bounded; on a timeout the CTA raises the status word, drains its own
+// tensor-core and copy work with bounded waits, frees TMEM and returns.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <functional>
+#include <queue>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "chym_internal.cuh"
@@ -64,11 +79,22 @@ constexpr uint32_t kCoreMN = (kKc / 8) * 128;  // M/N-direction core stride (512
 constexpr int kMaxStages = 8;
 constexpr int kWQ = 2;                         // epilogue warps per TMEM lane quarter
 constexpr int kEpiWarps = 4 * kWQ;
-constexpr int kRB = 4;                         // runs of one epilogue block
-constexpr int kThreads = 64 + 32 * kEpiWarps;  // producer + MMA + epilogue
+constexpr int kUnit = 8;                       // runs of an epilogue unit: a 16-byte core-matrix row of BF16
+constexpr int kPiece = 4;                      // runs finished at a time
+// Warps 0-3 are the producer, the MMA issuer, the publisher and the scout, the others the
+// epilogue.  The helpers' warpgroup hands registers to the epilogue's, which spilled at the
+// launch's even share of 168 (16 bytes at D = 4 cost 10 % of a step, 60 at D = 8 13 %: the ring
+// leaves the spills little L1).
+constexpr int kPubWarp = 2, kScoutWarp = 3, kEpiWarp0 = 4;
+constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
+constexpr int kLaunchRegs = 168, kHelperRegs = 64, kEpiRegs = 216;
+static_assert(128 * kHelperRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * kLaunchRegs &&
+                  kThreads * kLaunchRegs <= 65536, "register split");
 constexpr int kAccCols = 256;                  // TMEM columns of one accumulator
-constexpr size_t kRingBudget = 196 * 1024;     // shared memory for the stage ring
-constexpr int kGraphSteps = 16;                // steps per captured graph
+constexpr size_t kRingBudget = 192 * 1024;     // shared memory for the stage ring
+constexpr int kLaunchSteps = 1024;             // most steps of one launch
+constexpr int kPhaseTiles = 2;                 // tiles per CTA of a phase (at least)
+constexpr int kPhaseSteps = 32;                // fewest steps of a call that is split into phases
 constexpr uint32_t kA8Block = 128 * kKc;       // bytes of an e4m3 A block (4 KB)
 constexpr int kLoScaleLog2 = 16;               // FP8 mode: B operands carry 2^16
 
@@ -80,13 +106,15 @@ __host__ __device__ constexpr int k2_rt_max(int D) {
 
 // One large-N context of a launch.
 struct K2Desc {
+  int D;
+  int flag0;               // its first column-tile counter
   const uint8_t* Aimg;
   float* Xm;
   uint8_t* Xt;             // both buffers; buffer b at Xt + b * buf_bytes
   const float* ar;         // per run: 1 + dt (h - 1)
   const uint64_t* seeds;   // per run: Philox key
   const int64_t* koff;     // per run: global step of its (re)seeding
-  unsigned long long buf_bytes;
+  unsigned long long buf_bytes;  // even: a 256-byte multiple
   int N, KP, MT, KC, CT, RT, n, n_runs, a_terms, sched_kind;
   int lo8;                 // 1: lo half in e4m3 (FP8 mode, +-1 couplings)
   int stall;               // CHYM_FLAG_TEST_STALL: the accumulator-full signal is withheld
@@ -98,27 +126,36 @@ struct K2Tile {
   int desc, mt, ct, pad;
 };
 
-// Per-run quantities of one step, staged in shared memory by each epilogue warp for
-// the runs it finishes: Philox key, local step (noise counter and annealing),
-// 1 + dt (h - 1), and dt eps alpha_mu for the extra components mu >= 1.
-struct RunC {
-  uint32_t key0, key1;
-  uint32_t kl_lo, kl_hi;
-  float ar, erp;
+// Per-run quantities of one step, staged in shared memory by each epilogue warp for the
+// next slots() runs it finishes.  r12[blk] carries the first two Philox rounds as far as
+// they depend on the run and the step only (see philox_run), rk the keys of rounds 3..10.
+template <int D>
+struct __align__(16) RunC {
+  static constexpr int kSlots = 32;
+  uint4 r12[(D + 3) / 4];
+  uint4 rk[4];
+  float ar, erp;  // 1 + dt (h - 1), and dt eps alpha_mu of the extra components mu >= 1
 };
-constexpr int kRunSlots = 256 / kWQ;  // most runs per epilogue warp and tile (RT / kWQ)
+constexpr int kTileCache = 24;  // tiles of a CTA's list whose descriptors are kept in shared memory
 
 struct K2Launch {
   const K2Desc* descs;
   const K2Tile* tiles;
-  const int64_t* done;    // steps already taken in this call (device counter)
   int n_tiles;
-  int k_off;              // this launch's offset within the captured chunk
+  const int* cta_begin;   // list of CTA b: tiles [cta_begin[b], cta_begin[b + 1])
+  const int* phase_end;   // [CTA][phase]: ends of the phases in its list
+  int phases;
+  unsigned* sync;         // [0] CTAs present (kFrozen: count closed), [1] their number once closed
+  unsigned* flags;        // per column tile: M tiles finished, over all steps of the launch
+  int64_t step0;          // steps taken in this call before this launch
+  int steps;
   int stages;             // depth of the ring
   uint32_t stage_stride;  // bytes per stage
   unsigned* status;
   unsigned long long wait_ns;  // limit of every bounded wait
 };
+constexpr unsigned kFrozen = 0x80000000u;
+constexpr unsigned long long kJoinNs = 100000;
 
 __host__ __device__ inline uint32_t b_block_bytes(int n) { return (uint32_t)n * kKc * 2u; }
 // bytes of a lo block: BF16, or e4m3 in FP8 mode
@@ -161,31 +198,31 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
   return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
-// D (+)= A B on the tensor core, kind::f16 (BF16 operands, FP32 accumulator), with
-// both shared-memory descriptors given by their low words (their high words are
-// equal).
-__device__ __forceinline__ void mma_bf16_w(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                           uint32_t idesc, uint32_t accumulate) {
+// D (+)= A B on the tensor core, kind::f16 (BF16 operands, FP32 accumulator), issued by one
+// elected lane of a converged warp.  The whole warp runs the issue loop: its descriptors
+// stay in uniform registers (44 cycles a product of N = 48, 128 of N = 256, the tensor
+// core's own rates), while a lone thread's loop moves them there for every product (65 to
+// 150 cycles).
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}\n" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate));
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
-// D += A B on the tensor core, kind::f8f6f4 (e4m3 operands, K = 32, FP32 accumulator),
-// with the descriptors' low words and their own high words.
-__device__ __forceinline__ void mma_f8_w(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                         uint32_t b_hi, uint32_t idesc) {
+// D += A B, kind::f8f6f4 (e4m3 operands, K = 32, FP32 accumulator), issued likewise.
+__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc) {
   asm volatile(
-      "{\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %5, 1;\n\t}\n" ::"r"(d_tmem),
-      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc));
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, 1;\n\t}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc));
 }
+// Arrival on an mbarrier once the products issued so far are complete; the lane elected for
+// them (the same one for every elect.sync of a full warp).
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar)
+      : "memory");
 }
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile(
@@ -209,20 +246,9 @@ __device__ __forceinline__ void sincos_ftz(float x, float& s, float& c) {
   asm("sin.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(x));
   asm("cos.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(x));
 }
-// Box-Muller on one pair of words (see box_muller_f32 in chym_internal.cuh); the
-// noise scale sigma sqrt(dt) is folded into neg2ln2s2 = -2 ln2 (sigma^2 dt).
-__device__ __forceinline__ void box_muller(uint32_t wr, uint32_t wa, float neg2ln2s2, float& z0,
-                                           float& z1) {
-  const float ur = __fmaf_rn((float)wr, 2.3283064365386963e-10f, 1.1641532182693481e-10f);
-  const float th = __fmaf_rn((float)wa, 1.4629180792671596e-09f, -3.1415926528582302f);
-  const float r = -sqrt_ftz(neg2ln2s2 * lg2_ftz(ur));
-  float s, c;
-  sincos_ftz(th, s, c);
-  z0 = r * c;
-  z1 = r * s;
-}
-// The same transform for the word pairs of two runs at once, in paired FP32 arithmetic
-// (identical roundings): z0 = (z0 of run A, of run B), likewise z1.
+// Box-Muller on the word pairs of two runs at once (see box_muller_f32 in
+// chym_internal.cuh), in paired FP32 arithmetic: z0 = (z0 of run A, of run B), likewise z1;
+// the noise scale sigma sqrt(dt) is folded into neg2ln2s2 = -2 ln2 (sigma^2 dt).
 __device__ __forceinline__ void box_muller2(uint32_t wrA, uint32_t waA, uint32_t wrB, uint32_t waB,
                                             float neg2ln2s2, float2& z0, float2& z1) {
   const float2 ur = __ffma2_rn(make_float2((float)wrA, (float)wrB),
@@ -239,109 +265,448 @@ __device__ __forceinline__ void box_muller2(uint32_t wrA, uint32_t waA, uint32_t
   z0 = __fmul2_rn(r, make_float2(cA, cB));
   z1 = __fmul2_rn(r, make_float2(sA, sB));
 }
-// Philox4x32-10 (the generator of chym_internal.cuh) with each round's two
-// products as 32 x 32 -> 64-bit multiplies.
-__device__ __forceinline__ uint4 philox_wide(uint4 c, uint32_t k0, uint32_t k1) {
+// Philox4x32-10 of the block of spin (group) p of a run at its local step.  Counter (p, blk,
+// k_lo, k_hi) and key (k0, k1): round 1 multiplies p (a constant of the thread: mp = M0 p)
+// and k_lo, and round 2 the result of k_lo's product, which depends on the run and step
+// only.  RunC::r12 holds what is left of both rounds (k' = the round-2 key):
+//   x = k_hi ^ k1, y = lo(M1 k_lo) ^ k0', z = hi(M0 c) ^ k1', w = lo(M0 c) with
+//   c = hi(M1 k_lo) ^ blk ^ k0.
+__device__ __forceinline__ uint4 run_rounds12(uint32_t blk, uint32_t k_lo, uint32_t k_hi, uint32_t k0, uint32_t k1) {
+  const uint64_t p1 = (uint64_t)kPhiloxM1 * k_lo;
+  const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ blk ^ k0);
+  return make_uint4(k_hi ^ k1, (uint32_t)p1 ^ (k0 + kPhiloxW0), (uint32_t)(p0 >> 32) ^ (k1 + kPhiloxW1), (uint32_t)p0);
+}
+template <int D>
+__device__ __forceinline__ uint4 philox_run(uint64_t mp, const RunC<D>& rc, int blk) {
+  const uint4 t = rc.r12[blk];
+  const uint64_t q = (uint64_t)kPhiloxM1 * ((uint32_t)(mp >> 32) ^ t.x);
+  uint4 c = make_uint4((uint32_t)(q >> 32) ^ t.y, (uint32_t)q, t.z ^ (uint32_t)mp, t.w);
 #pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * c.x, p1 = (uint64_t)kPhiloxM1 * c.z;
-    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1,
-                   (uint32_t)p0);
-    k0 += kPhiloxW0;
-    k1 += kPhiloxW1;
+  for (int i = 0; i < 4; ++i) {
+    const uint4 kk = rc.rk[i];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint64_t p0 = (uint64_t)kPhiloxM0 * c.x, p1 = (uint64_t)kPhiloxM1 * c.z;
+      c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ (h ? kk.z : kk.x), (uint32_t)p1,
+                     (uint32_t)(p0 >> 32) ^ c.w ^ (h ? kk.w : kk.y), (uint32_t)p0);
+    }
   }
   return c;
 }
-
-// Four accumulator columns of two components (one component) for the warp's 32
-// lanes, with the wait in the same asm statement (tcgen05.ld fills its registers
-// asynchronously until tcgen05.wait::ld, so the compiler must not see them earlier).
-__device__ __forceinline__ void tmem_ld4x2(uint32_t a, uint32_t b, float (&ya)[kRB], float (&yb)[kRB]) {
-  uint32_t r[8];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-      : "r"(a), "r"(b)
-      : "memory");
-#pragma unroll
-  for (int j = 0; j < kRB; ++j) {
-    ya[j] = __uint_as_float(r[j]);
-    yb[j] = __uint_as_float(r[4 + j]);
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// Bounded wait until *p >= want (p: a counter other SMs add to).
+__device__ __forceinline__ bool counter_wait(const unsigned* p, unsigned want, unsigned long long limit_ns) {
+  uint64_t t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (ld_acquire(p) >= want) return true;
+    if ((it & 15u) == 0u) {
+      const uint64_t t = global_timer();
+      if (it == 0) t0 = t;
+      else if (t - t0 > limit_ns) return false;
+    }
   }
 }
-__device__ __forceinline__ void tmem_ld4(uint32_t a, float (&y)[kRB]) {
-  uint32_t r[4];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-      : "r"(a)
-      : "memory");
+__device__ __forceinline__ uint32_t ld_acquire_cta(uint32_t p) {
+  uint32_t v;
+  asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release_cta(uint32_t p, uint32_t v) {
+  asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// The accumulator columns of a piece's runs for M components, ld columns apart, for the warp's
+// 32 lanes, with the wait in the same asm statement (tcgen05.ld fills its registers
+// asynchronously until tcgen05.wait::ld, so the compiler must not see them earlier).  One
+// round trip for all of them: a load per run pair and component made the D = 8 step 13 %
+// slower.
+template <int M>
+__device__ __forceinline__ void tmem_ld_piece(uint32_t a, uint32_t ld, float (&y)[4][kPiece]) {
+  static_assert(kPiece == 4, "x4 loads");
+  uint32_t r[16] = {};
+  if constexpr (M == 4)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%17];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%18];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%19];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(a), "r"(a + ld), "r"(a + 2 * ld), "r"(a + 3 * ld)
+        : "memory");
+  else if constexpr (M == 3)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%12];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%13];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%14];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11])
+        : "r"(a), "r"(a + ld), "r"(a + 2 * ld)
+        : "memory");
+  else if constexpr (M == 2)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(a), "r"(a + ld)
+        : "memory");
+  else
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+        : "r"(a)
+        : "memory");
 #pragma unroll
-  for (int j = 0; j < kRB; ++j) y[j] = __uint_as_float(r[j]);
+  for (int m = 0; m < M; ++m)
+#pragma unroll
+    for (int j = 0; j < kPiece; ++j) y[m][j] = __uint_as_float(r[4 * m + j]);
 }
 
-// x of the runs [run0, run0 + kRB) and all components at spin p (zeros outside).
+// Streaming access to the master state.  Volatile: a thread reads back what it stored
+// itself one step earlier, and volatile asm statements keep their order.
+__device__ __forceinline__ float ld_stream(const float* p) {
+  float v;
+  asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void st_stream(float* p, float v) {
+  asm volatile("st.global.cs.f32 [%0], %1;" ::"l"(p), "f"(v));
+}
+
+// x of a piece's consecutive runs (the first `left` of them exist) and all components at the
+// thread's spin; x points at the first run's component 0.
 template <int D>
-__device__ __forceinline__ void load_block_x(const float* __restrict__ Xm, int KP, int n_runs, int run0,
-                                             int p, bool live, float (&x)[D][kRB]) {
-  const float* base = Xm + (size_t)run0 * D * KP + p;
+__device__ __forceinline__ void load_piece(const float* x, int KP, int left, bool live, float (&v)[D][kPiece]) {
 #pragma unroll
-  for (int j = 0; j < kRB; ++j) {
-    const bool ok = live && run0 + j < n_runs;
+  for (int j = 0; j < kPiece; ++j) {
+    const bool ok = live && j < left;
 #pragma unroll
-    for (int mu = 0; mu < D; ++mu) x[mu][j] = ok ? __ldcs(base + (j * D + mu) * KP) : 0.f;  // 32-bit offsets
+    for (int mu = 0; mu < D; ++mu) v[mu][j] = ok ? ld_stream(x + (j * D + mu) * KP) : 0.f;  // 32-bit offsets
   }
 }
 
-// BF16 hi/lo split of 4 new values of one component, stored as one half row of a
-// core matrix (8 bytes) in each of the next step's hi and lo B blocks.
-__device__ __forceinline__ void store_hilo(uint8_t* hi_dst, uint8_t* lo_dst, const float (&v)[kRB]) {
-  uint32_t hw[2], lw[2];
+// Split of a piece's n values of one component, packed: BF16 hi words, BF16 lo words.
+template <int n>
+__device__ __forceinline__ void split_piece(const float (&v)[n], uint32_t (&hi)[n / 2], uint32_t (&lo)[n / 2]) {
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
+  for (int j = 0; j < n / 2; ++j) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
     const float2 hf = __bfloat1622float2(h);
     const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * j] - hf.x, v[2 * j + 1] - hf.y);
-    hw[j] = *reinterpret_cast<const uint32_t*>(&h);
-    lw[j] = *reinterpret_cast<const uint32_t*>(&l);
+    hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+    lo[j] = *reinterpret_cast<const uint32_t*>(&l);
   }
-  *reinterpret_cast<uint2*>(hi_dst) = make_uint2(hw[0], hw[1]);
-  *reinterpret_cast<uint2*>(lo_dst) = make_uint2(lw[0], lw[1]);
 }
 
-// FP8 mode: 4 new values of one component as S bf16(v) (8 bytes, hi block) and
-// e4m3(S (v - bf16(v))) (4 bytes, lo block), S = 2^kLoScaleLog2.
-__device__ __forceinline__ void store_hilo8(uint8_t* hi_dst, uint8_t* lo_dst, const float (&v)[kRB]) {
+// FP8 mode: S bf16(v) and, in lo[0], the n bytes e4m3(S (v - bf16(v))), S = 2^kLoScaleLog2.
+template <int n>
+__device__ __forceinline__ void split_piece8(const float (&v)[n], uint32_t (&hi)[n / 2], uint32_t (&lo)[n / 2]) {
   constexpr float S = (float)(1u << kLoScaleLog2);
-  uint32_t hw[2], lw[2];
+  uint32_t l = 0;
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
+  for (int j = 0; j < n / 2; ++j) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
     const float2 hf = __bfloat1622float2(h);
     const __nv_bfloat162 hs = __floats2bfloat162_rn(hf.x * S, hf.y * S);  // exact
-    hw[j] = *reinterpret_cast<const uint32_t*>(&hs);
-    lw[j] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2((v[2 * j] - hf.x) * S, (v[2 * j + 1] - hf.y) * S),
-                                               __NV_SATFINITE, __NV_E4M3);
+    hi[j] = *reinterpret_cast<const uint32_t*>(&hs);
+    l |= (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2((v[2 * j] - hf.x) * S, (v[2 * j + 1] - hf.y) * S),
+                                            __NV_SATFINITE, __NV_E4M3)
+         << (16 * j);
   }
-  *reinterpret_cast<uint2*>(hi_dst) = make_uint2(hw[0], hw[1]);
-  *reinterpret_cast<uint32_t*>(lo_dst) = lw[0] | (lw[1] << 16);
+  lo[0] = l;
+}
+
+// Constants of one tile for the epilogue, in registers.
+struct EpiTile {
+  float* Xm;
+  int KP, n_runs, RT, run0;  // run0: the tile's first run
+  int p;
+  bool live;
+  float gdt, kdt, edt, nl2;
+  uint32_t acc;              // accumulator of the warp's lanes
+  uint64_t mp;               // M0 times the Philox counter of the spin
+};
+
+// A piece of one unit: x (in: state before the step, out: after it, zero for absent runs)
+// at the thread's spin, from the accumulator columns col.. of each component; writes x back.
+template <int D>
+__device__ __forceinline__ void advance_piece(const EpiTile& w, const RunC<D>* rc, int run, uint32_t col,
+                                              float (&x)[D][kPiece]) {
+  // per run: 1 + dt(h-1) - dt gamma |x_p|^2 from the state before the step
+  float tl[kPiece];
+#pragma unroll
+  for (int j = 0; j < kPiece; ++j) {
+    float n2 = 0.f;
+#pragma unroll
+    for (int mu = 0; mu < D; ++mu) n2 = fmaf(x[mu][j], x[mu][j], n2);
+    tl[j] = fmaf(-w.gdt, n2, rc[j].ar);
+  }
+  float* xrow = w.Xm + (size_t)run * D * w.KP + w.p;
+  auto block = [&](auto blk_c) {  // components 4 blk .. 4 blk + M - 1, one Philox block
+    constexpr int blk = decltype(blk_c)::value, M = D - 4 * blk < 4 ? D - 4 * blk : 4;
+    float y[4][kPiece];
+    tmem_ld_piece<M>(w.acc + (uint32_t)(4 * blk * w.RT) + col, (uint32_t)w.RT, y);
+#pragma unroll
+    for (int j = 0; j < kPiece; j += 2) {  // two runs at once, paired FP32 arithmetic
+      float2 z[4];
+      const RunC<D> &cA = rc[j], &cB = rc[j + 1];
+      const bool okA = w.live && run + j < w.n_runs, okB = w.live && run + j + 1 < w.n_runs;
+      const uint4 wA = philox_run<D>(w.mp, cA, blk), wB = philox_run<D>(w.mp, cB, blk);
+      if constexpr (D <= 2) {
+        // the 4/D spins with the same p / (4/D) share one block; spin p takes its
+        // normals (p % (4/D)) D .. + D - 1, one Box-Muller pair
+        constexpr uint32_t per = 4u / D;
+        const uint32_t j0 = ((uint32_t)w.p % per) * D;
+        const bool hi2 = j0 >= 2u;
+        float2 cz, sz;
+        box_muller2(hi2 ? wA.z : wA.x, hi2 ? wA.w : wA.y, hi2 ? wB.z : wB.x, hi2 ? wB.w : wB.y, w.nl2, cz, sz);
+        z[0] = (j0 & 1u) ? sz : cz;
+        z[1] = sz;
+      } else {
+        box_muller2(wA.x, wA.y, wB.x, wB.y, w.nl2, z[0], z[1]);
+        if constexpr (M > 2) box_muller2(wA.z, wA.w, wB.z, wB.w, w.nl2, z[2], z[3]);
+      }
+      const float2 t2 = make_float2(tl[j], tl[j + 1]), nk2 = make_float2(-w.kdt, -w.kdt);
+      const float2 e0 = make_float2(w.edt, w.edt), e1 = make_float2(cA.erp, cB.erp);
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const int mu = 4 * blk + m;
+        const float2 xv = make_float2(x[mu][j], x[mu][j + 1]);
+        const float2 sf = __ffma2_rn(__fmul2_rn(nk2, xv), xv, t2);
+        const float2 inner = __ffma2_rn(mu == 0 ? e0 : e1, make_float2(y[m][j], y[m][j + 1]), z[m]);
+        const float2 v = __ffma2_rn(xv, sf, inner);
+        x[mu][j] = okA ? v.x : 0.f;
+        x[mu][j + 1] = okB ? v.y : 0.f;
+        if (okA) st_stream(xrow + (j * D + mu) * w.KP, v.x);
+        if (okB) st_stream(xrow + ((j + 1) * D + mu) * w.KP, v.y);
+      }
+    }
+  };
+  block(std::integral_constant<int, 0>());
+  if constexpr (D > 4) block(std::integral_constant<int, 1>());
+}
+
+// A CTA's list of tiles: entry i is table entry base + i stride.  The list falls into phases,
+// each advanced by all steps before the next begins.
+struct TileWalk {
+  int base, stride, count, phases;
+  const int* phase_end;  // ends of the phases in the list (one phase: count)
+  const K2Launch* L;
+  const K2Desc* cache;   // descriptors of the first kTileCache tiles
+  __device__ __forceinline__ int index(int i) const { return base + i * stride; }
+  __device__ __forceinline__ K2Tile tile(int i) const { return L->tiles[index(i)]; }
+  __device__ __forceinline__ const K2Desc& desc(int i, const K2Tile& t) const {
+    return i < kTileCache ? cache[i] : L->descs[t.desc];
+  }
+  __device__ __forceinline__ int end_of(int ph) const { return phases > 1 ? phase_end[ph] : count; }
+};
+
+// A place in that walk, in the order in which all roles go: phase, step of the launch, tile.
+struct WalkPos {
+  int i, s, i0, i1, ph;
+  __device__ __forceinline__ explicit WalkPos(const TileWalk& W) : i(0), s(0), i0(0), i1(W.end_of(0)), ph(0) {
+    skip_empty(W);
+  }
+  __device__ __forceinline__ bool done(const TileWalk& W) const { return ph >= W.phases; }
+  __device__ __forceinline__ void next(const TileWalk& W) {
+    if (++i < i1) return;
+    i = i0;
+    if (++s < W.L->steps) return;
+    s = 0;
+    enter(W, i1);
+    skip_empty(W);
+  }
+
+ private:
+  __device__ __forceinline__ void enter(const TileWalk& W, int from) {
+    i = i0 = from;
+    if (++ph < W.phases) i1 = W.end_of(ph);
+  }
+  __device__ __forceinline__ void skip_empty(const TileWalk& W) {
+    while (ph < W.phases && i0 == i1) enter(W, i1);
+  }
+};
+
+// The epilogue warps' loop over the CTA's tiles (see step_k2_kernel); e: share of the warp
+// among the kWQ of its lane quarter.
+template <int D, typename Done>
+__device__ __forceinline__ bool epilogue(const TileWalk& W, const K2Launch& L, RunC<D>* rc, const uint64_t* acc_full,
+                                         volatile int* abort, uint32_t lane_base, int e, Done done) {
+  constexpr int kSlots = RunC<D>::kSlots;
+  // The loads of x run one piece ahead, into the next tile's first piece at the end of a tile
+  // (with its first run constants).  The split of a unit's first piece waits for the second,
+  // so that both go out as one 16-byte row: 8-byte stores to half rows cost 9 % of a step at
+  // N = 1000, D = 4.
+  const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) & 3;
+  float xn[D][kPiece];
+  uint64_t key_n = 0;
+  int64_t koff_n = 0;
+  float ar_n = 0.f;
+  bool ahead = false;  // xn and key_n.. hold the coming tile's first pieces and runs
+  // the units of the warp in tile i of the list: e' + kWQ ui, ui < nu; the shares go round
+  // with the tile, so that uneven ones (RT = 24: 3 units) even out over a list
+  auto first_unit = [&](int i) { return (e + W.index(i)) % kWQ; };
+  auto n_units = [&](const K2Desc& d, int e0) { return max(0, (d.RT / kUnit - e0 + kWQ - 1) / kWQ); };
+  // global loads of the run constants of slot `lane` from unit ui on
+  auto fetch_run = [&](const K2Desc& d, int ct, int e0, int nu, int ui) {
+    const int u = ui + lane / kUnit;
+    if (lane < kSlots && u < nu) {
+      const int r = min(ct * d.RT + kUnit * (e0 + kWQ * u) + lane % kUnit, d.n_runs - 1);
+      key_n = __ldg(d.seeds + r);
+      koff_n = __ldg(d.koff + r);
+      ar_n = __ldg(d.ar + r);
+    }
+  };
+  uint32_t it = 0;
+  for (WalkPos at(W); !at.done(W); ++it) {
+    const int i = at.i;
+    const int64_t step = L.step0 + at.s;
+    at.next(W);  // the tile after this one
+    const K2Tile tile = W.tile(i);
+    const K2Desc& d = W.desc(i, tile);
+    const int e0 = first_unit(i), nu = n_units(d, e0);
+    EpiTile w;
+    w.Xm = d.Xm;
+    w.KP = d.KP;
+    w.n_runs = d.n_runs;
+    w.RT = d.RT;
+    w.run0 = tile.ct * d.RT;
+    w.p = tile.mt * 128 + q * 32 + lane;
+    w.live = w.p < d.N;
+    w.gdt = d.gdt;
+    w.kdt = d.kdt;
+    w.edt = d.edt;
+    w.nl2 = d.neg2ln2s2;
+    w.acc = lane_base + (it & 1u) * (uint32_t)kAccCols;
+    w.mp = (uint64_t)kPhiloxM0 * (D <= 2 ? (uint32_t)w.p / (4u / (D <= 2 ? D : 4)) : (uint32_t)w.p);
+    const uint32_t BB = b_block_bytes(d.n), BL = b_lo_bytes(d.n, d.lo8);
+    const bool lo8 = d.lo8 != 0;
+    // this thread's spin (row k = p of the next step's B) in its hi and lo blocks
+    uint8_t* hi_row = d.Xt + (size_t)((step + 1) & 1) * d.buf_bytes;
+    uint8_t* lo_row = hi_row + (size_t)d.CT * d.KC * BB;
+    const size_t blk = (size_t)tile.ct * d.KC + (w.p / kKc);
+    const size_t row_in = (size_t)((w.p % kKc) >> 3) * kCoreK + (size_t)(w.p & 7) * 16u;
+    hi_row += blk * BB + row_in;
+    lo_row += blk * BL + row_in;
+    const int64_t k = d.k0 + step;
+    // run constants of the warp's units ui .. into its slots, from key_n, koff_n and ar_n
+    auto stage = [&](int ui) {
+      __syncwarp();
+      if (lane < kSlots && ui + lane / kUnit < nu) {
+        const int64_t kl = k - koff_n;
+        float ramp = 1.f;
+        if (d.sched_kind == 1 && kl >= d.k_anneal)
+          ramp = kl >= d.k_total ? 0.f : fmaxf(0.f, 1.f - (float)(kl - d.k_anneal) * d.inv_ramp);
+        const uint32_t k0 = (uint32_t)key_n, k1 = (uint32_t)(key_n >> 32);
+        RunC<D>& o = rc[lane];
+#pragma unroll
+        for (int b = 0; b < (D + 3) / 4; ++b)
+          o.r12[b] = run_rounds12((uint32_t)b, (uint32_t)kl, (uint32_t)((uint64_t)kl >> 32), k0, k1);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {  // Weyl key schedule: round j (0-based) uses key + j (W0, W1)
+          const uint32_t j = 2u * r + 2u;
+          o.rk[r] = make_uint4(k0 + j * kPhiloxW0, k1 + j * kPhiloxW1, k0 + (j + 1u) * kPhiloxW0,
+                               k1 + (j + 1u) * kPhiloxW1);
+        }
+        o.ar = ar_n;
+        o.erp = w.edt * ramp;
+      }
+      __syncwarp();
+    };
+    auto x_of = [&](int run) { return w.Xm + (size_t)run * D * w.KP + w.p; };
+    if (nu > 0) {
+      const int run = w.run0 + kUnit * e0;
+      if (!ahead) load_piece<D>(x_of(run), w.KP, w.n_runs - run, w.live, xn);
+      if (!ahead) fetch_run(d, tile.ct, e0, nu, 0);
+      stage(0);
+    }
+    ahead = false;
+    const uint32_t bar = smem_addr(acc_full + (it & 1u));
+    if (!__all_sync(0xffffffffu, mbar_wait(bar, (it >> 1) & 1u, L.wait_ns) && !*abort)) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+    for (int ui = 0; ui < nu; ++ui) {
+      if (ui > 0 && ui % (kSlots / kUnit) == 0) {
+        fetch_run(d, tile.ct, e0, nu, ui);
+        stage(ui);
+      }
+      const int u = e0 + kWQ * ui;
+      uint32_t hs[D][kPiece / 2], ls[D][kPiece / 2];  // the split that waits
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int run = w.run0 + kUnit * u + kPiece * h;
+        float x[D][kPiece];
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu)
+#pragma unroll
+          for (int j = 0; j < kPiece; ++j) x[mu][j] = xn[mu][j];
+        if (h == 0 || ui + 1 < nu) {
+          const int nx = h == 0 ? run + kPiece : w.run0 + kUnit * (u + kWQ);
+          load_piece<D>(x_of(nx), w.KP, w.n_runs - nx, w.live, xn);
+        } else if (!at.done(W)) {  // the next tile's first piece and run constants
+          const int i2 = at.i;
+          const K2Tile t2 = W.tile(i2);
+          const K2Desc& d2 = W.desc(i2, t2);
+          const int f2 = first_unit(i2), nu2 = n_units(d2, f2);
+          if (nu2 > 0) {
+            const int nx = t2.ct * d2.RT + kUnit * f2, p2 = t2.mt * 128 + q * 32 + lane;
+            load_piece<D>(d2.Xm + (size_t)nx * D * d2.KP + p2, d2.KP, d2.n_runs - nx, p2 < d2.N, xn);
+            fetch_run(d2, t2.ct, f2, nu2, 0);
+            ahead = true;
+          }
+        }
+        advance_piece<D>(w, rc + kUnit * (ui % (kSlots / kUnit)) + kPiece * h, run,
+                         (uint32_t)(kUnit * u + kPiece * h), x);
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu) {
+          uint32_t hv[kPiece / 2], lv[kPiece / 2];
+          if (lo8) split_piece8<kPiece>(x[mu], hv, lv);
+          else split_piece<kPiece>(x[mu], hv, lv);
+          const int col = mu * w.RT + kUnit * u;
+          uint8_t* hd = hi_row + (size_t)(col >> 3) * kCoreMN;  // a row of the unit's 8 columns
+          uint8_t* ld = lo8 ? lo_row + (size_t)(col >> 4) * kCoreMN + (size_t)(col & 15)
+                            : lo_row + (size_t)(col >> 3) * kCoreMN;
+          if (h == 0) {
+#pragma unroll
+            for (int j = 0; j < kPiece / 2; ++j) {
+              hs[mu][j] = hv[j];
+              ls[mu][j] = lv[j];
+            }
+          } else {
+            *reinterpret_cast<uint4*>(hd) = make_uint4(hs[mu][0], hs[mu][1], hv[0], hv[1]);
+            if (lo8) *reinterpret_cast<uint2*>(ld) = make_uint2(ls[mu][0], lv[0]);
+            else *reinterpret_cast<uint4*>(ld) = make_uint4(ls[mu][0], ls[mu][1], lv[0], lv[1]);
+          }
+        }
+      }
+    }
+    done(it);
+  }
+  return true;
 }
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
-  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], drain_bar;
-  __shared__ uint32_t s_tmem;
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], drain_bar, stored;
+  __shared__ uint32_t s_tmem, s_cleared;
+  __shared__ int s_rank, s_P;
   __shared__ volatile int s_abort;
-  __shared__ RunC s_runc[kEpiWarps][kRunSlots];
+  __shared__ RunC<D> s_runc[kEpiWarps][RunC<D>::kSlots];
+  __shared__ K2Desc s_desc[kTileCache];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int S = L.stages;
-  const int64_t step = *L.done + L.k_off;  // steps taken in this call before this one
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -350,6 +715,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
   }
   if (tid == 32) {
     s_abort = 0;
+    s_cleared = 0;
     for (int s = 0; s < S; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&full_bar[s])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&empty_bar[s])));
@@ -360,285 +726,233 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
                    "r"(kEpiWarps));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&drain_bar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&stored)), "r"(kEpiWarps));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (tid == 64) {  // count this CTA in; the first one closes the count
+    const unsigned old = atomicAdd(L.sync, 1u);
+    int P = 0;
+    if (!(old & kFrozen)) {
+      if (old == 0) {
+        counter_wait(L.sync, gridDim.x, kJoinNs);
+        P = (int)(atomicOr(L.sync, kFrozen) & ~kFrozen);
+        __threadfence();
+        atomicExch(L.sync + 1, (unsigned)P);
+      } else if (counter_wait(L.sync + 1, 1u, L.wait_ns)) {
+        P = (int)ld_acquire(L.sync + 1);
+      } else {
+        atomicOr(L.status, STATUS_TIMEOUT);
+      }
+    }
+    s_rank = (int)old;
+    s_P = P;  // 0: too late (or timed out), nothing to do
+  }
+  __syncthreads();
+  const int P = s_P, rank = s_rank;
+  // all present: this CTA's own list; else the table is dealt out round the present ones
+  TileWalk W{0, 1, 0, 1, nullptr, &L, s_desc};
+  if (P == (int)gridDim.x) {
+    W.base = L.cta_begin[rank];
+    W.count = L.cta_begin[rank + 1] - W.base;
+    W.phases = L.phases;
+    W.phase_end = L.phase_end + (size_t)rank * L.phases;
+  } else if (P > 0) {
+    W.base = rank;
+    W.stride = P;
+    W.count = (L.n_tiles - rank + P - 1) / P;
+  }
+  {  // descriptors of the first tiles, word by word
+    constexpr int kWords = sizeof(K2Desc) / 4;
+    static_assert(sizeof(K2Desc) % 4 == 0, "copied by words");
+    for (int i = tid; i < min(W.count, kTileCache) * kWords; i += kThreads)
+      reinterpret_cast<uint32_t*>(s_desc)[i] =
+          reinterpret_cast<const uint32_t*>(L.descs + L.tiles[W.index(i / kWords)].desc)[i % kWords];
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
+  auto give_up = [&]() {
+    atomicOr(L.status, STATUS_TIMEOUT);
+    s_abort = 1;
+  };
 
-  if (warp == 0) {
-    // ---------------- producer ----------------
-    if (lane == 0) {
-      uint32_t g = 0;  // stage uses issued
-      for (int t = blockIdx.x; t < L.n_tiles && !s_abort; t += gridDim.x) {
-        const K2Tile tile = L.tiles[t];
-        const K2Desc& d = L.descs[tile.desc];
-        // the tile's constants in registers (the loop's asm statements clobber memory)
-        const int KC = d.KC, terms = d.a_terms, lo8 = d.lo8;
-        const uint32_t BB = b_block_bytes(d.n), BL = b_lo_bytes(d.n, lo8);
-        const uint32_t bytes = stage_bytes(d.n, terms, lo8);
-        const uint32_t a2 = terms > 1 ? kABlock : lo8 ? kA8Block : 0u;  // second A term
-        const uint8_t* a_src = d.Aimg + (size_t)tile.mt * KC * kABlock;       // term 0, K chunk 0
-        const size_t a_term = (size_t)d.MT * KC * kABlock;                    // to the second term
-        const uint8_t* a2_src = d.Aimg + a_term + (size_t)tile.mt * KC * a2;
-        const uint8_t* bx = d.Xt + (size_t)(step & 1) * d.buf_bytes;
-        const uint8_t* b_src = bx + (size_t)tile.ct * KC * BB;
-        const uint8_t* bl_src = bx + (size_t)d.CT * KC * BB + (size_t)tile.ct * KC * BL;
-        bool stop = false;
-        for (int kc = 0; kc < KC; ++kc, ++g, a_src += kABlock, a2_src += a2, b_src += BB, bl_src += BL) {
-          const uint32_t s = g % (uint32_t)S;
-          if (g >= (uint32_t)S && !mbar_wait(smem_addr(&empty_bar[s]), ((g / S) - 1u) & 1u, L.wait_ns)) {
-            atomicOr(L.status, STATUS_TIMEOUT);
-            s_abort = 1;
-            stop = true;
-            break;
+  if (W.count == 0) {
+    // too late: the CTAs present do this one's tiles
+  } else if (warp < kEpiWarp0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs));
+    if (warp == 0) {
+      // ---------------- producer ----------------
+      if (lane == 0) {
+        uint32_t s = 0, ph = 1, g = 0, it = 0;  // stage, parity of its empty barrier, uses, tiles
+        bool ok = true;
+        for (WalkPos at(W); ok && !at.done(W); at.next(W), ++it) {
+          const int i = at.i, st = at.s;
+          const K2Tile tile = W.tile(i);
+          const K2Desc& d = W.desc(i, tile);
+          // the tile's constants in registers (the loop's asm statements clobber memory)
+          const int KC = d.KC, terms = d.a_terms, lo8 = d.lo8;
+          const uint32_t BB = b_block_bytes(d.n), BL = b_lo_bytes(d.n, lo8);
+          const uint32_t bytes = stage_bytes(d.n, terms, lo8);
+          const uint32_t a2 = terms > 1 ? kABlock : lo8 ? kA8Block : 0u;  // second A term
+          const uint8_t* a_src = d.Aimg + (size_t)tile.mt * KC * kABlock;       // term 0, K chunk 0
+          const size_t a_term = (size_t)d.MT * KC * kABlock;                    // to the second term
+          const uint8_t* a2_src = d.Aimg + a_term + (size_t)tile.mt * KC * a2;
+          const uint8_t* bx = d.Xt + (size_t)((L.step0 + st) & 1) * d.buf_bytes;
+          const uint8_t* b_src = bx + (size_t)tile.ct * KC * BB;
+          const uint8_t* bl_src = bx + (size_t)d.CT * KC * BB + (size_t)tile.ct * KC * BL;
+          // the scout has cleared this tile
+          uint64_t t0 = 0;
+          for (uint32_t n = 0; (int32_t)(ld_acquire_cta(smem_addr(&s_cleared)) - it) <= 0; ++n) {
+            const uint64_t t = global_timer();
+            if (n == 0) t0 = t;
+            if (s_abort || t - t0 > L.wait_ns) {
+              ok = false;
+              break;
+            }
           }
-          const uint32_t base = smem_addr(smem) + s * L.stage_stride;
-          const uint32_t fb = smem_addr(&full_bar[s]);
-          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes)
-                       : "memory");
-          bulk_g2s(base, a_src, kABlock, fb);
-          if (a2) bulk_g2s(base + kABlock, a2_src, a2, fb);
-          const uint32_t bb = base + kABlock + a2;
-          bulk_g2s(bb, b_src, BB, fb);
-          bulk_g2s(bb + BB, bl_src, BL, fb);
+          for (int kc = 0; kc < KC && ok; ++kc, ++g, a_src += kABlock, a2_src += a2, b_src += BB, bl_src += BL) {
+            if (g >= (uint32_t)S && !mbar_wait(smem_addr(&empty_bar[s]), ph, L.wait_ns)) {
+              ok = false;
+              break;
+            }
+            const uint32_t base = smem_addr(smem) + s * L.stage_stride;
+            const uint32_t fb = smem_addr(&full_bar[s]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes)
+                         : "memory");
+            bulk_g2s(base, a_src, kABlock, fb);
+            if (a2) bulk_g2s(base + kABlock, a2_src, a2, fb);
+            const uint32_t bb = base + kABlock + a2;
+            bulk_g2s(bb, b_src, BB, fb);
+            bulk_g2s(bb + BB, bl_src, BL, fb);
+            if (++s == (uint32_t)S) {
+              s = 0;
+              ph ^= 1u;
+            }
+          }
+          if (s_abort) break;
         }
-        if (stop) break;
+        if (!ok) give_up();
+        // drain: every copy issued must have landed before the CTA may exit
+        const uint32_t first = g > (uint32_t)S ? g - (uint32_t)S : 0u;
+        for (uint32_t u = first; u < g; ++u)
+          if (!mbar_wait(smem_addr(&full_bar[u % S]), (u / S) & 1u, L.wait_ns)) atomicOr(L.status, STATUS_TIMEOUT);
       }
-      // drain: every copy issued must have landed before the CTA may exit
-      const uint32_t first = g > (uint32_t)S ? g - (uint32_t)S : 0u;
-      for (uint32_t u = first; u < g; ++u)
-        if (!mbar_wait(smem_addr(&full_bar[u % S]), (u / S) & 1u, L.wait_ns)) atomicOr(L.status, STATUS_TIMEOUT);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      uint32_t g = 0, it = 0;
+    } else if (warp == 1) {
+      // ---------------- MMA issuer (the whole warp, see mma_bf16) ----------------
+      uint32_t s = 0, ph = 0, it = 0;  // ring stage and its phase, tiles
       bool ok = true;
-      for (int t = blockIdx.x; t < L.n_tiles && ok; t += gridDim.x, ++it) {
-        const K2Tile tile = L.tiles[t];
-        const K2Desc& d = L.descs[tile.desc];
-        const uint32_t BB = b_block_bytes(d.n);
+      for (WalkPos at(W); ok && !at.done(W); at.next(W), ++it) {
+        const int i = at.i;
+        const K2Tile tile = W.tile(i);
+        const K2Desc& d = W.desc(i, tile);
+        const uint32_t n = (uint32_t)d.n, BB = b_block_bytes(d.n);
         const uint32_t b = it & 1u, use = it >> 1;
+        // kind::f16, FP32 accumulator, BF16 A (K-major) and B (MN-major), N = n, M = 128
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((n >> 3) << 17) |
+                               ((uint32_t)(128 >> 4) << 24);
+        // FP8 mode: e4m3 J (K-major, 8 x 16-byte cores, 256 bytes between row groups) and
+        // e4m3 lo (MN-major, 16 columns a core row, 512 bytes between column groups)
+        const uint32_t idesc8 = (1u << 4) | (1u << 16) | ((n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        const uint32_t acc = tmem + b * (uint32_t)kAccCols;
+        const bool real_j = d.a_terms > 1, lo8 = d.lo8 != 0;
+        const bool stall = d.stall != 0;
+        const uint32_t a2 = real_j ? kABlock : lo8 ? kA8Block : 0u;
+        // a stage and a K step move only the start-address field (shared addresses stay below
+        // 256 KB, so the field never carries)
+        const uint64_t d0 = smem_desc(smem_addr(smem), kCoreK, kCoreMN), d80 = smem_desc(smem_addr(smem), kCoreK, 256u);
+        const uint64_t o_bhi = (kABlock + a2) >> 4, o_blo = o_bhi + (BB >> 4), o_alo = kABlock >> 4;
+        constexpr uint64_t kStep = 2u * kCoreK >> 4;
+        const int KC = d.KC;
         if (use > 0 && !mbar_wait(smem_addr(&acc_empty[b]), (use - 1u) & 1u, L.wait_ns)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // kind::f16, FP32 accumulator, BF16 A (K-major) and B (MN-major), N = n, M = 128
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) |
-                               ((uint32_t)(d.n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-        const uint32_t acc = tmem + b * (uint32_t)kAccCols;
-        // Descriptors as two 32-bit words: the low word (start address >> 4, LBO)
-        // is the only part that moves between stages and K steps, so each product
-        // costs one add; the high word (SBO, version) is the same for all of them.
-        const uint32_t d_hi = (uint32_t)(smem_desc(0u, kCoreK, kCoreMN) >> 32);
-        const uint32_t d_lo0 = (uint32_t)smem_desc(smem_addr(smem), kCoreK, kCoreMN);
-        const bool real_j = d.a_terms > 1, lo8 = d.lo8 != 0;
-        const uint32_t a2 = real_j ? kABlock : lo8 ? kA8Block : 0u;
-        const uint32_t o_bhi = (kABlock + a2) >> 4, o_blo = o_bhi + (BB >> 4);
-        const uint32_t o_alo = kABlock >> 4, stride16 = L.stage_stride >> 4;
-        // FP8 mode: e4m3 J (K-major, 8 x 16-byte cores, 256 bytes between row groups) and
-        // e4m3 lo (MN-major, 16 columns a core row, 512 bytes between column groups)
-        const uint32_t a8_hi = (uint32_t)(smem_desc(0u, kCoreK, 256u) >> 32);
-        const uint32_t idesc8 = (1u << 4) | (1u << 16) | ((uint32_t)(d.n >> 3) << 17) |
-                                ((uint32_t)(128 >> 4) << 24);
-        const int KC = d.KC;
-        for (int kc = 0; kc < KC; ++kc, ++g) {
-          const uint32_t s = g % (uint32_t)S;
-          if (!mbar_wait(smem_addr(&full_bar[s]), (g / S) & 1u, L.wait_ns) || s_abort) {
+        for (int kc = 0; kc < KC; ++kc) {
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_addr(&full_bar[s]), ph, L.wait_ns) && !s_abort)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t a0 = d_lo0 + s * stride16;
+          const uint64_t off = (uint64_t)(s * (L.stage_stride >> 4));
+          const uint64_t a = d0 + off;
+          const uint32_t acc0 = kc > 0 ? 1u : 0u;
+          static_assert(kKc == 32, "two BF16 K steps per chunk");
+          mma_bf16(acc, a, a + o_bhi, idesc, acc0);
           if (lo8) {
-#pragma unroll
-            for (int ks = 0; ks < kKc / 16; ++ks) {
-              const uint32_t a = a0 + (uint32_t)ks * (2u * kCoreK >> 4);
-              mma_bf16_w(acc, a, a + o_bhi, d_hi, idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-            }
-            mma_f8_w(acc, a0 + o_alo, a8_hi, a0 + o_blo, d_hi, idesc8);
+            mma_bf16(acc, a + kStep, a + o_bhi + kStep, idesc, 1u);
+            mma_f8(acc, d80 + off + o_alo, a + o_blo, idesc8);
           } else {
-#pragma unroll
-            for (int ks = 0; ks < kKc / 16; ++ks) {
-              const uint32_t a = a0 + (uint32_t)ks * (2u * kCoreK >> 4);
-              mma_bf16_w(acc, a, a + o_bhi, d_hi, idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-              mma_bf16_w(acc, a, a + o_blo, d_hi, idesc, 1u);
-              if (real_j) mma_bf16_w(acc, a + o_alo, a + o_bhi, d_hi, idesc, 1u);
-            }
+            mma_bf16(acc, a, a + o_blo, idesc, 1u);
+            if (real_j) mma_bf16(acc, a + o_alo, a + o_bhi, idesc, 1u);
+            mma_bf16(acc, a + kStep, a + o_bhi + kStep, idesc, 1u);
+            mma_bf16(acc, a + kStep, a + o_blo + kStep, idesc, 1u);
+            if (real_j) mma_bf16(acc, a + o_alo + kStep, a + o_bhi + kStep, idesc, 1u);
           }
           mma_commit(smem_addr(&empty_bar[s]));
+          if (++s == (uint32_t)S) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        if (!ok) break;
         // (test of the timeout path: the signal is withheld, so the epilogue's wait runs
         // out; the drain below still waits for every product issued)
-        if (!d.stall) mma_commit(smem_addr(&acc_full[b]));
+        if (ok && !stall) mma_commit(smem_addr(&acc_full[b]));
       }
-      if (!ok) {
-        atomicOr(L.status, STATUS_TIMEOUT);
-        s_abort = 1;
-      }
+      if (!ok && lane == 0) give_up();
       // every product issued must be complete before TMEM is freed
       mma_commit(smem_addr(&drain_bar));
-      if (!mbar_wait(smem_addr(&drain_bar), 0u, L.wait_ns)) atomicOr(L.status, STATUS_TIMEOUT);
+      if (!mbar_wait(smem_addr(&drain_bar), 0u, L.wait_ns) && lane == 0) atomicOr(L.status, STATUS_TIMEOUT);
+    } else if (warp == kPubWarp) {
+      // ---------------- publisher ----------------
+      if (lane == 0) {
+        uint32_t it = 0;
+        bool ok = true;
+        for (WalkPos at(W); ok && !at.done(W); at.next(W), ++it) {
+          const int i = at.i;
+          const K2Tile tile = W.tile(i);
+          unsigned* done = L.flags + W.desc(i, tile).flag0 + tile.ct;
+          ok = mbar_wait(smem_addr(&stored), it & 1u, L.wait_ns) && !s_abort;
+          if (!ok) break;
+          fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
+          __threadfence();
+          asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
+        }
+        if (!ok) give_up();
+      }
+    } else {
+      // ---------------- scout ----------------
+      if (lane == 0) {
+        uint32_t it = 0;
+        bool ok = true;
+        for (WalkPos at(W); ok && !at.done(W); at.next(W)) {
+          const int i = at.i, st = at.s;
+          const K2Tile tile = W.tile(i);
+          const K2Desc& d = W.desc(i, tile);
+          // every M tile of the column tile has finished the steps before this one
+          ok = counter_wait(L.flags + d.flag0 + tile.ct, (unsigned)d.MT * (unsigned)st, L.wait_ns) && !s_abort;
+          if (!ok) break;
+          fence_proxy_async();  // their stores before this CTA's TMA reads
+          st_release_cta(smem_addr(&s_cleared), ++it);
+        }
+        if (!ok) give_up();
+      }
     }
   } else {
     // ---------------- epilogue: 4 kWQ warps ----------------
-    const int q = warp & 3;             // TMEM lane quarter of this warp
-    const int e = (warp - 2) >> 2;      // its 4-run blocks: rb = e, e + kWQ, e + 2 kWQ, ...
-    const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
-    RunC* rc = s_runc[warp - 2];
-    uint32_t it = 0;
-    for (int t = blockIdx.x; t < L.n_tiles; t += gridDim.x, ++it) {
-      const K2Tile tile = L.tiles[t];
-      const K2Desc& dref = L.descs[tile.desc];
-      // the context's constants, read once per tile into registers
-      float* __restrict__ Xm = dref.Xm;
-      const int KP = dref.KP, n_runs = dref.n_runs, RT = dref.RT, nb = RT / (kRB * kWQ);
-      const float gdt = dref.gdt, kdt = dref.kdt, edt = dref.edt, nl2 = dref.neg2ln2s2;
-      const int p = tile.mt * 128 + q * 32 + lane;
-      const bool live = p < dref.N;
-      const uint32_t BB = b_block_bytes(dref.n);
-      const bool lo8 = dref.lo8 != 0;
-      const uint32_t BL = b_lo_bytes(dref.n, dref.lo8);
-      uint8_t* Xt_next = dref.Xt + (size_t)((step + 1) & 1) * dref.buf_bytes;
-      uint8_t* Xl_next = Xt_next + (size_t)dref.CT * dref.KC * BB;
-      // byte offset of this thread's spin (row k = p of the next step's B) in its hi and
-      // lo blocks
-      const size_t row_in = (size_t)((p % kKc) >> 3) * kCoreK + (size_t)(p & 7) * 16u;
-      const size_t row_off = ((size_t)tile.ct * dref.KC + (p / kKc)) * BB + row_in;
-      const size_t row_lo = ((size_t)tile.ct * dref.KC + (p / kKc)) * BL + row_in;
-      const int run_tile = tile.ct * RT;
-      float xc[D][kRB];
-      load_block_x<D>(Xm, KP, n_runs, run_tile + kRB * e, p, live, xc);  // in flight during the products
-      {
-        // stage the per-run quantities of this warp's runs (slot = kRB jb + j)
-        const int64_t k = dref.k0 + step;
-        const int sk = dref.sched_kind;
-        const int64_t ka = dref.k_anneal, kt = dref.k_total;
-        const float inv_ramp = dref.inv_ramp;
-        __syncwarp();
-        for (int sl = lane; sl < kRB * nb; sl += 32) {
-          const int r = min(run_tile + kRB * (e + kWQ * (sl / kRB)) + (sl % kRB), n_runs - 1);
-          const int64_t kl = k - __ldg(dref.koff + r);
-          float ramp = 1.f;
-          if (sk == 1 && kl >= ka) ramp = kl >= kt ? 0.f : fmaxf(0.f, 1.f - (float)(kl - ka) * inv_ramp);
-          const uint64_t key = __ldg(dref.seeds + r);
-          rc[sl] = RunC{(uint32_t)key, (uint32_t)(key >> 32), (uint32_t)kl, (uint32_t)((uint64_t)kl >> 32),
-                        __ldg(dref.ar + r), edt * ramp};
-        }
-        __syncwarp();
-      }
-      const uint32_t b = it & 1u;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&acc_full[b]), (it >> 1) & 1u, L.wait_ns)) &&
-                      !s_abort;
-      if (!ok) {
-        if (lane == 0) {
-          atomicOr(L.status, STATUS_TIMEOUT);
-          s_abort = 1;
-        }
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t acc = lane_base + b * (uint32_t)kAccCols;
-#pragma unroll 1
-      for (int jb = 0; jb < nb; ++jb) {
-        const int rb = e + kWQ * jb;
-        const int run0 = run_tile + kRB * rb;
-        const bool more = jb + 1 < nb;
-        float xnext[D][kRB];
-        if (more) load_block_x<D>(Xm, KP, n_runs, run0 + kRB * kWQ, p, live, xnext);
-        const RunC* rcb = rc + kRB * jb;
-        // per run: 1 + dt(h-1) - dt gamma |x_p|^2 from the state before the step
-        float tl[kRB];
-#pragma unroll
-        for (int j = 0; j < kRB; ++j) {
-          float n2 = 0.f;
-#pragma unroll
-          for (int mu = 0; mu < D; ++mu) n2 = fmaf(xc[mu][j], xc[mu][j], n2);
-          tl[j] = fmaf(-gdt, n2, rcb[j].ar);
-        }
-        float* xrow = Xm + (size_t)run0 * D * KP + p;
-#pragma unroll
-        for (int blk = 0; blk < (D + 3) / 4; ++blk) {
-          constexpr int kZ = 4;
-          const int M = D - 4 * blk < kZ ? D - 4 * blk : kZ;  // components of this block
-          float y[4][kRB];
-          const uint32_t c0 = acc + (uint32_t)(4 * blk * RT + kRB * rb);
-          // only the M components of this block: columns stay inside the accumulator
-          if (M >= 2) tmem_ld4x2(c0, c0 + (uint32_t)RT, y[0], y[1]);
-          else tmem_ld4(c0, y[0]);
-          if (M == 4) tmem_ld4x2(c0 + 2u * (uint32_t)RT, c0 + 3u * (uint32_t)RT, y[2], y[3]);
-          else if (M == 3) tmem_ld4(c0 + 2u * (uint32_t)RT, y[2]);
-#pragma unroll
-          for (int j = 0; j < kRB; j += 2) {  // two runs at once, paired FP32 arithmetic
-            const RunC cA = rcb[j], cB = rcb[j + 1];
-            const bool okA = live && run0 + j < n_runs, okB = live && run0 + j + 1 < n_runs;
-            float2 z[4];
-            if constexpr (D <= 2) {
-              // the 4/D spins with the same p / (4/D) share one block; spin p takes its
-              // normals (p % (4/D)) D .. + D - 1, one Box-Muller pair
-              constexpr uint32_t per = 4u / D;
-              const uint4 wA = philox_wide(make_uint4((uint32_t)p / per, 0u, cA.kl_lo, cA.kl_hi), cA.key0, cA.key1);
-              const uint4 wB = philox_wide(make_uint4((uint32_t)p / per, 0u, cB.kl_lo, cB.kl_hi), cB.key0, cB.key1);
-              const uint32_t j0 = ((uint32_t)p % per) * D;
-              const bool hi2 = j0 >= 2u;
-              float2 cz, sz;
-              box_muller2(hi2 ? wA.z : wA.x, hi2 ? wA.w : wA.y, hi2 ? wB.z : wB.x, hi2 ? wB.w : wB.y, nl2, cz, sz);
-              z[0] = (j0 & 1u) ? sz : cz;
-              z[1] = sz;
-            } else {
-              const uint4 wA = philox_wide(make_uint4((uint32_t)p, (uint32_t)blk, cA.kl_lo, cA.kl_hi), cA.key0, cA.key1);
-              const uint4 wB = philox_wide(make_uint4((uint32_t)p, (uint32_t)blk, cB.kl_lo, cB.kl_hi), cB.key0, cB.key1);
-              box_muller2(wA.x, wA.y, wB.x, wB.y, nl2, z[0], z[1]);
-              if (M > 2) box_muller2(wA.z, wA.w, wB.z, wB.w, nl2, z[2], z[3]);
-            }
-            const float2 t2 = make_float2(tl[j], tl[j + 1]), nk2 = make_float2(-kdt, -kdt);
-            const float2 e0 = make_float2(edt, edt), e1 = make_float2(cA.erp, cB.erp);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              if (m < M) {
-                const int mu = 4 * blk + m;
-                const float2 xv = make_float2(xc[mu][j], xc[mu][j + 1]);
-                const float2 sf = __ffma2_rn(__fmul2_rn(nk2, xv), xv, t2);
-                const float2 inner = __ffma2_rn(mu == 0 ? e0 : e1, make_float2(y[m][j], y[m][j + 1]), z[m]);
-                const float2 v = __ffma2_rn(xv, sf, inner);
-                xc[mu][j] = okA ? v.x : 0.f;
-                xc[mu][j + 1] = okB ? v.y : 0.f;
-                if (okA) __stcs(xrow + (j * D + mu) * KP, v.x);
-                if (okB) __stcs(xrow + ((j + 1) * D + mu) * KP, v.y);
-              }
-            }
-          }
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            if (m < M) {
-              const int mu = 4 * blk + m;
-              const int col = mu * RT + kRB * rb;
-              const size_t off = row_off + (size_t)(col >> 3) * kCoreMN + (size_t)(col & 7) * 2u;
-              if (lo8)
-                store_hilo8(Xt_next + off, Xl_next + row_lo + (size_t)(col >> 4) * kCoreMN + (size_t)(col & 15),
-                            xc[mu]);
-              else
-                store_hilo(Xt_next + off, Xl_next + off, xc[mu]);  // BF16 lo blocks mirror hi
-            }
-          }
-        }
-        if (more) {
-#pragma unroll
-          for (int mu = 0; mu < D; ++mu)
-#pragma unroll
-            for (int j = 0; j < kRB; ++j) xc[mu][j] = xnext[mu][j];
-        }
-      }
-      // this accumulator may be overwritten now
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
+    const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const bool ok = epilogue<D>(W, L, s_runc[warp - kEpiWarp0], acc_full, &s_abort, lane_base, (warp - kEpiWarp0) >> 2, [&](uint32_t it) {
+      // this accumulator may be overwritten now, and the tile's stores published
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0)
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[b])) : "memory");
-    }
+      if (lane == 0) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&stored)) : "memory");
+      }
+    });
+    if (!ok && lane == 0) give_up();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -647,8 +961,6 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kAccCols));
   }
 }
-
-__global__ void k2_advance_kernel(int64_t* done, int64_t by) { *done += by; }
 
 // X[run][p][mu] (float) -> Xm[c][p] and the hi/lo blocks of buffer 0 (the
 // buffer is zeroed beforehand, so padding spins and runs stay zero).
@@ -729,29 +1041,6 @@ __global__ void k2_aimg_kernel(const double* __restrict__ J, int N, int MT, int 
   }
 }
 
-template <int D>
-cudaError_t k2_launch_typed(const K2Launch& L, int grid, size_t smem, cudaStream_t st) {
-  auto kern = step_k2_kernel<D>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, kThreads, smem, st>>>(L);
-  return cudaGetLastError();
-}
-
-cudaError_t k2_launch(int D, const K2Launch& L, int grid, size_t smem, cudaStream_t st) {
-  switch (D) {
-    case 1: return k2_launch_typed<1>(L, grid, smem, st);
-    case 2: return k2_launch_typed<2>(L, grid, smem, st);
-    case 3: return k2_launch_typed<3>(L, grid, smem, st);
-    case 4: return k2_launch_typed<4>(L, grid, smem, st);
-    case 5: return k2_launch_typed<5>(L, grid, smem, st);
-    case 6: return k2_launch_typed<6>(L, grid, smem, st);
-    case 7: return k2_launch_typed<7>(L, grid, smem, st);
-    case 8: return k2_launch_typed<8>(L, grid, smem, st);
-  }
-  return cudaErrorInvalidValue;
-}
-
 // Runs per column tile of a context: the most for its D (or the autotuner's choice
 // `want`), shrunk (in multiples of 32) for contexts with fewer runs so that small
 // instances waste no columns.
@@ -761,7 +1050,55 @@ int k2_rt(int D, int n_runs, int want = 0) {
   return std::min(top, std::max(32, r32));
 }
 
+// Time of a tile in the planner's units (ns): the ring's feed against the epilogue, which
+// overlap.  95 bytes a ns of feed and 42 ns per run and component (two passes of the eight
+// warps over 128 spins) were measured with one side of the tile loop emptied (N = 800,
+// D = 4, FP8 mode); the constant is the hand-over between them.
+double k2_tile_ns(int N, int D, int RT, int a_terms, int lo8) {
+  const int KC = (N + 127) / 128 * 128 / kKc;
+  const double feed = KC * (double)stage_bytes(D * RT, a_terms, lo8) / 95.0, epi = 42.0 * D * RT;
+  return std::max(feed, epi) + 0.3 * std::min(feed, epi) + 1000.0;
+}
+
 }  // namespace
+
+// Runs per column tile of every context of a call on `ctas` CTAs.  While the tiles do not
+// fill the CTAs, the costliest tile's context takes column tiles of half the runs: with
+// fewer tiles than SMs a step lasts as long as its costliest tile (N = 250, D = 3, 1024
+// runs: 32 tiles of 64 runs, 128 of 16).  Below 16 runs a tile's J blocks outweigh its
+// columns.  A context whose tile width was chosen (want) keeps it.
+std::vector<int> k2_pick_rt(const std::vector<K2Shape>& shapes, int ctas) {
+  std::vector<int> rt;
+  long long tiles = 0;
+  auto count = [&](const K2Shape& s, int r) {
+    return (long long)((s.N + 127) / 128) * ((s.n_runs + r - 1) / r);
+  };
+  for (const K2Shape& s : shapes) {
+    rt.push_back(k2_rt(s.D, s.n_runs, s.want));
+    tiles += count(s, rt.back());
+  }
+  for (;;) {
+    int best = -1;
+    double cost = 0.0;
+    for (size_t i = 0; i < shapes.size(); ++i) {
+      const K2Shape& s = shapes[i];
+      // whole 4-run blocks for the two warps of a lane quarter, n = D RT a multiple of 16
+      const int half = rt[i] / 2;
+      if (s.want > 0 || half < 16 || rt[i] % 16 || s.D * half % 16) continue;
+      const double c = k2_tile_ns(s.N, s.D, rt[i], s.a_terms, s.lo8);
+      if (c > cost) {
+        cost = c;
+        best = (int)i;
+      }
+    }
+    if (best < 0) return rt;
+    const int half = rt[best] / 2;
+    const long long more = count(shapes[best], half) - count(shapes[best], rt[best]);
+    if (tiles + more > ctas) return rt;
+    rt[best] = half;
+    tiles += more;
+  }
+}
 
 int k2_max_stages(int D, int rt, int n_runs, int a_terms, int lo8) {
   const int n = D * k2_rt(D, n_runs, rt);
@@ -797,12 +1134,12 @@ cudaError_t prepare_k2_operand(chym_ctx* c) {
 // Runner: a set of large-N contexts integrated together for `steps` steps.
 // ---------------------------------------------------------------------------
 // Workspace, per-run constants and buffer 0 of one context; fills its descriptor.
-cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void* desc_out, int rt) {
+cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void* desc_out, int RT) {
   cudaError_t e = prepare_k2_operand(c);
   if (e != cudaSuccess) return e;
   K2Desc& d = *reinterpret_cast<K2Desc*>(desc_out);
   const int N = c->N, D = c->D, MT = (N + 127) / 128, KP = MT * 128, KC = KP / kKc;
-  const int RT = k2_rt(D, sc.n_runs, rt), n = D * RT;
+  const int n = D * RT;
   const int CT = (sc.n_runs + RT - 1) / RT;
   const int lo8 = sc.fp8 && c->kind == CHYM_J_PM1 ? 1 : 0;
   const size_t BB = b_block_bytes(n), BL = b_lo_bytes(n, lo8);
@@ -828,6 +1165,8 @@ cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void*
   k2_runconst_kernel<<<(sc.n_runs + 255) / 256, 256, 0, st>>>(c->d_h, c->d_hidx, sc.n_runs, sc.dt, ar);
   k2_pack_kernel<<<152 * 8, 256, 0, st>>>((const float*)c->d_X, Xm, Xt, N, D, KP, KC, CT, RT,
                                            sc.n_runs, lo8);
+  d.D = D;
+  d.flag0 = 0;  // set by k2_integrate
   d.Aimg = (const uint8_t*)c->d_Ak2;
   d.Xm = Xm;
   d.Xt = Xt;
@@ -867,157 +1206,228 @@ cudaError_t k2_finish(chym_ctx* c, const void* desc, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+namespace {
+
+cudaError_t k2_launch(int D, const K2Launch& L, int grid, size_t smem, cudaStream_t st) {
+  auto go = [&](auto kern) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, kThreads, smem, st>>>(L);
+    return cudaGetLastError();
+  };
+  switch (D) {
+    case 1: return go(step_k2_kernel<1>);
+    case 2: return go(step_k2_kernel<2>);
+    case 3: return go(step_k2_kernel<3>);
+    case 4: return go(step_k2_kernel<4>);
+    case 5: return go(step_k2_kernel<5>);
+    case 6: return go(step_k2_kernel<6>);
+    case 7: return go(step_k2_kernel<7>);
+    case 8: return go(step_k2_kernel<8>);
+  }
+  return cudaErrorInvalidValue;
+}
+
+// The contexts of one D: their tiles in lists per CTA, and where these sit in the device block.
+struct K2Group {
+  int D = 0, grid = 0, phases = 1;
+  double cost = 0.0;
+  size_t n_tiles = 0, o_sync = 0, n_sync = 0, o_tile = 0, o_cta = 0;
+  std::vector<int> descs;
+  std::vector<std::vector<K2Tile>> lists;
+  std::vector<std::vector<int>> phase_end;  // per CTA
+};
+
+}  // namespace
+
 // Integrate the contexts whose descriptors are in `descs` (host copies, dims[i] =
-// their D) for `steps` steps on stream st: one persistent launch per dimension
-// per step, chunks of kGraphSteps steps captured once into a CUDA graph and
-// replayed.
-cudaError_t k2_integrate(K2Runner& R, const std::vector<unsigned char>& descs,
-                         const std::vector<int>& dims, int64_t steps, unsigned* status,
-                         cudaStream_t st, int max_ctas, const int* stage_choice) {
+// their D) for `steps` steps on stream st: one persistent launch per D and kLaunchSteps
+// steps.  With several D the CTAs are split in proportion to their work and the launches
+// run side by side on the runner's streams.
+cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const std::vector<int>& dims,
+                         int64_t steps, unsigned* status, cudaStream_t st, int ctas, const int* stage_choice) {
   const size_t db = sizeof(K2Desc);
   const int n_desc = (int)dims.size();
   cudaError_t e = cudaSuccess;
-  if (R.sms == 0) {
-    int dev = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&R.sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  auto desc = [&](int i) -> K2Desc& { return *reinterpret_cast<K2Desc*>(descs.data() + i * db); };
   bool stall = false;  // CHYM_FLAG_TEST_STALL on any context: the short wait limit
-  for (int i = 0; i < n_desc; ++i) stall = stall || reinterpret_cast<const K2Desc*>(descs.data() + i * db)->stall;
-  // tile tables per dimension; ring stride per dimension
-  std::vector<K2Tile> tiles;
-  std::vector<int> dim_first(9, 0), dim_count(9, 0);
-  std::vector<uint32_t> dim_stride(9, 0);
+  std::vector<double> tile_ns(n_desc);
+  std::vector<K2Group> groups;
+  double total = 0.0;
   for (int D = 1; D <= 8; ++D) {
-    dim_first[D] = (int)tiles.size();
-    // contexts in decreasing order of tile cost (K x columns x product terms): the
-    // persistent CTAs take tiles round-robin, so the costly tiles go out first and
-    // the cheap ones fill in at the end (mixed sizes otherwise leave long tails)
-    std::vector<int> order;
-    for (int i = 0; i < n_desc; ++i)
-      if (dims[i] == D) order.push_back(i);
-    auto cost = [&](int i) {
-      const K2Desc& d = *reinterpret_cast<const K2Desc*>(descs.data() + i * db);
-      return (long long)d.KP * d.n * (d.a_terms > 1 ? 6 : d.lo8 ? 3 : 4);  // in half BF16 products
-    };
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost(x) > cost(y); });
-    for (int i : order) {
-      const K2Desc& d = *reinterpret_cast<const K2Desc*>(descs.data() + i * db);
-      const uint32_t bytes = stage_bytes(d.n, d.a_terms, d.lo8);
-      dim_stride[D] = std::max(dim_stride[D], (bytes + 1023u) / 1024u * 1024u);
-      for (int ct = 0; ct < d.CT; ++ct)
-        for (int mt = 0; mt < d.MT; ++mt) tiles.push_back(K2Tile{i, mt, ct, 0});  // mt fastest
+    K2Group g;
+    g.D = D;
+    for (int i = 0; i < n_desc; ++i) {
+      if (dims[i] != D) continue;
+      K2Desc& d = desc(i);
+      stall = stall || d.stall;
+      d.flag0 = (int)g.n_sync;  // column-tile counters of the group so far
+      g.n_sync += d.CT;
+      tile_ns[i] = k2_tile_ns(d.N, D, d.RT, d.a_terms, d.lo8);
+      g.n_tiles += (size_t)d.CT * d.MT;
+      g.cost += tile_ns[i] * d.CT * d.MT;
+      g.descs.push_back(i);
     }
-    dim_count[D] = (int)tiles.size() - dim_first[D];
-    // boustrophedon rounds: every other full round of `grid` tiles goes to the CTAs in
-    // reverse, so the CTA that drew the largest tile of one round draws the smallest of
-    // the next
-    const int grid = std::min(dim_count[D], max_ctas > 0 ? std::min(max_ctas, R.sms) : R.sms);
-    for (int r0 = grid; grid > 0 && r0 + grid <= dim_count[D]; r0 += 2 * grid)
-      std::reverse(tiles.begin() + dim_first[D] + r0, tiles.begin() + dim_first[D] + r0 + grid);
+    if (g.descs.empty()) continue;
+    g.n_sync += 4;  // join words
+    total += g.cost;
+    groups.push_back(g);
   }
-  const size_t bytes = 64 + descs.size() + tiles.size() * sizeof(K2Tile);
-  if (bytes > R.bytes) {
-    if (R.exec) cudaGraphExecDestroy(R.exec);
-    R.exec = nullptr;
+  // side by side, each on its share of the CTAs; one after the other where they are too few
+  const bool beside = groups.size() > 1 && ctas >= 2 * (int)groups.size();
+  int left = ctas;
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    K2Group& g = groups[gi];
+    const int others = (int)(groups.size() - gi) - 1;
+    int share = ctas;
+    if (beside) {
+      share = std::min(left - others, std::max(1, (int)(left * g.cost / total + 0.5)));
+      left -= share;
+      total -= g.cost;
+    }
+    g.grid = (int)std::min<size_t>(g.n_tiles, (size_t)share);
+    // the costliest tiles first, each to the CTA with the least work so far (the lowest of
+    // equals: tiles of one cost go round), so the lists end close together
+    std::stable_sort(g.descs.begin(), g.descs.end(), [&](int x, int y) { return tile_ns[x] > tile_ns[y]; });
+    g.lists.resize(g.grid);
+    g.phase_end.resize(g.grid);
+    g.phases = steps >= kPhaseSteps ? std::max(1, (int)(g.n_tiles / ((size_t)g.grid * kPhaseTiles))) : 1;
+    using Load = std::pair<double, int>;
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
+    for (int b = 0; b < g.grid; ++b) heap.push({0.0, b});
+    // phases of whole rounds of the grid, as far as the column tiles allow, so that no phase
+    // but the last leaves CTAs idle
+    const size_t rounds = (g.n_tiles + g.grid - 1) / g.grid;
+    size_t dealt = 0;
+    int ph = 0;
+    auto close_phase = [&]() {
+      for (int b = 0; b < g.grid; ++b) g.phase_end[b].push_back((int)g.lists[b].size());
+      ++ph;
+    };
+    for (int i : g.descs)
+      for (int ct = 0; ct < desc(i).CT; ++ct) {
+        if (ph + 1 < g.phases && dealt + desc(i).MT > rounds * (size_t)(ph + 1) / g.phases * (size_t)g.grid) close_phase();
+        for (int mt = 0; mt < desc(i).MT; ++mt, ++dealt) {  // mt fastest
+          const Load l = heap.top();
+          heap.pop();
+          g.lists[l.second].push_back(K2Tile{i, mt, ct, 0});
+          heap.push({l.first + tile_ns[i], l.second});
+        }
+      }
+    while (ph < g.phases) close_phase();
+  }
+  // device block: [join words | column-tile counters] of every group (zeroed per launch), then
+  // descriptors, tiles and lists
+  auto up16 = [](size_t x) { return (x + 15) / 16 * 16; };
+  size_t at = 0;
+  for (K2Group& g : groups) {
+    g.o_sync = at;
+    at = up16(at + sizeof(unsigned) * g.n_sync);
+  }
+  const size_t o_desc = at;
+  at = up16(at + descs.size());
+  for (K2Group& g : groups) {
+    g.o_tile = at;
+    g.o_cta = at + g.n_tiles * sizeof(K2Tile);
+    at = up16(g.o_cta + sizeof(int) * (size_t)(g.grid + 1 + g.grid * g.phases));
+  }
+  if (at > R.bytes) {
     if (R.d_buf) cudaFree(R.d_buf);
     R.d_buf = nullptr;
     R.bytes = 0;
-    e = cudaMalloc(&R.d_buf, bytes);
+    e = cudaMalloc(&R.d_buf, at);
     if (e != cudaSuccess) return e;
-    R.bytes = bytes;
+    R.bytes = at;
   }
-  if (!R.stream) {
-    e = cudaStreamCreateWithFlags(&R.stream, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
+  std::vector<unsigned char> blob(at, 0);
+  memcpy(blob.data() + o_desc, descs.data(), descs.size());
+  for (const K2Group& g : groups) {
+    K2Tile* bt = reinterpret_cast<K2Tile*>(blob.data() + g.o_tile);
+    int* bc = reinterpret_cast<int*>(blob.data() + g.o_cta);
+    int n = 0;
+    for (int b = 0; b < g.grid; ++b) {
+      bc[b] = n;
+      for (const K2Tile& t : g.lists[b]) bt[n++] = t;
+    }
+    bc[g.grid] = n;
+    for (int b = 0; b < g.grid; ++b)
+      for (int ph = 0; ph < g.phases; ++ph) bc[g.grid + 1 + b * g.phases + ph] = g.phase_end[b][ph];
   }
   unsigned char* base = (unsigned char*)R.d_buf;
-  int64_t* d_done = (int64_t*)base;
-  const K2Desc* d_descs = (const K2Desc*)(base + 64);
-  const K2Tile* d_tiles = (const K2Tile*)(base + 64 + descs.size());
-  std::vector<unsigned char> blob(bytes, 0);
-  memcpy(blob.data() + 64, descs.data(), descs.size());
-  memcpy(blob.data() + 64 + descs.size(), tiles.data(), tiles.size() * sizeof(K2Tile));
-  e = cudaMemcpyAsync(base, blob.data(), bytes, cudaMemcpyHostToDevice, st);  // also zeroes *done
+  e = cudaMemcpyAsync(base, blob.data(), at, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
-
-  // ring depth per dimension: as many stages as the ring budget holds, or fewer when
-  // the autotuner chose so
-  std::vector<int> dim_stages(9, 0);
-  for (int D = 1; D <= 8; ++D) {
-    if (!dim_count[D]) continue;
-    dim_stages[D] = (int)std::min<size_t>(kMaxStages, std::max<size_t>(2, kRingBudget / dim_stride[D]));
-    if (stage_choice && stage_choice[D] >= 2) dim_stages[D] = std::min(dim_stages[D], stage_choice[D]);
-  }
-  auto issue = [&](int k_off, cudaStream_t s) -> cudaError_t {
-    for (int D = 1; D <= 8; ++D) {
-      if (!dim_count[D]) continue;
-      const int stages = dim_stages[D];
-      // at least 120 KB: one CTA (which owns 512 TMEM columns) per SM
-      const size_t smem = std::max<size_t>((size_t)stages * dim_stride[D], 120 * 1024);
-      const int grid = std::min(dim_count[D], max_ctas > 0 ? std::min(max_ctas, R.sms) : R.sms);  // as above
-      K2Launch L{d_descs, d_tiles + dim_first[D], d_done, dim_count[D], k_off, stages, dim_stride[D],
-                 status, stall ? kTestWaitLimitNs : kWaitLimitNs};
-      cudaError_t r = k2_launch(D, L, grid, smem, s);
-      if (r != cudaSuccess) return r;
+  if (beside) {
+    if (!R.fork) e = cudaEventCreateWithFlags(&R.fork, cudaEventDisableTiming);
+    for (size_t gi = 1; gi < groups.size() && e == cudaSuccess; ++gi) {
+      if (!R.streams[gi]) e = cudaStreamCreateWithFlags(&R.streams[gi], cudaStreamNonBlocking);
+      if (e == cudaSuccess && !R.joins[gi]) e = cudaEventCreateWithFlags(&R.joins[gi], cudaEventDisableTiming);
     }
-    return cudaSuccess;
-  };
-  const int64_t chunks = steps / kGraphSteps, rem = steps % kGraphSteps;
-  if (chunks > 0) {
-    // the graph stays valid while the tile table keeps its shape; the descriptor
-    // contents are refreshed in place above
-    const bool reuse = R.exec && R.sig_tiles == tiles.size() && R.sig_dims == dim_count &&
-                       R.sig_buf == R.d_buf && R.sig_cap == max_ctas && R.sig_stall == stall &&
-                       R.sig_stages == dim_stages;
-    if (!reuse) {
-      if (R.exec) cudaGraphExecDestroy(R.exec);
-      R.exec = nullptr;
-      cudaGraph_t g = nullptr;
-      e = cudaStreamBeginCapture(R.stream, cudaStreamCaptureModeRelaxed);
-      if (e != cudaSuccess) return e;
-      for (int s = 0; s < kGraphSteps && e == cudaSuccess; ++s) e = issue(s, R.stream);
-      if (e == cudaSuccess) {
-        k2_advance_kernel<<<1, 1, 0, R.stream>>>(d_done, kGraphSteps);
-        e = cudaGetLastError();
-      }
-      cudaError_t e2 = cudaStreamEndCapture(R.stream, &g);
-      if (e == cudaSuccess) e = e2;
-      if (e == cudaSuccess) e = cudaGraphInstantiate(&R.exec, g, 0);
-      if (g) cudaGraphDestroy(g);
-      if (e != cudaSuccess) return e;
-      R.sig_tiles = tiles.size();
-      R.sig_dims = dim_count;
-      R.sig_buf = R.d_buf;
-      R.sig_cap = max_ctas;
-      R.sig_stall = stall;
-      R.sig_stages = dim_stages;
-    }
-    for (int64_t c = 0; c < chunks; ++c) {
-      e = cudaGraphLaunch(R.exec, st);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  for (int s = 0; s < rem; ++s) {
-    e = issue(s, st);
+    if (e == cudaSuccess) e = cudaEventRecord(R.fork, st);
     if (e != cudaSuccess) return e;
+  }
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    const K2Group& g = groups[gi];
+    uint32_t stride = 0;
+    for (int i : g.descs) {
+      const K2Desc& d = desc(i);
+      stride = std::max(stride, (stage_bytes(d.n, d.a_terms, d.lo8) + 1023u) / 1024u * 1024u);
+    }
+    // ring depth: as many stages as the ring budget holds, or fewer when the autotuner chose so
+    int stages = (int)std::min<size_t>(kMaxStages, std::max<size_t>(2, kRingBudget / stride));
+    if (stage_choice && stage_choice[g.D] >= 2) stages = std::min(stages, stage_choice[g.D]);
+    // at least 120 KB: one CTA (which owns 512 TMEM columns) per SM
+    const size_t smem = std::max<size_t>((size_t)stages * stride, 120 * 1024);
+    const bool side = beside && gi > 0;
+    cudaStream_t s = side ? R.streams[gi] : st;
+    if (side && (e = cudaStreamWaitEvent(s, R.fork, 0)) != cudaSuccess) return e;
+    for (int64_t s0 = 0; s0 < steps; s0 += kLaunchSteps) {
+      if (s0 > 0 && (e = cudaMemsetAsync(base + g.o_sync, 0, sizeof(unsigned) * g.n_sync, s)) != cudaSuccess) return e;
+      K2Launch L;
+      L.descs = (const K2Desc*)(base + o_desc);
+      L.tiles = (const K2Tile*)(base + g.o_tile);
+      L.n_tiles = (int)g.n_tiles;
+      L.cta_begin = (const int*)(base + g.o_cta);
+      L.phase_end = L.cta_begin + g.grid + 1;
+      L.phases = g.phases;
+      L.sync = (unsigned*)(base + g.o_sync);
+      L.flags = L.sync + 4;
+      L.step0 = s0;
+      L.steps = (int)std::min<int64_t>(kLaunchSteps, steps - s0);
+      L.stages = stages;
+      L.stage_stride = stride;
+      L.status = status;
+      L.wait_ns = stall ? kTestWaitLimitNs : kWaitLimitNs;
+      e = k2_launch(g.D, L, g.grid, smem, s);
+      if (e != cudaSuccess) return e;
+    }
+    if (side) {
+      e = cudaEventRecord(R.joins[gi], s);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(st, R.joins[gi], 0);
+      if (e != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
 
 void k2_runner_release(K2Runner& R) {
-  if (R.exec) cudaGraphExecDestroy(R.exec);
   if (R.d_buf) cudaFree(R.d_buf);
-  if (R.stream) cudaStreamDestroy(R.stream);
+  if (R.fork) cudaEventDestroy(R.fork);
+  for (int i = 0; i < 8; ++i) {
+    if (R.streams[i]) cudaStreamDestroy(R.streams[i]);
+    if (R.joins[i]) cudaEventDestroy(R.joins[i]);
+  }
   R = K2Runner();
 }
 
 cudaError_t launch_step_k2(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
-  std::vector<unsigned char> desc(sizeof(K2Desc));
-  cudaError_t e = k2_prepare(c, sc, st, desc.data());
+  int sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (e != cudaSuccess) return e;
-  e = k2_integrate(c->k2_runner, desc, std::vector<int>{c->D}, sc.steps, c->d_status, st);
+  const int rt = k2_pick_rt({k2_shape(c, sc.fp8, sc.n_runs, 0)}, sms)[0];
+  std::vector<unsigned char> desc(sizeof(K2Desc));
+  e = k2_prepare(c, sc, st, desc.data(), rt);
+  if (e != cudaSuccess) return e;
+  e = k2_integrate(c->k2_runner, desc, std::vector<int>{c->D}, sc.steps, c->d_status, st, sms, nullptr);
   if (e != cudaSuccess) return e;
   return k2_finish(c, desc.data(), st);
 }

@@ -1,0 +1,86 @@
+"""Large-N tensor-core path: a run's trajectory depends neither on the column tiles, lists and
+phases its context's work is cut into, nor on the launches a call is cut into, nor on how
+many SMs the persistent launch finds free."""
+import numpy as np
+import pytest
+
+from paper_2308_02329_gb300 import chym, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(N, D, kind):
+    J = inputs.gaussian(N, 3) if kind == "gauss" else inputs.sk_pm1(N, 3)
+    ctx = chym.Context(J, D, chym.J_REAL if kind == "gauss" else chym.J_PM1)
+    eps = 0.25 if kind == "gauss" else 0.25 / np.sqrt(N)
+    return ctx, eps
+
+
+def _states(ctx, prm, sched, seeds, steps, stream=0):
+    ctx.run(prm, np.array([0.8]), seeds, steps, sched, stream)
+    X, k = ctx.get_state(stream)
+    assert k == steps
+    return X
+
+
+@pytest.mark.parametrize("N,D,kind,prec", [
+    (129, 1, "sk", chym.PREC_BF16X2), (256, 2, "sk", chym.PREC_FP8), (257, 3, "gauss", chym.PREC_BF16X2),
+    (385, 4, "sk", chym.PREC_FP8), (200, 5, "gauss", chym.PREC_BF16X2), (130, 8, "sk", chym.PREC_FP8)])
+@pytest.mark.parametrize("R", [1, 9, 24, 100, 130, 1030])
+def test_tiling_leaves_states_unchanged(N, D, kind, prec, R):
+    ctx, eps = _ctx(N, D, kind)
+    prm = chym.Params(eps=eps, prec=prec)
+    sched = chym.Schedule(1, 3, 8)
+    seeds = inputs.run_seeds(5, R)
+    X = _states(ctx, prm, sched, seeds, 6)
+    few = min(R, 5)   # the last runs alone: other tiles, widths and lists
+    assert np.array_equal(X[R - few:], _states(ctx, prm, sched, seeds[R - few:], 6))
+    ctx.close()
+
+
+@pytest.mark.parametrize("D,R", [(8, 9760), (4, 19500)])
+def test_phases_leave_states_unchanged(D, R):
+    """More tiles than four per SM and enough steps: the column tiles advance in phases."""
+    ctx, eps = _ctx(130, D, "sk")
+    prm = chym.Params(eps=eps, prec=chym.PREC_BF16X2)
+    sched = chym.Schedule(1, 16, 33)
+    seeds = inputs.run_seeds(6, R)
+    X = _states(ctx, prm, sched, seeds, 33)
+    for lo in (0, R // 2, R - 64):
+        assert np.array_equal(X[lo:lo + 64], _states(ctx, prm, sched, seeds[lo:lo + 64], 33))
+    ctx.close()
+
+
+def test_launch_boundaries_leave_states_unchanged():
+    """2060 steps take three launches; two calls cut them elsewhere."""
+    ctx, eps = _ctx(140, 3, "sk")
+    prm = chym.Params(eps=eps, prec=chym.PREC_FP8)
+    sched = chym.Schedule(1, 1000, 2060)
+    seeds = inputs.run_seeds(7, 40)
+    X = _states(ctx, prm, sched, seeds, 2060)
+    ctx.run(prm, np.array([0.8]), seeds, 777, sched)
+    ctx.run(prm, None, None, 2060 - 777, sched)
+    assert np.array_equal(ctx.get_state()[0], X)
+    ctx.close()
+
+
+@pytest.mark.parametrize("busy_runs", [40, 300, 590])
+def test_fewer_free_sms_leave_states_unchanged(busy_runs):
+    """Another stream's persistent small-N launch holds some SMs while the large-N one starts."""
+    torch = pytest.importorskip("torch")
+    ctx, eps = _ctx(260, 4, "sk")
+    prm = chym.Params(eps=eps, prec=chym.PREC_BF16X2)
+    sched = chym.Schedule(1, 5, 20)
+    seeds = inputs.run_seeds(8, 4096)
+    X = _states(ctx, prm, sched, seeds, 15)
+    small, seps = _ctx(100, 4, "sk")
+    sprm = chym.Params(eps=seps, prec=chym.PREC_BF16X2)
+    ssched, sseeds = chym.Schedule(1, 10000, 20000), inputs.run_seeds(9, busy_runs)
+    S = _states(small, sprm, ssched, sseeds, 20000)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    small.run(sprm, np.array([0.8]), sseeds, 20000, ssched, a.cuda_stream)
+    ctx.run(prm, np.array([0.8]), seeds, 15, sched, b.cuda_stream)
+    assert np.array_equal(ctx.get_state(b.cuda_stream)[0], X)
+    assert np.array_equal(small.get_state(a.cuda_stream)[0], S)
+    small.close()
+    ctx.close()
