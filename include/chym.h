@@ -350,7 +350,8 @@ CHYM_API chym_status chym_batch_set_tuning(chym_batch* b, const double* chunk_co
  * 256 / 128 / 64 / 32 for D = 1 / 2 / 3-4 / 5-8, fewer for contexts with fewer runs);
  * stages, the depth of its operand ring (2..8, capped by what its shared memory holds;
  * default: the most that fit); chunk, the runs per epilogue chunk of the small-N path
- * (4 or 8 for D <= 4; default 8).  chym_batch_tune chooses them by measurement after
+ * (4 or 8 for D <= 4, default
+ * 8; D = 4 runs in chunks of 4 either way).  chym_batch_tune chooses them by measurement after
  * its cost-model rounds: for each D with large-N contexts every valid rt, then the
  * three ring depths below the largest; for each D <= 4 with small-N contexts both
  * chunks; each part keeps the shape under which it ran fastest (the whole batch runs

@@ -33,11 +33,11 @@ struct chym_batch {
   int sms = 0;
   chym::K2Runner k2;
   // Cost model of the planner, in SM-microseconds: one 8- or 4-run chunk advanced
-  // one step on the small-N path, per dimension D; and one (128-row tile x K chunk
+  // one step on the small-N path, per dimension D (of a full item, see tc_step_chunks); and one (128-row tile x K chunk
   // of 64) advanced one step on the large-N path.  The defaults were measured on a
   // GB300; chym_batch_tune re-measures them for the batch's own contexts.
-  double chunk_cost[9] = {0, 1.10, 0.555, 0.89, 1.07, 1.27, 1.43, 1.60, 1.76};
-  double k2_cost = 1.05;
+  double chunk_cost[9] = {0, 0.27, 0.44, 0.70, 0.84, 0.66, 0.70, 0.94, 0.91};
+  double k2_cost = 0.65;
   bool tuned = false;
   // Tile shapes (0: the kernels' defaults), chosen by chym_batch_tune's search or set by
   // the caller: large-N runs per column tile and ring depth, small-N epilogue chunk.
@@ -142,28 +142,44 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
       if (e != cudaSuccess) return cuda_fail(e, "J operand image");
     }
   }
-  // work in SM-microseconds per step: each small-N dimension and the large-N group.
-  // The SMs are split in proportion, so that all parts finish together; the
-  // large-N launches take the SMs that the persistent small-N CTAs leave free.
-  double cost[9] = {0};
-  double total = 0.0;
+  // work in SM-microseconds per step: the small-N dimensions and the large-N group.  The SMs
+  // are split in proportion, so that all parts finish together; the large-N launches take the
+  // SMs that the persistent small-N CTAs leave free.
+  long long runs_of[9] = {0};
+  double small_total = 0.0, total = 0.0;
+  int dims = 0;
   for (int D = 1; D <= 8; ++D) {
-    for (int i : by_dim[D]) {
-      const int CH = tc_chunk_runs(D);
-      cost[D] += b->chunk_cost[D] * ((b->ctxs[i]->n_runs + CH - 1) / CH);
-    }
-    total += cost[D];
+    for (int i : by_dim[D]) runs_of[D] += b->ctxs[i]->n_runs;
+    if (runs_of[D]) small_total += b->chunk_cost[D] * (double)runs_of[D] / tc_chunk_runs(D);
+    dims += runs_of[D] ? 1 : 0;
   }
-  double small_total = total;
+  total = small_total;
   for (int i = 0; i < n; ++i) {
     const chym_ctx* c = b->ctxs[i];
     if (is_tc_prec(params[i].prec) && c->N > 128 && !uses_csr(c, params[i].prec))
       total += b->k2_cost * (double)k2_work_units(c->N, c->D, c->n_runs, b->shapes.rt[c->D]);
   }
-  // SMs for the small-N dimensions (all of them when there is no large-N work)
+  // SMs for the small-N dimensions (all of them when there is no large-N work), each next one
+  // to the dimension whose step takes longest on those it has: the chunks and items of its
+  // CTAs are whole numbers, so a split in proportion to the work can leave one dimension a
+  // whole item behind (N = 100, D = 2, 3, 4: 15.6 against 14.0 us a step)
   const int sms_small = small_total > 0.0
-                            ? std::min(b->sms, std::max(1, (int)llround(b->sms * small_total / total)))
+                            ? std::max(dims, std::min(b->sms, std::max(1, (int)llround(b->sms * small_total / total))))
                             : 0;
+  int ctas_of[9] = {0};
+  for (int s = 0; s < sms_small; ++s) {
+    int next = 0;
+    double longest = -1.0;
+    for (int D = 1; D <= 8; ++D) {
+      if (!runs_of[D]) continue;
+      const double t = ctas_of[D] ? b->chunk_cost[D] * tc_step_chunks(D, runs_of[D], ctas_of[D]) : INFINITY;
+      if (t > longest) {
+        longest = t;
+        next = D;
+      }
+    }
+    ++ctas_of[next];
+  }
   // plan: descriptors of all small-N contexts, then per dimension its items and CTA ranges
   std::vector<unsigned char> blob;
   const size_t db = tc_desc_bytes();
@@ -182,17 +198,9 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     bool stall;
   };
   std::vector<DimLaunch> dl;
-  int dims_left = 0;
-  for (int D = 1; D <= 8; ++D) dims_left += by_dim[D].empty() ? 0 : 1;
-  int sms_left = std::max(sms_small, dims_left);
   for (int D = 1; D <= 8; ++D) {
     if (by_dim[D].empty()) continue;
-    int P = std::max(1, (int)llround(sms_left * cost[D] / small_total));
-    small_total -= cost[D];
-    P = std::min(P, sms_left - (dims_left - 1));
-    P = std::max(P, 1);
-    sms_left -= P;
-    --dims_left;
+    const int P = ctas_of[D];
     std::vector<TcJob> jobs;
     int kp_max = 16, terms_max = 1;
     bool stall = false;
@@ -204,14 +212,11 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     }
     std::vector<unsigned char> items;
     std::vector<int> cta;
-    long long runs = 0;
-    for (const auto& j : jobs) runs += j.n_runs;
-    const int chunk = b->shapes.ch[D] ? b->shapes.ch[D] : tc_pick_chunk(D, runs, P);
+    const int chunk = b->shapes.ch[D] ? b->shapes.ch[D] : tc_pick_chunk(D, runs_of[D], P);
     tc_plan_items(jobs, chunk, tc_runs_per_item(D), P, items, cta);
     DimLaunch L{D, (int)cta.size() - 1, kp_max, terms_max, chunk, 0, 0, stall};
     b->part_ctas[D] = L.P;
-    b->part_units[D] = 0.0;
-    for (const auto& jj : jobs) b->part_units[D] += (double)((jj.n_runs + tc_chunk_runs(D) - 1) / tc_chunk_runs(D));
+    b->part_units[D] = tc_step_chunks(D, runs_of[D], L.P) * L.P;
     blob.resize((blob.size() + 15) / 16 * 16);
     L.items_off = blob.size();
     blob.insert(blob.end(), items.begin(), items.end());

@@ -278,6 +278,8 @@ struct TcJob {
 };
 // runs per epilogue chunk for `runs` runs of dimension D on P CTAs
 int tc_pick_chunk(int D, long long runs, int P);
+// cost of one step of `runs` runs of dimension D on P CTAs, in chunks of tc_chunk_runs(D) runs
+double tc_step_chunks(int D, long long runs, int P);
 // Split the runs of `jobs` (all of one dimension) over at most P CTAs in near-equal
 // numbers of `chunk`-run chunks; items never cross a context and hold at most `per_item`
 // runs.  items: packed TcItem records; cta_begin: first item of each CTA, and the end.

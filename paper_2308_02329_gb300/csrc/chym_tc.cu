@@ -3,9 +3,10 @@
 //
 // Per step, for every group of runs (one warpgroup of 128 threads, thread = spin
 // p = TMEM lane):
-//   1. one thread issues tcgen05.mma:  Y (128 x C, FP32 in TMEM) =
+//   1. one warp issues tcgen05.mma:  Y (128 x C, FP32 in TMEM) =
 //        J_hi X_hi + J_hi X_lo (+ J_lo X_hi for real J)            (C = J_N (x) 1_D, Eq. 1)
-//      A = J (BF16, K-major canonical layout, staged once by a TMA bulk copy),
+//      A = J (BF16): in TMEM, one row per lane (D = 1-4 and 6), or in shared memory
+//      (K-major canonical layout, staged once by a TMA bulk copy),
 //      B = X split into BF16 hi + lo (MN-major canonical layout in shared memory),
 //      columns ordered c = mu * R + r so a thread's 8 consecutive runs of one
 //      component are 8 consecutive columns;
@@ -63,12 +64,20 @@ struct TcLaunch {
 
 // CH_ = 0: the default runs per epilogue chunk (8 for D <= 4, else 4); the batch
 // autotuner may choose 4 for D <= 4.
+// kATmem: J sits in TMEM beside the accumulators and masters instead of shared memory.  A
+// product of N = 48 columns reads 4 KB of J against 1.5 KB of X, which keeps shared memory
+// busy for its whole 44 cycles (24 from TMEM) and stalls the other groups' epilogues: at
+// N = 100 the products of four groups added 1.2 us to a step of 4.8 to 7.2 us, overlapped
+// with nothing.  Groups are as wide as that leaves room for (CG = 48; J takes up to 128
+// columns); at D = 5, 7 and 8 it would cost whole groups, and J stays in shared memory.
 template <int D, int CH_ = 0>
 struct TcCfg {
-  static constexpr int RG = D == 1 ? 64 : D == 2 ? 32 : (D == 6 || D == 8) ? 8 : 16;
+  static constexpr bool kATmem = D <= 4 || D == 6;
+  static constexpr int RG = D == 1 ? 48 : D == 2 ? 24 : D == 4 ? 12 : (D == 6 || D == 8) ? 8 : 16;
   static constexpr int CG = D * RG;        // MMA N: columns of one group
-  static constexpr int CH = CH_ ? CH_ : D <= 4 ? 8 : 4;  // runs per epilogue chunk
-  static constexpr int G = std::min(4, 512 / (2 * CG));
+  static constexpr int CH = D <= 3 ? (CH_ ? CH_ : 8) : 4;  // runs per epilogue chunk
+  static constexpr int G = std::min(4, (kATmem ? 384 : 512) / (2 * CG));
+  static constexpr int kACol = 2 * G * CG;  // J's first TMEM column
   static_assert(CG % 16 == 0 && CG <= 256, "MMA N must be a multiple of 16 in [16, 256]");
   static_assert(RG % CH == 0, "chunk must divide the group");
 };
@@ -112,12 +121,30 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
+// D (+)= A B, issued by one elected lane of a converged warp: the whole warp runs the issue
+// loop, so that the descriptors stay in uniform registers (44 cycles a product of N = 48, the
+// tensor core's own rate; a lone thread's loop took 65 to 150).
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+// The same with A in TMEM (lane = row, two BF16 of K per column).
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate));
+}
+// Arrival on an mbarrier once the products issued so far are complete (same elected lane).
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(bar)
+      : "memory");
 }
 
 // Loads of the accumulator (ya) and master state (xa) columns followed by the wait
@@ -240,11 +267,25 @@ __device__ __forceinline__ void philox_round(uint4& c, uint32_t k0, uint32_t k1)
                  (uint32_t)p0);
 }
 
-// Philox4x32-10 with the ten round keys precomputed (two rounds per uint4):
-// the key schedule depends on the run only, so it is built once per launch.
-__device__ __forceinline__ uint4 philox_rk(uint4 c, const uint4* __restrict__ rk) {
+// The first two Philox rounds of counter (p, blk, k_lo, k_hi) as far as they depend on the
+// run and the step only (k' = the round-2 key): round 1 multiplies p and k_lo, round 2 the
+// result c of k_lo's product:
+//   x = k_hi ^ k1, y = lo(M1 k_lo) ^ k0', z = hi(M0 c) ^ k1', w = lo(M0 c) with
+//   c = hi(M1 k_lo) ^ blk ^ k0.
+__device__ __forceinline__ uint4 run_rounds12(uint32_t blk, uint64_t k, uint32_t k0, uint32_t k1) {
+  const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint32_t)k;
+  const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ blk ^ k0);
+  return make_uint4((uint32_t)(k >> 32) ^ k1, (uint32_t)p1 ^ (k0 + kPhiloxW0), (uint32_t)(p0 >> 32) ^ (k1 + kPhiloxW1),
+                    (uint32_t)p0);
+}
+
+// Philox4x32-10 of the thread's spin (mp = M0 p) from that table entry t of the run and its
+// keys rk of rounds 3..10 (two rounds per uint4): 17 products instead of 20.
+__device__ __forceinline__ uint4 philox_run(uint64_t mp, const uint4& t, const uint4* __restrict__ rk) {
+  const uint64_t q = (uint64_t)kPhiloxM1 * ((uint32_t)(mp >> 32) ^ t.x);
+  uint4 c = make_uint4((uint32_t)(q >> 32) ^ t.y, (uint32_t)q, t.z ^ (uint32_t)mp, t.w);
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
+  for (int i = 0; i < 4; ++i) {
     const uint4 kk = rk[i];
     philox_round(c, kk.x, kk.y);
     philox_round(c, kk.z, kk.w);
@@ -314,9 +355,10 @@ __device__ __forceinline__ void quad_transpose(float v0, float v1, float v2, flo
 }
 
 template <int D, int CH_>
-__global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
+__global__ void __launch_bounds__(128 * TcCfg<D, CH_>::G, 1) step_tc_kernel(TcLaunch L) {
   using Cfg = TcCfg<D, CH_>;
   constexpr int RG = Cfg::RG, CG = Cfg::CG, CH = Cfg::CH, G = Cfg::G;
+  constexpr bool kATmem = Cfg::kATmem;
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
@@ -324,17 +366,21 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
   __shared__ __align__(8) uint64_t s_abar;
   __shared__ __align__(8) uint64_t s_wh[G];  // CHYM_FLAG_TEST_STALL: where the completion goes instead
   __shared__ __align__(8) float s_ar[G][RG];
-  __shared__ uint4 s_rk[G][RG][5];  // Philox round keys of each run
+  __shared__ uint4 s_rk[G][RG][4];  // Philox keys of rounds 3..10 of each run
+  constexpr int NB = (D + 3) / 4;   // Philox blocks per spin
+  // run_rounds12 of each run at the current step, double buffered by step parity (written
+  // one step ahead by the run's own thread)
+  __shared__ uint4 s_r12[2][G][NB][RG];
   __shared__ int64_t s_koff[G][RG];  // each run's (re)seeding step
   __shared__ int s_kuni[G];           // 1 when all runs of the group share one offset
-  // when they do not: each run's local step and annealing scale at the current step,
-  // double buffered by step parity (written one step ahead by the run's own thread)
-  __shared__ __align__(16) int64_t s_kl[2][G][RG];
+  // when they do not: each run's annealing scale at the current step, likewise
   __shared__ __align__(8) float s_rp[2][G][RG];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = warp >> 2, wq = warp & 3;
   const int p = wq * 32 + lane;  // spin = TMEM lane
+  // one warp of each group issues its products, another scheduler's in each group
+  const bool issuer = wq == (g & 3);
   const uint32_t b_bytes = (uint32_t)L.kp_max * CG * 2u;
   uint8_t* Bhi = smem + L.a_region + (size_t)g * 2 * b_bytes;
   uint8_t* Blo = Bhi + b_bytes;
@@ -368,6 +414,8 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
                          ((uint32_t)(CG >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   const uint32_t a_base = smem_addr(smem);
   const uint32_t bhi_base = smem_addr(Bhi), blo_base = smem_addr(Blo);
+  // first product of Philox: spin p, or its group of 4/D spins for D <= 2
+  const uint64_t mp = (uint64_t)kPhiloxM0 * (D == 1 ? (uint32_t)p >> 2 : D == 2 ? (uint32_t)p >> 1 : (uint32_t)p);
   uint32_t phase = 0, a_phase = 0;
   int a_desc = -1;
   bool aborted = false;
@@ -377,12 +425,25 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
     const TcDesc d = L.descs[item.desc];
     const int N = d.N, KP = d.KP;
     const uint32_t a_bytes = 128u * (uint32_t)KP * 2u;
-    // the item's runs are spread evenly over the groups in whole chunks
-    const int per_g = min(RG, ((item.run_count + G - 1) / G + CH - 1) / CH * CH);
-    const int run0 = item.run_begin + g * per_g;
-    const int nr = max(0, min(per_g, item.run_begin + item.run_count - run0));
+    // the item's runs are spread evenly over the groups in whole chunks (34 runs at D = 4: 3, 2,
+    // 2 and 2 chunks of 4 rather than 3, 3, 3 and none)
+    const int chunks = (item.run_count + CH - 1) / CH, even = chunks / G, extra = chunks % G;
+    const int run0 = item.run_begin + CH * (g * even + min(g, extra));
+    const int nr = max(0, min(CH * (even + (g < extra ? 1 : 0)), item.run_begin + item.run_count - run0));
     const bool new_a = item.desc != a_desc;  // CTA-uniform
-    if (new_a && tid == 0) {                 // TMA bulk copy of the context's J image
+    if (kATmem && new_a) {
+      // row p of the context's J image into TMEM, four columns (8 couplings) a store, the
+      // groups taking turns; the previous item's products are complete
+      const int k8 = KP / 8;
+      for (int kb = g; kb < d.a_terms * k8; kb += G) {
+        const uint8_t* row = d.Aimg + (size_t)(kb / k8) * a_bytes + (size_t)(p / 8) * k8 * 128u + (size_t)(kb % k8) * 128u +
+                             (size_t)(p % 8) * 16u;
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(row));
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(t_lane + (uint32_t)(Cfg::kACol + 4 * kb)),
+                     "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w));
+      }
+    }
+    if (!kATmem && new_a && tid == 0) {      // TMA bulk copy of the context's J image
       const uint32_t bytes = (uint32_t)d.a_terms * a_bytes;
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_abar)),
                    "r"(bytes)
@@ -394,6 +455,7 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
           : "memory");
     }
     // per-run constants of this group: 1 + dt (h - 1) and the Philox round keys
+    uint32_t key0 = 0u, key1 = 0u;  // of run p
     if (p < RG) {
       const int run = run0 + p;
       float ar = 0.f;
@@ -406,9 +468,12 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
       }
       s_ar[g][p] = ar;
       s_koff[g][p] = p < nr ? d.koff[run] : 0;
-      for (int i = 0; i < 5; ++i) {  // Weyl key schedule: round r uses key + r * (W0, W1)
-        s_rk[g][p][i] = make_uint4(k0 + (2u * i) * kPhiloxW0, k1 + (2u * i) * kPhiloxW1,
-                                   k0 + (2u * i + 1u) * kPhiloxW0, k1 + (2u * i + 1u) * kPhiloxW1);
+      key0 = k0;
+      key1 = k1;
+      for (uint32_t i = 0; i < 4; ++i) {  // Weyl key schedule: round r (0-based) uses key + r * (W0, W1)
+        const uint32_t r = 2u * i + 2u;
+        s_rk[g][p][i] = make_uint4(k0 + r * kPhiloxW0, k1 + r * kPhiloxW1, k0 + (r + 1u) * kPhiloxW0,
+                                   k1 + (r + 1u) * kPhiloxW1);
       }
     }
     if (p == 0) s_kuni[g] = 1;
@@ -417,15 +482,16 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
       *reinterpret_cast<uint4*>(Bhi + o) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();  // every zero must land before any thread writes its state into B
     if (p < nr && s_koff[g][p] != s_koff[g][0]) s_kuni[g] = 0;
-    // run p's local step at step kk (noise counter) and its annealing scale alpha_mu
-    // (mu >= 1), for the per-run path
+    // run p's first Philox rounds at step kk and, for the per-run path, its annealing scale
+    // alpha_mu (mu >= 1)
     auto put_step = [&](int64_t kk) {
       if (p < RG) {
         const int64_t kl = kk - s_koff[g][p];
+#pragma unroll
+        for (int b = 0; b < NB; ++b) s_r12[kk & 1][g][b][p] = run_rounds12((uint32_t)b, (uint64_t)kl, key0, key1);
         float rp = 1.f;
         if (d.sched_kind == 1 && kl >= d.k_anneal)
           rp = kl >= d.k_total ? 0.f : fmaxf(0.f, 1.f - (float)(kl - d.k_anneal) * d.inv_ramp);
-        s_kl[kk & 1][g][p] = kl;
         s_rp[kk & 1][g][p] = rp;
       }
     };
@@ -459,40 +525,44 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
     const int ksteps = KP / 16;
     const float neg2ln2s2 = -1.3862943611198906f * d.noise_scale * d.noise_scale;
     const float2 ngdt = make_float2(-d.gdt, -d.gdt), nkdt = make_float2(-d.kdt, -d.kdt);
-    bool timed_out = false, a_pending = new_a;
+    bool timed_out = false, a_pending = !kATmem && new_a;
     if (nr > 0) {
       for (int64_t k = d.k0; k < d.k0 + L.steps; ++k) {
-        if (wq == 0 && lane == 0) {
+        if (issuer) {
           bool ok = true;
-          if (a_pending) ok = mbar_wait(smem_addr(&s_abar), a_phase, L.wait_ns);
+          if (a_pending) ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_abar), a_phase, L.wait_ns));
           a_pending = false;
           tc_fence_after();
           if (ok) {
             // a K step moves only the 14-bit start-address field of each descriptor
-            // (shared addresses stay below 256 KB, so the field never carries)
-            const uint64_t da0 = smem_desc(a_base, 128u, a_sbo), dj0 = smem_desc(a_base + a_bytes, 128u, a_sbo);
+            // (shared addresses stay below 256 KB, so the field never carries), or 8 columns of TMEM
             const uint64_t dh0 = smem_desc(bhi_base, lbo_b, 128u), dl0 = smem_desc(blo_base, lbo_b, 128u);
             const uint64_t sa = 256u >> 4, sb = (2u * lbo_b) >> 4;
-            for (int ks = 0; ks < ksteps; ++ks)
-              mma_bf16(tmem + acc_col, da0 + ks * sa, dh0 + ks * sb, idesc, ks > 0);
-            for (int ks = 0; ks < ksteps; ++ks)
-              mma_bf16(tmem + acc_col, da0 + ks * sa, dl0 + ks * sb, idesc, 1u);
-            if (d.a_terms > 1) {
-              for (int ks = 0; ks < ksteps; ++ks)
-                mma_bf16(tmem + acc_col, dj0 + ks * sa, dh0 + ks * sb, idesc, 1u);
+            const uint32_t acc = tmem + acc_col;
+            if constexpr (kATmem) {
+              const uint32_t ta = tmem + (uint32_t)Cfg::kACol;
+              for (int ks = 0; ks < ksteps; ++ks) mma_bf16_ts(acc, ta + 8 * ks, dh0 + ks * sb, idesc, ks > 0);
+              for (int ks = 0; ks < ksteps; ++ks) mma_bf16_ts(acc, ta + 8 * ks, dl0 + ks * sb, idesc, 1u);
+              if (d.a_terms > 1)
+                for (int ks = 0; ks < ksteps; ++ks)
+                  mma_bf16_ts(acc, ta + 8 * (ksteps + ks), dh0 + ks * sb, idesc, 1u);
+            } else {
+              const uint64_t da0 = smem_desc(a_base, 128u, a_sbo), dj0 = smem_desc(a_base + a_bytes, 128u, a_sbo);
+              for (int ks = 0; ks < ksteps; ++ks) mma_bf16(acc, da0 + ks * sa, dh0 + ks * sb, idesc, ks > 0);
+              for (int ks = 0; ks < ksteps; ++ks) mma_bf16(acc, da0 + ks * sa, dl0 + ks * sb, idesc, 1u);
+              if (d.a_terms > 1)
+                for (int ks = 0; ks < ksteps; ++ks) mma_bf16(acc, dj0 + ks * sa, dh0 + ks * sb, idesc, 1u);
             }
             // (test of the timeout path: the completion signal goes elsewhere, so the
             // group's wait below runs out; the drain after the loop waits for it)
-            asm volatile(
-                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_addr(d.stall ? &s_wh[g] : &s_mbar[g]))
-                : "memory");
-          } else {
+            mma_commit(smem_addr(d.stall ? &s_wh[g] : &s_mbar[g]));
+          } else if (lane == 0) {
             atomicOr(L.status, STATUS_TIMEOUT);
             s_abort = 1;
             // nothing was issued: complete the phase so the group does not wait
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&s_mbar[g])) : "memory");
           }
+          __syncwarp();
         }
         // warp-uniform outcome: the TMEM loads below are warp-collective
         const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&s_mbar[g]), phase, L.wait_ns));
@@ -522,14 +592,9 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
               for (int j = 0; j < CH; j += 2) {  // two runs at once, FP32x2 arithmetic
                 const int r = r0 + j;
                 const float2 ar = *reinterpret_cast<const float2*>(&s_ar[g][r]);
-                // each run's local step: noise counter and annealing scale alpha_mu
-                int64_t klA = kl_u, klB = kl_u;
-                float rA = ramp_u, rB = ramp_u;
+                float rA = ramp_u, rB = ramp_u;  // each run's annealing scale alpha_mu
                 if (!k_uniform) {
-                  const longlong2 kl2 = *reinterpret_cast<const longlong2*>(&s_kl[k & 1][g][r]);
                   const float2 rp2 = *reinterpret_cast<const float2*>(&s_rp[k & 1][g][r]);
-                  klA = kl2.x;
-                  klB = kl2.y;
                   rA = rp2.x;
                   rB = rp2.y;
                 }
@@ -540,8 +605,8 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
                   // spin, pair 1: the odd one): each lane draws the block of one of the
                   // two runs and hands the partner spin's pair to the partner lane
                   const bool odd = (p & 1) != 0;
-                  const uint4 w = philox_rk(noise_counter((uint32_t)p >> 1, 0u, 0u, (uint64_t)(odd ? klB : klA)),
-                                            s_rk[g][odd ? r + 1 : r]);
+                  const int ro = odd ? r + 1 : r;
+                  const uint4 w = philox_run(mp, s_r12[k & 1][g][0][ro], s_rk[g][ro]);
                   float2 zc, zs;
                   box_muller_x2(w.x, w.y, w.z, w.w, neg2ln2s2, zc, zs);
                   const float kc = odd ? zc.y : zc.x, ks = odd ? zs.y : zs.x;  // own spin, own run
@@ -556,8 +621,7 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
                   // and the quad transposes the normals
                   if ((j & 3) == 0) {
                     const int m = p & 3, rm = r + m;
-                    const int64_t klm = k_uniform ? kl_u : s_kl[k & 1][g][rm];
-                    const uint4 w = philox_rk(noise_counter((uint32_t)p >> 2, 0u, 0u, (uint64_t)klm), s_rk[g][rm]);
+                    const uint4 w = philox_run(mp, s_r12[k & 1][g][0][rm], s_rk[g][rm]);
                     float2 zc, zs;  // normals (0, 2) and (1, 3) of the block
                     box_muller_x2(w.x, w.y, w.z, w.w, neg2ln2s2, zc, zs);
                     quad_transpose(zc.x, zs.x, zc.y, zs.y, m, nq);
@@ -566,11 +630,9 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
                   if (!live) continue;
                 } else {
 #pragma unroll
-                  for (int blk = 0; blk < (D + 3) / 4; ++blk) {
-                    const uint4 wA = philox_rk(noise_counter((uint32_t)p, (uint32_t)blk, 0u, (uint64_t)klA),
-                                               s_rk[g][r]);
-                    const uint4 wB = philox_rk(noise_counter((uint32_t)p, (uint32_t)blk, 0u, (uint64_t)klB),
-                                               s_rk[g][r + 1]);
+                  for (int blk = 0; blk < NB; ++blk) {
+                    const uint4 wA = philox_run(mp, s_r12[k & 1][g][blk][r], s_rk[g][r]);
+                    const uint4 wB = philox_run(mp, s_r12[k & 1][g][blk][r + 1], s_rk[g][r + 1]);
                     box_muller_x2(wA.x, wA.y, wB.x, wB.y, neg2ln2s2, z[4 * blk], z[4 * blk + 1]);
                     if (D - 4 * blk > 2)
                       box_muller_x2(wA.z, wA.w, wB.z, wB.w, neg2ln2s2, z[4 * blk + 2], z[4 * blk + 3]);
@@ -602,14 +664,14 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
             }
           }
         }
-        if (!k_uniform) put_step(k + 1);  // the other parity: nobody reads it in this step
+        put_step(k + 1);  // the other parity: nobody reads it in this step
         tmem_wait_st();
         fence_async_smem();
         tc_fence_before();
         if (group_bar_or(1 + g, s_abort)) break;
       }
     }
-    if (wq == 0 && lane == 0) {
+    if (issuer && lane == 0) {
       // the J copy must have landed before the next item may overwrite it
       if (a_pending) mbar_wait(smem_addr(&s_abar), a_phase, L.wait_ns);
       // the tensor core may still own this group's accumulator: wait once more (bounded)
@@ -620,7 +682,7 @@ __global__ void __launch_bounds__(512, 1) step_tc_kernel(TcLaunch L) {
       }
     }
     if (new_a) {
-      a_phase ^= 1u;
+      if (!kATmem) a_phase ^= 1u;
       a_desc = item.desc;
     }
     tc_fence_before();
@@ -671,12 +733,13 @@ float bf16_value(uint16_t b) {
 }
 
 template <int D, int CH_>
-cudaError_t launch_tc_plan(const TcLaunch& L, int n_cta, cudaStream_t st) {
+cudaError_t launch_tc_plan(TcLaunch L, int n_cta, cudaStream_t st) {
   using Cfg = TcCfg<D, CH_>;
   const size_t b_bytes = (size_t)L.kp_max * Cfg::CG * 2u;
   // at least 128 KB: one CTA owns all 512 TMEM columns of its SM, so neither a
   // second CTA of this kernel nor a large-N step CTA (>= 104 KB) may be placed
   // beside it (it would wait in tcgen05.alloc until this CTA exits)
+  if (Cfg::kATmem) L.a_region = 0;
   const size_t smem = std::max<size_t>(L.a_region + (size_t)Cfg::G * 2 * b_bytes, 128 * 1024);
   auto kern = step_tc_kernel<D, CH_>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -758,10 +821,30 @@ void tc_fill_item(void* out, int desc, int run_begin, int run_count) {
 
 // Four-run chunks while every group of the P CTAs has at most one of them: a step then
 // waits for half an epilogue (the step is a serial chain of products, epilogue and group
-// barrier).  From there on eight-run chunks, which issue fewer TMEM and shared-memory
-// instructions per run (N = 100 batch: 4 % faster than four-run chunks).
+// barrier; N = 100, D = 3, 16 runs a CTA: 2.18 us a step in four chunks, 2.48 in two of 8).
+// From there on eight-run chunks, which issue fewer TMEM and shared-memory instructions per
+// run (32 runs: 3.22 against 3.31).
 int tc_pick_chunk(int D, long long runs, int P) {
-  return D <= 4 && runs > 4LL * tc_groups(D) * P ? 8 : 4;
+  return D <= 3 && runs > 4LL * tc_groups(D) * P ? 8 : 4;
+}
+
+// One step of an item with c chunks takes fixed + round ceil(c / groups) + chunk c microseconds:
+// its products, waits and barriers, the longest group's chunks one after the other, and the
+// chunks' share of the arithmetic units.  Fitted at N = 100 to within 5 % (D = 3: 3.23 us with 4
+// chunks, 4.45 with 5, 5.62 with 8).  In chunks of the cost of a full item's.
+double tc_step_chunks(int D, long long runs, int P) {
+  struct Fit {
+    double fixed, round, chunk;
+  };
+  constexpr Fit fits[9] = {{},           {1.00, 0.06, 0.21}, {0.97, 0.60, 0.21}, {0.82, 0.93, 0.37}, {0.90, 0.58, 0.20},
+                           {1.50, 0.40, 0.40}, {0.90, 0.87, 0.37}, {1.25, 0.05, 0.75}, {1.75, 0.35, 0.60}};
+  const int unit = D <= 3 ? 8 : 4, full = tc_runs_per_item(D) / unit, G = tc_groups(D);
+  auto item = [&](long long c) {
+    return c ? fits[D].fixed + fits[D].round * (double)((c + G - 1) / G) + fits[D].chunk * (double)c : 0.0;
+  };
+  const long long k = ((runs + unit - 1) / unit + P - 1) / P;  // chunks of the longest list
+  const double t = (double)(k / full) * item(full) + item(k % full);
+  return t * full * unit / (item(full) * tc_chunk_runs(D));
 }
 
 void tc_plan_items(const std::vector<TcJob>& jobs, int chunk, int per_item, int P,
@@ -816,7 +899,7 @@ cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, con
     case 1: return chunk == 4 ? launch_tc_plan<1, 4>(L, n_cta, st) : launch_tc_plan<1, 0>(L, n_cta, st);
     case 2: return chunk == 4 ? launch_tc_plan<2, 4>(L, n_cta, st) : launch_tc_plan<2, 0>(L, n_cta, st);
     case 3: return chunk == 4 ? launch_tc_plan<3, 4>(L, n_cta, st) : launch_tc_plan<3, 0>(L, n_cta, st);
-    case 4: return chunk == 4 ? launch_tc_plan<4, 4>(L, n_cta, st) : launch_tc_plan<4, 0>(L, n_cta, st);
+    case 4: return launch_tc_plan<4, 0>(L, n_cta, st);
     case 5: return launch_tc_plan<5, 0>(L, n_cta, st);
     case 6: return launch_tc_plan<6, 0>(L, n_cta, st);
     case 7: return launch_tc_plan<7, 0>(L, n_cta, st);
