@@ -9,8 +9,9 @@
 //   phase B  x <- x + dt [(h-1) x - kappa x^3 - gamma x |x_p|^2 + eps alpha_mu y]
 //            + sigma sqrt(dt) xi  with xi from Philox4x32-10 + Box-Muller.
 // FP32 runs on the register-tiled kernel (step_simt_tiled_kernel, below), whose
-// threads each own 4 spins x RB runs through both phases; FP64, and FP32 where a
-// tile's state does not fit, run on the per-spin kernel (step_simt_kernel), whose
+// threads each own 4 spins x RB runs through both phases; FP64 runs on step_f64_kernel,
+// with the noise drawn ahead by warps of its own; both, where their buffers do not fit, run on
+// the per-spin kernel (step_simt_kernel), whose
 // threads each take one (spin, run group) in phase A and one (spin, run) in phase B,
 // with J staged in shared memory when it fits and read through L1/L2 otherwise.
 #include <algorithm>
@@ -224,6 +225,140 @@ __global__ void __launch_bounds__(CSR && sizeof(T) == 4 ? 1024 : 512) step_simt_
     __syncthreads();
   }
   for (int i = tid; i < nr * N * D; i += nt) Xg[(size_t)run0 * N * D + i] = Xs[i];
+}
+
+// ---------------------------------------------------------------------------
+// FP64 form.  The FP64 units take 16 cycles for a warp's instruction, so what counts is full
+// warps and several of them under way: the state's warps take one (run, spin, component)
+// per thread, and the noise's warps draw the next step's Box-Muller pairs, one per thread,
+// at the same time.  State and noise are double buffered, one barrier a step.  N = 20, D = 3,
+// 256 runs: 3.9 us a step (8.9 with one thread per (run, spin) through product, noise and
+// update, 20 of 64 threads busy).  Every value is formed by the same operations as there.
+template <int D, bool J_SMEM, bool CSR>
+__global__ void __launch_bounds__(512) step_f64_kernel(const double* __restrict__ Jg, double* __restrict__ Xg,
+                                                       const double* __restrict__ hg,
+                                                       const uint64_t* __restrict__ seeds, StepConsts sc, int RC,
+                                                       int state_warps, CsrRows<double> csr) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = sc.N, size = RC * N * D;
+  double* Js = reinterpret_cast<double*>(smem_raw);
+  double* Xs = J_SMEM ? Js + (size_t)N * N : Js;  // two state buffers, two noise buffers
+  double* Zs = Xs + 2 * (size_t)size;
+  const int run0 = blockIdx.x * RC;
+  const int nr = min(RC, sc.n_runs - run0), used = nr * N * D;
+  const int tid = threadIdx.x, nt = blockDim.x, ns = 32 * state_warps;
+  if (J_SMEM)
+    for (int i = tid; i < N * N; i += nt) Js[i] = Jg[i];
+  for (int i = tid; i < used; i += nt) Xs[i] = Xg[(size_t)run0 * N * D + i];
+  const double* Jsrc = J_SMEM ? Js : Jg;
+  // the pairs of a run: a spin's pairs (D >= 3: ceil(D / 2)), or for D <= 2 the pairs of the
+  // blocks that 4 / D spins share
+  constexpr int kPairs = (D + 1) / 2;  // per spin, D >= 3
+  const int pairs = D >= 3 ? N * kPairs : (N * D + 1) / 2;
+  auto draw = [&](int64_t k, double* Z, int first, int stride) {
+    for (int t = first; t < nr * pairs; t += stride) {
+      const int r = t / pairs, j = t % pairs, run = run0 + r;
+      const uint64_t kl = (uint64_t)(k - sc.koff[run]), seed = seeds[run];
+      uint32_t ctr, blk;
+      int half, at;  // half: pair of the block; at: first value in the run's N D
+      if constexpr (D >= 3) {
+        const int p = j / kPairs, m = j % kPairs;
+        ctr = (uint32_t)p;
+        blk = (uint32_t)(m / 2);
+        half = m % 2;
+        at = p * D + 2 * m;
+      } else {
+        ctr = (uint32_t)(j / 2);
+        blk = 0u;
+        half = j % 2;
+        at = 2 * j;
+      }
+      const uint4 w = philox4x32_10(noise_counter(ctr, blk, 0u, kl), (uint32_t)seed, (uint32_t)(seed >> 32));
+      double z0, z1;
+      box_muller_f64(half ? w.z : w.x, half ? w.w : w.y, z0, z1);
+      double* z = Z + (size_t)r * N * D + at;
+      z[0] = z0 * sc.noise_scale;
+      if (D >= 3 ? at % D + 1 < D : at + 1 < N * D) z[1] = z1 * sc.noise_scale;
+    }
+  };
+  draw(sc.k0, Zs, tid, nt);
+  __syncthreads();
+  const double dt = sc.dt, gamma = sc.gamma, kappa = sc.kappa;
+  const double inv_ramp = sc.sched_kind == 1 ? 1.0 / (double)(sc.k_total - sc.k_anneal) : 0.0;
+  int cur = 0;
+  for (int64_t k = sc.k0; k < sc.k0 + sc.steps; ++k, cur ^= 1) {
+    const double* X = Xs + (size_t)cur * size;
+    const double* Z = Zs + (size_t)cur * size;
+    if (tid >= ns) {
+      if (k + 1 < sc.k0 + sc.steps) draw(k + 1, Zs + (size_t)(cur ^ 1) * size, tid - ns, nt - ns);
+    } else {
+      double* Xn = Xs + (size_t)(cur ^ 1) * size;
+      for (int i = tid; i < used; i += ns) {
+        const int mu = i % D, p = i / D % N, r = i / (N * D), run = run0 + r;
+        const double* xr = X + (size_t)r * N * D;
+        double y = 0.0;
+        if constexpr (CSR) {
+          const int e1 = __ldg(csr.rp + p + 1);
+          for (int e = __ldg(csr.rp + p); e < e1; ++e) y = fma(__ldg(csr.cv + e), xr[__ldg(csr.ci + e) * D + mu], y);
+        } else {
+#pragma unroll 4
+          for (int q = 0; q < N; ++q) y = fma(J_SMEM ? Jsrc[q * N + p] : __ldg(Jsrc + (size_t)q * N + p), xr[q * D + mu], y);
+        }
+        const int64_t kl = k - sc.koff[run];
+        double ramp = 1.0;  // alpha_mu(kl) for mu >= 1; mu = 0 keeps alpha = 1
+        if (mu > 0 && sc.sched_kind == 1 && kl >= sc.k_anneal)
+          ramp = kl >= sc.k_total ? 0.0 : 1.0 - (double)(kl - sc.k_anneal) * inv_ramp;
+        const double wp = sc.w ? sc.w[p] : 1.0;  // this spin's coupling weight
+        const double hm1 = hg[sc.hidx[run]] - 1.0;
+        double n2 = 0.0;
+#pragma unroll
+        for (int m = 0; m < D; ++m) n2 = fma(xr[p * D + m], xr[p * D + m], n2);
+        const double xm = xr[p * D + mu];
+        const double f = hm1 * xm - kappa * xm * xm * xm - gamma * xm * n2 + sc.eps * wp * ramp * y;
+        Xn[i] = xm + dt * f + Z[i];
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < used; i += nt) Xg[(size_t)run0 * N * D + i] = Xs[(size_t)cur * size + i];
+}
+
+// Launch of the FP64 form; InvalidConfiguration when a run's buffers do not fit its shared
+// memory (the caller then takes the per-spin kernel, which holds half as much).
+template <int D>
+cudaError_t launch_f64(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
+  const int N = c->N;
+  const bool csr = c->sparse;
+  const size_t j_bytes = (size_t)N * N * sizeof(double), per_run = (size_t)4 * N * D * sizeof(double);
+  const bool j_smem = !csr && j_bytes <= kSimtSmemBudget / 2;
+  const size_t avail = kSimtSmemBudget - (j_smem ? j_bytes : 0);
+  if (per_run > avail) return cudaErrorInvalidConfiguration;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  // as many runs a CTA as give every SM one, within shared memory and one state value a thread
+  // of 512 where that suffices
+  const int fit = (int)std::min<size_t>(avail / per_run, 64);
+  int RC = std::max(1, std::min(fit, (sc.n_runs + sms - 1) / sms));
+  while (RC > 1 && RC * N * D > 512) --RC;
+  // warps in proportion to the FP64 work: a state value costs a row of J and about 12
+  // operations, a pair of normals about 70 (logarithm, square root, sine and cosine)
+  const double row = csr ? (double)c->nnz / N : (double)N;
+  const int values = RC * N * D, pairs = RC * (D >= 3 ? N * ((D + 1) / 2) : (N * D + 1) / 2);
+  const double ws = values * (row + 12.0), wn = pairs * 70.0;
+  const int want_s = (values + 31) / 32, want_n = (pairs + 31) / 32;
+  int state_warps = want_s, noise_warps = want_n;
+  if (want_s + want_n > 16) {
+    state_warps = std::min(want_s, std::max(1, std::min(15, (int)(16.0 * ws / (ws + wn) + 0.5))));
+    noise_warps = std::min(want_n, 16 - state_warps);
+  }
+  const size_t smem = (j_smem ? j_bytes : 0) + (size_t)RC * per_run;
+  const CsrRows<double> rows{c->d_rp, c->d_ci, c->d_cv64};
+  auto kern = csr ? step_f64_kernel<D, false, true> : j_smem ? step_f64_kernel<D, true, false> : step_f64_kernel<D, false, false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(sc.n_runs + RC - 1) / RC, 32 * (state_warps + noise_warps), smem, st>>>(
+      c->d_J64, (double*)c->d_X, c->d_h, c->d_seeds, sc, RC, state_warps, rows);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -475,6 +610,9 @@ cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st
   const bool csr = c->sparse;  // the SIMT kernels use the compressed rows whenever they exist
   if constexpr (sizeof(T) == 4) {
     const cudaError_t e = csr ? launch_simt_tiled<D, true>(c, sc, st) : launch_simt_tiled<D, false>(c, sc, st);
+    if (e != cudaErrorInvalidConfiguration) return e;
+  } else {
+    const cudaError_t e = launch_f64<D>(c, sc, st);
     if (e != cudaErrorInvalidConfiguration) return e;
   }
   const int RB = csr ? 1 : SimtTraits<T>::RB;

@@ -1,0 +1,31 @@
+"""FP64 form against the oracle where its split of the work has edges: several runs per block
+with a ragged last one, odd N D (noise pairs across spins), one or two Philox blocks per
+spin, sparse rows, more values than threads, buffers beyond shared memory."""
+import numpy as np
+import pytest
+
+import oracle.oracle as O
+from paper_2308_02329_gb300 import chym, inputs
+from tests.helpers import make_case, oracle_params, oracle_schedule, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,D,n_h,reps,graph", [
+    (1, 1, 1, 2, "sk"), (7, 1, 2, 200, "sk"), (9, 2, 1, 307, "gauss"), (20, 3, 8, 61, "sk"),
+    (5, 4, 1, 1601, "sk"), (13, 5, 3, 120, "sk"), (40, 6, 2, 90, "gauss"), (33, 7, 1, 155, "sk"),
+    (25, 8, 2, 160, "sk"), (100, 4, 1, 311, "mobius"), (301, 2, 1, 5, "mobius"), (1300, 8, 1, 2, "gauss")])
+def test_state_matches_oracle(N, D, n_h, reps, graph):
+    if graph == "mobius":
+        N += N % 2
+    J, eps, h, seeds = make_case(N, D, n_h, reps, 23, graph)
+    ctx = chym.Context(J, D, chym.J_REAL if graph == "gauss" else chym.J_PM1)
+    prm = chym.Params(eps=eps, prec=chym.PREC_FP64)
+    steps = 12 if N < 1000 else 3
+    sch = chym.Schedule(1, steps // 3, steps - 1)   # ramp and its end inside the run
+    ctx.run(prm, h, seeds, steps, sch)
+    X, k = ctx.get_state()
+    assert k == steps
+    Xo = O.run(J, D, inputs.h_per_run(h, reps), seeds, oracle_params(prm), oracle_schedule(sch), steps)
+    assert rel_err(X, Xo) <= 1e-10   # FP64 mode, as in the other parity tests
+    ctx.close()
