@@ -9,9 +9,10 @@
 //   phase B  x <- x + dt [(h-1) x - kappa x^3 - gamma x |x_p|^2 + eps alpha_mu y]
 //            + sigma sqrt(dt) xi  with xi from Philox4x32-10 + Box-Muller.
 // FP32 runs on the register-tiled kernel (step_simt_tiled_kernel, below), whose
-// threads each own 4 spins x RB runs through both phases; FP64 runs on step_f64_kernel,
-// with the noise drawn ahead by warps of its own; both, where their buffers do not fit, run on
-// the per-spin kernel (step_simt_kernel), whose
+// threads each own 4 spins x RB runs through both phases, or, for a sparse J whose run
+// groups do not fit it, on step_csr_kernel; FP64 runs on step_f64_kernel, with the noise
+// drawn ahead by warps of its own.  A dense FP32 J and FP64 runs whose buffers do not fit
+// these run on the per-spin kernel (step_simt_kernel), whose
 // threads each take one (spin, run group) in phase A and one (spin, run) in phase B,
 // with J staged in shared memory when it fits and read through L1/L2 otherwise.
 #include <algorithm>
@@ -136,7 +137,7 @@ struct CsrRows {
 };
 
 template <typename T, int D, bool J_SMEM, bool CSR>
-__global__ void __launch_bounds__(CSR && sizeof(T) == 4 ? 1024 : 512) step_simt_kernel(const T* __restrict__ Jg,
+__global__ void __launch_bounds__(512) step_simt_kernel(const T* __restrict__ Jg,
                                                         T* __restrict__ Xg,
                                                         const double* __restrict__ hg,
                                                         const uint64_t* __restrict__ seeds,
@@ -605,12 +606,195 @@ cudaError_t launch_simt_tiled(chym_ctx* c, const StepConsts& sc, cudaStream_t st
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// FP32 form over the compressed rows of a large sparse J (a run group does not fit the tiled
+// kernel).  A thread owns its spins for the whole launch, with the first kHeld nonzeros of
+// their rows in registers, and takes every run of the CTA through product, noise and update
+// in one pass; the state is double buffered, one barrier a step.  What depends on the run
+// and step only (the first two Philox rounds as far as they do, round keys, pump, annealing
+// scale) is formed once per run and step and read from shared memory.  (Two passes with the
+// product through shared memory and all of that per spin: ladder N = 2048, D = 3, 2048 runs,
+// 63 us a step.)
+struct __align__(16) CsrRun {
+  uint4 r12[2];  // per Philox block, see csr_rounds12
+  uint4 rk[4];   // keys of rounds 3..10
+  float hm1, ramp;
+};
+// Philox counter (p, blk, k_lo, k_hi), key (k0, k1), k' the round-2 key: what rounds 1 and 2
+// leave that does not depend on p:
+//   x = k_hi ^ k1, y = lo(M1 k_lo) ^ k0', z = hi(M0 c) ^ k1', w = lo(M0 c) with
+//   c = hi(M1 k_lo) ^ blk ^ k0.
+__device__ __forceinline__ uint4 csr_rounds12(uint32_t blk, uint64_t k, uint32_t k0, uint32_t k1) {
+  const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint32_t)k;
+  const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ blk ^ k0);
+  return make_uint4((uint32_t)(k >> 32) ^ k1, (uint32_t)p1 ^ (k0 + kPhiloxW0), (uint32_t)(p0 >> 32) ^ (k1 + kPhiloxW1),
+                    (uint32_t)p0);
+}
+
+template <int D>
+__global__ void __launch_bounds__(D <= 4 ? 1024 : 512) step_csr_kernel(float* __restrict__ Xg,
+                                                                       const double* __restrict__ hg,
+                                                                       const uint64_t* __restrict__ seeds,
+                                                                       StepConsts sc, int RC, CsrRows<float> csr) {
+  constexpr int kHeld = 3, NB = (D + 3) / 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = sc.N, tid = threadIdx.x, nt = blockDim.x;
+  CsrRun* s_run = reinterpret_cast<CsrRun*>(smem_raw);  // 2 RC: by step parity
+  float* Xs = reinterpret_cast<float*>(s_run + 2 * RC);  // 2 x RC x N x D
+  const int run0 = blockIdx.x * RC;
+  const int nr = min(RC, sc.n_runs - run0), used = nr * N * D;
+  const size_t buf = (size_t)RC * N * D;
+  for (int i = tid; i < used; i += nt) Xs[i] = Xg[(size_t)run0 * N * D + i];
+  // run r's constants at step k, by thread r (its keys stay in registers)
+  uint32_t k0 = 0u, k1 = 0u;
+  int64_t koff = 0;
+  float hm1 = 0.f;
+  if (tid < nr) {
+    const uint64_t seed = seeds[run0 + tid];
+    k0 = (uint32_t)seed;
+    k1 = (uint32_t)(seed >> 32);
+    koff = sc.koff[run0 + tid];
+    hm1 = (float)(hg[sc.hidx[run0 + tid]] - 1.0);
+  }
+  const float inv_ramp = sc.sched_kind == 1 ? 1.f / (float)(sc.k_total - sc.k_anneal) : 0.f;
+  auto put_run = [&](int64_t k, bool keys) {
+    if (tid >= nr) return;
+    CsrRun& o = s_run[(k & 1) * RC + tid];
+    const int64_t kl = k - koff;
+#pragma unroll
+    for (int b = 0; b < NB; ++b) o.r12[b] = csr_rounds12((uint32_t)b, (uint64_t)kl, k0, k1);
+    float ramp = 1.f;  // alpha_mu(kl) for mu >= 1
+    if (sc.sched_kind == 1 && kl >= sc.k_anneal) ramp = kl >= sc.k_total ? 0.f : 1.f - (float)(kl - sc.k_anneal) * inv_ramp;
+    o.ramp = ramp;
+    if (keys) {
+      o.hm1 = hm1;
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {  // Weyl key schedule: round j (0-based) uses key + j (W0, W1)
+        const uint32_t j = 2u * i + 2u;
+        o.rk[i] = make_uint4(k0 + j * kPhiloxW0, k1 + j * kPhiloxW1, k0 + (j + 1u) * kPhiloxW0, k1 + (j + 1u) * kPhiloxW1);
+      }
+    }
+  };
+  put_run(sc.k0, true);
+  put_run(sc.k0 + 1, true);
+  __syncthreads();
+  const float dt = (float)sc.dt, gamma = (float)sc.gamma, kappa = (float)sc.kappa, scale = (float)sc.noise_scale;
+  for (int64_t k = sc.k0; k < sc.k0 + sc.steps; ++k) {
+    const float* X = Xs + (size_t)((k - sc.k0) & 1) * buf;
+    float* Xn = Xs + (size_t)((k - sc.k0 + 1) & 1) * buf;
+    const CsrRun* runs = s_run + (k & 1) * RC;
+    for (int p = tid; p < N; p += nt) {
+      const int e0 = __ldg(csr.rp + p), e1 = __ldg(csr.rp + p + 1);
+      float jv[kHeld];
+      int jo[kHeld];
+#pragma unroll
+      for (int t = 0; t < kHeld; ++t) {
+        const bool in = e0 + t < e1;
+        jv[t] = in ? __ldg(csr.cv + e0 + t) : 0.f;
+        jo[t] = in ? __ldg(csr.ci + e0 + t) * D : p * D;
+      }
+      const float ew = (float)sc.eps * (sc.w ? (float)sc.w[p] : 1.f);
+      const uint64_t mp = (uint64_t)kPhiloxM0 * (D <= 2 ? (uint32_t)p / (4u / (D <= 2 ? D : 4)) : (uint32_t)p);
+      for (int r = 0; r < nr; ++r) {
+        const float* xr = X + (size_t)r * N * D;
+        const CsrRun& rc = runs[r];
+        float y[D], x[D], z[4 * NB], n2 = 0.f;
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu) {
+          y[mu] = 0.f;
+#pragma unroll
+          for (int t = 0; t < kHeld; ++t)
+            if (e0 + t < e1) y[mu] = fmaf(jv[t], xr[jo[t] + mu], y[mu]);
+          x[mu] = xr[p * D + mu];
+        }
+        for (int e = e0 + kHeld; e < e1; ++e) {
+          const float j = __ldg(csr.cv + e);
+          const int o = __ldg(csr.ci + e) * D;
+#pragma unroll
+          for (int mu = 0; mu < D; ++mu) y[mu] = fmaf(j, xr[o + mu], y[mu]);
+        }
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu) n2 = fmaf(x[mu], x[mu], n2);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          const uint4 t = rc.r12[b];
+          const uint64_t q = (uint64_t)kPhiloxM1 * ((uint32_t)(mp >> 32) ^ t.x);
+          uint4 c = make_uint4((uint32_t)(q >> 32) ^ t.y, (uint32_t)q, t.z ^ (uint32_t)mp, t.w);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint4 kk = rc.rk[i];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const uint64_t p0 = (uint64_t)kPhiloxM0 * c.x, p1 = (uint64_t)kPhiloxM1 * c.z;
+              c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ (h ? kk.z : kk.x), (uint32_t)p1,
+                             (uint32_t)(p0 >> 32) ^ c.w ^ (h ? kk.w : kk.y), (uint32_t)p0);
+            }
+          }
+          if constexpr (D <= 2) {  // the spin's pair of a block it shares
+            const uint32_t j0 = ((uint32_t)p % (4u / D)) * D;
+            float cz, sz;
+            box_muller_f32(j0 >= 2u ? c.z : c.x, j0 >= 2u ? c.w : c.y, scale, cz, sz);
+            z[0] = (j0 & 1u) ? sz : cz;
+            z[1] = sz;
+          } else {
+            box_muller_f32(c.x, c.y, scale, z[4 * b], z[4 * b + 1]);
+            if (D - 4 * b > 2) box_muller_f32(c.z, c.w, scale, z[4 * b + 2], z[4 * b + 3]);
+          }
+        }
+        float* xo = Xn + (size_t)r * N * D + p * D;
+#pragma unroll
+        for (int mu = 0; mu < D; ++mu) {
+          const float xm = x[mu];
+          const float f = rc.hm1 * xm - kappa * xm * xm * xm - gamma * xm * n2 + ew * (mu == 0 ? 1.f : rc.ramp) * y[mu];
+          xo[mu] = xm + dt * f + z[mu];
+        }
+      }
+    }
+    __syncthreads();
+    put_run(k + 2, false);  // this step's parity: read next after the barrier of step k + 1
+  }
+  const float* X = Xs + (size_t)(sc.steps & 1) * buf;
+  for (int i = tid; i < used; i += nt) Xg[(size_t)run0 * N * D + i] = X[i];
+}
+
+template <int D>
+cudaError_t launch_csr(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
+  const int N = c->N;
+  const size_t per_run = (size_t)2 * N * D * sizeof(float);
+  const int fit = (int)std::min<size_t>(kSimtSmemBudget / per_run, 32);
+  if (fit < 1) return cudaErrorInvalidConfiguration;  // N too large
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  // runs per CTA (one CTA per SM): the fewest run slots over the waves of CTAs, each wave
+  // counted half a run more for its barriers and constants (2048 runs, up to 4 a CTA: 7 waves
+  // of 2 rather than 4 of 4)
+  int RC = 1;
+  double best = 0.0;
+  for (int rc = 1; rc <= fit; ++rc) {
+    const int grid = (sc.n_runs + rc - 1) / rc;
+    const double t = (double)((grid + sms - 1) / sms) * (rc + 0.5);
+    if (rc == 1 || t < best) {
+      best = t;
+      RC = rc;
+    }
+  }
+  const int threads = std::min(D <= 4 ? 1024 : 512, std::max(64, (N + 31) / 32 * 32));
+  const size_t smem = (size_t)RC * (per_run + 2 * sizeof(CsrRun));
+  const CsrRows<float> rows{c->d_rp, c->d_ci, c->d_cv32};
+  auto kern = step_csr_kernel<D>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<(sc.n_runs + RC - 1) / RC, threads, smem, st>>>((float*)c->d_X, c->d_h, c->d_seeds, sc, RC, rows);
+  return cudaGetLastError();
+}
+
 template <typename T, int D>
 cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   const bool csr = c->sparse;  // the SIMT kernels use the compressed rows whenever they exist
   if constexpr (sizeof(T) == 4) {
     const cudaError_t e = csr ? launch_simt_tiled<D, true>(c, sc, st) : launch_simt_tiled<D, false>(c, sc, st);
     if (e != cudaErrorInvalidConfiguration) return e;
+    if (csr) return launch_csr<D>(c, sc, st);
   } else {
     const cudaError_t e = launch_f64<D>(c, sc, st);
     if (e != cudaErrorInvalidConfiguration) return e;
@@ -630,14 +814,14 @@ cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   while (RC > RB && (int64_t)((sc.n_runs + RC - 1) / RC) < sms) RC -= RB;
   const size_t smem = (j_smem ? j_bytes : 0) + (size_t)RC * per_run;
-  // the FP32 compressed-row form needs few registers: twice the warps hide its gathers
-  const int threads = std::min(csr && sizeof(T) == 4 ? 1024 : 512, std::max(64, ((N * (RC / RB) + 31) / 32) * 32));
+  const int threads = std::min(512, std::max(64, ((N * (RC / RB) + 31) / 32) * 32));
   const int grid = (sc.n_runs + RC - 1) / RC;
   const T* J = sizeof(T) == 8 ? (const T*)c->d_J64 : (const T*)c->d_J32;
   T* X = (T*)c->d_X;
   const CsrRows<T> rows{c->d_rp, c->d_ci, sizeof(T) == 8 ? (const T*)c->d_cv64 : (const T*)c->d_cv32};
-  auto kern = csr ? step_simt_kernel<T, D, false, true>
-                  : j_smem ? step_simt_kernel<T, D, true, false> : step_simt_kernel<T, D, false, false>;
+  auto kern = j_smem ? step_simt_kernel<T, D, true, false> : step_simt_kernel<T, D, false, false>;
+  if constexpr (sizeof(T) == 8)
+    if (csr) kern = step_simt_kernel<T, D, false, true>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, threads, smem, st>>>(J, X, c->d_h, c->d_seeds, sc, RC, rows);
