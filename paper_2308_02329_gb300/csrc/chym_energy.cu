@@ -42,6 +42,7 @@ template <typename T, typename Bad>
 __device__ __forceinline__ void read_spins(const T* __restrict__ X, int run0, int nr, int N, int D,
                                            uint64_t (*sw)[kMaxSpinWords], Bad bad) {
   const int words = (N + 63) / 64, lane = threadIdx.x & 31;
+#pragma unroll 2
   for (int t = threadIdx.x >> 5; t < nr * words; t += blockDim.x >> 5) {
     const int r = t / words, w = t % words;
     uint32_t half[2];
@@ -52,7 +53,8 @@ __device__ __forceinline__ void read_spins(const T* __restrict__ X, int run0, in
       if (q < N) {
         const T* x = X + ((size_t)(run0 + r) * N + q) * D;
         up = x[0] >= T(0);
-        for (int mu = 0; mu < D; ++mu) finite = finite && isfinite((double)x[mu]);
+#pragma unroll 4
+        for (int mu = 0; mu < D; ++mu) finite &= isfinite(x[mu]) != 0;  // no short cut: independent loads
       }
       if (!finite) bad(r, q);
       half[i] = __ballot_sync(0xffffffffu, up);
@@ -70,7 +72,11 @@ __device__ __forceinline__ void read_spins(const T* __restrict__ X, int run0, in
 // With d_p = the spins that differ from s_p (one xor of the spin words),
 //   sum_q J_pq s_p s_q = deg_p - 2 (popc(Jpos_p & d_p) - popc(Jneg_p & d_p)),
 // deg_p = (#J = +1) - (#J = -1) in row p: an exact integer from N/64 words a row.
-template <typename T, int RB>
+//
+// kSplit: block (x, y) takes the y-th share of the rows and adds its part to E (zeroed
+// before; integers, so the order does not matter): a few dozen runs of a large N would
+// otherwise leave most SMs idle (64 runs, N = 1000: 42 us).
+template <typename T, int RB, bool kSplit>
 __global__ void __launch_bounds__(kEnergyThreads) energy_pm1_kernel(
     const T* __restrict__ X, int N, int D, int n_runs, const uint64_t* __restrict__ Jpos,
     const uint64_t* __restrict__ Jneg, const int32_t* __restrict__ deg, double* __restrict__ E,
@@ -82,12 +88,14 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_pm1_kernel(
   if (tid < RB) bad[tid] = sum[tid] = 0;
   __syncthreads();
   read_spins<T>(X, run0, nr, N, D, sw, [&](int r, int) { bad[r] = 1; });
-  if (spins)
+  if (spins && (!kSplit || blockIdx.y == 0))
     for (int t = tid; t < nr * words; t += blockDim.x) spins[(size_t)run0 * words + t] = sw[t / words][t % words];
   int acc[RB];  // at most N^2 <= 2^24 in magnitude
 #pragma unroll
   for (int r = 0; r < RB; ++r) acc[r] = 0;
-  for (int p = tid; p < N; p += blockDim.x) {
+  const int p_begin = kSplit ? (int)((long long)N * blockIdx.y / gridDim.y) : 0;
+  const int p_end = kSplit ? (int)((long long)N * (blockIdx.y + 1) / gridDim.y) : N;
+  for (int p = p_begin + tid; p < p_end; p += blockDim.x) {
     uint64_t flip[RB];  // d = spins unlike s_p (padding bits meet no J)
     int c[RB];
 #pragma unroll
@@ -113,7 +121,10 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_pm1_kernel(
     if ((tid & 31) == 0) atomicAdd(&sum[r], t);
   }
   __syncthreads();
-  if (tid < nr) E[run0 + tid] = bad[tid] ? (double)NAN : -(double)sum[tid];
+  if (tid >= nr) return;
+  const double part = bad[tid] ? (double)NAN : -(double)sum[tid];
+  if (kSplit) atomicAdd(E + run0 + tid, part);
+  else E[run0 + tid] = part;
 }
 
 // Real J in fixed point on the tensor cores.  Row p of J times 2^e_p is rounded to integers,
@@ -451,11 +462,20 @@ cudaError_t launch_energy_typed(chym_ctx* c, double* d_E, uint64_t* d_spins, cud
   const int W = (N + 63) / 64;
   if (c->kind == CHYM_J_PM1) {
     const uint64_t *jp = c->d_Jbits, *jn = c->d_Jbits + (size_t)W * N;
-    if (many_runs(c, kEnergyRuns))
-      energy_pm1_kernel<T, kEnergyRuns><<<(R + kEnergyRuns - 1) / kEnergyRuns, energy_threads(N), 0, st>>>(
+    const int groups = (R + kEnergyRuns - 1) / kEnergyRuns;
+    if (many_runs(c, kEnergyRuns)) {
+      energy_pm1_kernel<T, kEnergyRuns, false>
+          <<<groups, energy_threads(N), 0, st>>>(X, N, c->D, R, jp, jn, c->d_jdeg, d_E, d_spins);
+    } else if (N >= 2 * kEnergyThreads) {
+      // shares of at least one row a thread, up to four blocks per SM
+      const int shares = std::max(1, std::min(N / kEnergyThreads, 4 * 152 / R));
+      cudaError_t e = cudaMemsetAsync(d_E, 0, sizeof(double) * (size_t)R, st);
+      if (e != cudaSuccess) return e;
+      energy_pm1_kernel<T, 1, true><<<dim3((unsigned)R, (unsigned)shares), kEnergyThreads, 0, st>>>(
           X, N, c->D, R, jp, jn, c->d_jdeg, d_E, d_spins);
-    else
-      energy_pm1_kernel<T, 1><<<R, energy_threads(N), 0, st>>>(X, N, c->D, R, jp, jn, c->d_jdeg, d_E, d_spins);
+    } else {
+      energy_pm1_kernel<T, 1, false><<<R, energy_threads(N), 0, st>>>(X, N, c->D, R, jp, jn, c->d_jdeg, d_E, d_spins);
+    }
   } else if (many_runs(c, 8 * kEnergyRealTiles)) {
     energy_real_kernel<T, kEnergyRealTiles>
         <<<(R + 8 * kEnergyRealTiles - 1) / (8 * kEnergyRealTiles), kEnergyThreads, 0, st>>>(

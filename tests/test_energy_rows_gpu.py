@@ -76,3 +76,19 @@ def test_segment_energies_match_numpy(kind, N, D, R, cuts):
         tol = 0.0 if kind == "pm1" else 4 * (b - a) * 2.0 ** -53 * np.abs(J[a:b, a:b]).sum()
         assert np.max(np.abs(E[ok, i] - want[ok]), initial=0.0) <= tol
     ctx.close()
+
+
+@pytest.mark.parametrize("N,R,prec", [(511, 9, chym.PREC_FP32), (512, 1, chym.PREC_FP64), (513, 65, chym.PREC_FP32),
+                                      (1500, 64, chym.PREC_FP8), (777, 1215, chym.PREC_FP32)])
+def test_rows_shared_between_blocks(N, R, prec):
+    """Few runs of a large +-1 J: the rows of a run are split over several blocks."""
+    J = inputs.sk_pm1(N, 5)
+    ctx = chym.Context(J, 2, chym.J_PM1)
+    X = _state(ctx, N, 2, R, prec, 13)
+    E, S = ctx.energy(spins=True)
+    s = np.where(X[..., 0] >= 0, 1.0, -1.0)
+    ok = np.isfinite(X).all(axis=(1, 2))
+    assert np.array_equal(np.isfinite(E), ok)
+    assert np.array_equal(chym.unpack_spins(S, N)[ok], s[ok])
+    assert np.array_equal(E[ok], _field_energy(J, s)[ok])
+    ctx.close()
