@@ -106,9 +106,8 @@ __device__ __forceinline__ uint4 philox_rounds(uint4 c, const uint4* rk) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const uint32_t k0 = h ? kk.z : kk.x, k1 = h ? kk.w : kk.y;
-      const uint32_t lo0 = kPhiloxM0 * c.x, hi0 = __umulhi(kPhiloxM0, c.x);
-      const uint32_t lo1 = kPhiloxM1 * c.z, hi1 = __umulhi(kPhiloxM1, c.z);
-      c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+      const uint64_t p0 = (uint64_t)kPhiloxM0 * c.x, p1 = (uint64_t)kPhiloxM1 * c.z;
+      c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1, (uint32_t)p0);
     }
   }
   return c;
@@ -374,12 +373,15 @@ cudaError_t launch_f64(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
 // coupling product never leaves registers, and its noise follows the counter layout of
 // the other kernels; a tile of four spins holds whole Philox blocks for D <= 2.
 // (J in shared memory instead of L1 measured slower: it leaves fewer CTAs per SM.)
-template <int D, bool CSR>
+// RB shrinks (by SH halvings) while the threads would not fill the SMs: the work per thread is
+// a long chain, and 4096 runs of N = 100, D = 4 at RB = 4 left 5 warps on an SM.
+template <int D, int SH>
 struct TileCfg {
   static constexpr int DP = D == 3 ? 4 : (D > 4 ? 8 : D);
-  static constexpr int RB = D == 1 ? 8 : D <= 4 ? 4 : 2;
+  static constexpr int RB = (D == 1 ? 8 : D <= 4 ? 4 : 2) >> SH;
   static_assert(RB * DP <= 2 || (RB * DP) % 4 == 0, "state loads are 4, 8 or 16k bytes");
 };
+constexpr int tile_halvings(int D) { return D <= 4 ? 2 : 1; }
 
 // The n = RB DP consecutive state values of one spin and run group (n = 1, 2 or 4k).
 template <int n>
@@ -402,14 +404,14 @@ __device__ __forceinline__ void load_x(const float* src, float (&xv)[n]) {
   }
 }
 
-template <int D, bool CSR>
+template <int D, bool CSR, int SH>
 __global__ void __launch_bounds__(512) step_simt_tiled_kernel(const float* __restrict__ Jp,
                                                               float* __restrict__ Xg,
                                                               const double* __restrict__ hg,
                                                               const uint64_t* __restrict__ seeds,
                                                               StepConsts sc, int RC, int NP,
                                                               CsrRows<float> csr) {
-  using Cfg = TileCfg<D, CSR>;
+  using Cfg = TileCfg<D, SH>;
   constexpr int DP = Cfg::DP, RB = Cfg::RB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = sc.N;
@@ -574,36 +576,47 @@ __global__ void __launch_bounds__(512) step_simt_tiled_kernel(const float* __res
   }
 }
 
-// Launch of the tiled FP32 form; InvalidConfiguration when a run group does not fit its
-// shared memory (the caller then takes the per-spin kernel).
-template <int D, bool CSR>
-cudaError_t launch_simt_tiled(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
-  using Cfg = TileCfg<D, CSR>;
-  const int N = c->N, NP = c->j32p_ld;
-  const bool csr = CSR;
-  if (!csr && (!c->d_J32p || NP < N)) return cudaErrorInvalidConfiguration;
-  const size_t per_run = (size_t)NP * Cfg::DP * sizeof(float) + 5 * sizeof(uint4) + sizeof(int64_t) + sizeof(float);
-  if (Cfg::RB * per_run > kSimtSmemBudget) return cudaErrorInvalidConfiguration;
-  // sparse J with long rows of state (N of about 1000 and more): the per-spin kernel,
-  // whose 1024-thread CTAs measured faster there than CTAs of a few run groups
-  if (CSR && kSimtSmemBudget / per_run < (size_t)(4 * Cfg::RB)) return cudaErrorInvalidConfiguration;
-  int RC = (int)std::min<size_t>(kSimtSmemBudget / per_run, 512);
-  RC = RC / Cfg::RB * Cfg::RB;
-  // at most 512 threads, and no larger CTAs than it takes to fill the GPU
-  while (RC > Cfg::RB && (NP / 4) * (RC / Cfg::RB) > 512) RC -= Cfg::RB;
-  if ((NP / 4) * (RC / Cfg::RB) > 512) return cudaErrorInvalidConfiguration;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  while (RC > Cfg::RB && (int64_t)((sc.n_runs + RC - 1) / RC) < sms) RC -= Cfg::RB;
-  const int threads = std::max(32, ((NP / 4) * (RC / Cfg::RB) + 31) / 32 * 32);
+template <int D, bool CSR, int SH>
+cudaError_t launch_simt_tiles(chym_ctx* c, const StepConsts& sc, int sms, size_t per_run, cudaStream_t st) {
+  constexpr int RB = TileCfg<D, SH>::RB;
+  const int NP = c->j32p_ld, tiles = NP / 4;
+  // Fewer threads than kTileWarps warps an SM: halve the runs per thread.
+  constexpr int kTileWarps = 10;
+  if constexpr (SH < tile_halvings(D))
+    if ((long long)tiles * ((sc.n_runs + RB - 1) / RB) < (long long)sms * 32 * kTileWarps)
+      return launch_simt_tiles<D, CSR, SH + 1>(c, sc, sms, per_run, st);
+  int RC = (int)std::min<size_t>(kSimtSmemBudget / per_run, (size_t)std::max(1, 512 / tiles) * RB);
+  RC = RC / RB * RB;
+  if (RC < RB || tiles * (RC / RB) > 512) return cudaErrorInvalidConfiguration;
+  // CTAs of equal size: the runs of an SM over as few of them as that takes
+  const int share = (sc.n_runs + sms - 1) / sms, per_sm = (share + RC - 1) / RC;
+  RC = std::min(RC, ((share + per_sm - 1) / per_sm + RB - 1) / RB * RB);
+  const int threads = std::max(32, (tiles * (RC / RB) + 31) / 32 * 32);
   const size_t smem = (size_t)RC * per_run;
   const int grid = (sc.n_runs + RC - 1) / RC;
   const CsrRows<float> rows{c->d_rp, c->d_ci, c->d_cv32};
-  auto kern = step_simt_tiled_kernel<D, CSR>;
+  auto kern = step_simt_tiled_kernel<D, CSR, SH>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, threads, smem, st>>>(c->d_J32p, (float*)c->d_X, c->d_h, c->d_seeds, sc, RC, NP, rows);
   return cudaGetLastError();
+}
+
+// Launch of the tiled FP32 form; InvalidConfiguration when a run group does not fit its
+// shared memory (the caller then takes another kernel).
+template <int D, bool CSR>
+cudaError_t launch_simt_tiled(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
+  using Cfg = TileCfg<D, 0>;
+  const int N = c->N, NP = c->j32p_ld;
+  if (!CSR && (!c->d_J32p || NP < N)) return cudaErrorInvalidConfiguration;
+  const size_t per_run = (size_t)NP * Cfg::DP * sizeof(float) + 5 * sizeof(uint4) + sizeof(int64_t) + sizeof(float);
+  if (Cfg::RB * per_run > kSimtSmemBudget || NP / 4 > 512) return cudaErrorInvalidConfiguration;
+  // sparse J with long rows of state (N of about 1000 and more): the compressed-row kernel,
+  // whose 1024-thread CTAs measured faster there than CTAs of a few run groups
+  if (CSR && kSimtSmemBudget / per_run < (size_t)(4 * Cfg::RB)) return cudaErrorInvalidConfiguration;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  return launch_simt_tiles<D, CSR, 0>(c, sc, sms, per_run, st);
 }
 
 // ---------------------------------------------------------------------------
