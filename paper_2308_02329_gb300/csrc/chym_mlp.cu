@@ -10,7 +10,7 @@
 //                     snapshot (exact integers for +-1 couplings), extra-dimension
 //                     weight, sign flips, hyperspin energy (Eq. 3), norms;
 //   mlp_forward       one warp per sample, weights (BF16-rounded) in shared memory;
-//   mlp_grad          4 warps per CTA, per-warp gradient buffers in shared memory,
+//   mlp_grad          7 warps per CTA, per-warp gradient buffers in shared memory,
 //                     per-CTA partial gradients reduced by mlp_adam in a fixed order;
 //   mlp_adam          reduction of the partials, Adam on the FP32 master weights,
 //                     refresh of the BF16 copy used by the forward pass.
@@ -31,7 +31,9 @@ namespace {
 constexpr int kF = 24, kH = 64;
 constexpr int oW1 = 0, oB1 = kH * kF, oW2 = oB1 + kH, oB2 = oW2 + kH * kH, oW3 = oB2 + kH,
               oB3 = oW3 + kH, kP = oB3 + 1;  // 5825 parameters
-constexpr int kGradWarps = 4, kGradSamplesPerCta = 64;
+// 7 warps' gradient buffers fill a CTA's shared memory, 7 samples a warp: 4096 samples on 86 SMs
+// (on 64 with 4 warps of 16 samples they took 70 us)
+constexpr int kGradWarps = 7, kGradSamplesPerCta = 48;
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
@@ -60,9 +62,11 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(
     const T* __restrict__ X, const T* __restrict__ Xs, int N, int D, int P2,
     const int8_t* __restrict__ J8, const double* __restrict__ J64, const double* __restrict__ h,
     const int32_t* __restrict__ hidx, float k_frac, float* __restrict__ F) {
-  extern __shared__ float sm[];
-  float* buf = sm;                         // P2 floats: sort buffer, then sigma_mu
-  float* inv = buf + P2;                   // N floats: 1/|x_p|
+  extern __shared__ __align__(16) float sm[];
+  constexpr int kG = 4;                    // components per pass over the couplings
+  float* buf = sm;                         // P2 floats: sort buffer
+  float* sig = sm;                         // then N x kG floats: sigma of a pass
+  float* inv = sm + max(P2, kG * N);       // N floats: 1/|x_p|
   int8_t* s = reinterpret_cast<int8_t*>(inv + N);
   int8_t* ss = s + N;
   __shared__ float red_f[32];
@@ -126,52 +130,72 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(
 #pragma unroll
   for (int j = 0; j < 12; ++j) q12[j] = buf[(int)floorf(j * (N - 1) / 11.0f + 0.5f)];
   __syncthreads();
-  // Ising energies of the signs now and at the snapshot: E = -sum_p s_p sum_q J_pq s_q
+  // Ising energies of the signs now and at the snapshot, E = -sum_p s_p sum_q J_pq s_q, and the
+  // hyperspin energy (Eq. 3), -sum_mu sum_p sigma_p,mu sum_q J_pq sigma_q,mu, with one pass
+  // over the couplings for up to kG components (one pass each, and int8 sums for the signs:
+  // N = 100, D = 3, 4096 runs 121 us)
   double E = 0.0, Es = 0.0;
-  if (PM1) {
-    long long a = 0, b = 0;
-    for (int p = tid; p < N; p += blockDim.x) {
-      int f = 0, fs = 0;
-      for (int q = 0; q < N; ++q) {
-        const int j = J8[(size_t)q * N + p];
-        f += j * s[q];
-        fs += j * ss[q];
-      }
-      a += (long long)s[p] * f;
-      b += (long long)ss[p] * fs;
-    }
-    E = -(double)block_sum<long long>(a, red_i);
-    Es = -(double)block_sum<long long>(b, red_i);
-  } else {
-    double a = 0.0, b = 0.0;
-    for (int p = tid; p < N; p += blockDim.x) {
-      double f = 0.0, fs = 0.0;
-      for (int q = 0; q < N; ++q) {
-        const double j = J64[(size_t)q * N + p];
-        f += j * s[q];
-        fs += j * ss[q];
-      }
-      a += s[p] * f;
-      b += ss[p] * fs;
-    }
-    E = -block_sum<double>(a, red_d);
-    Es = -block_sum<double>(b, red_d);
-  }
-  // hyperspin energy (Eq. 3): -sum_mu sum_p sigma_p,mu sum_q J_pq sigma_q,mu
   float ehs = 0.f;
-  for (int mu = 0; mu < D; ++mu) {
+  long long ea = 0, eb = 0;
+  double da = 0.0, db = 0.0;
+  for (int m0 = 0; m0 < D; m0 += kG) {
+    const int mg = min(kG, D - m0);
     __syncthreads();
-    for (int q = tid; q < N; q += blockDim.x) buf[q] = (float)x[(size_t)q * D + mu] * inv[q];
+    for (int e = tid; e < N * kG; e += blockDim.x) {
+      const int q = e / kG, m = e % kG;
+      sig[e] = m < mg ? (float)x[(size_t)q * D + m0 + m] * inv[q] : 0.f;
+    }
     __syncthreads();
     for (int p = tid; p < N; p += blockDim.x) {
-      float f = 0.f;
-      if (PM1)
-        for (int q = 0; q < N; ++q) f += (float)J8[(size_t)q * N + p] * buf[q];
-      else
-        for (int q = 0; q < N; ++q) f += (float)J64[(size_t)q * N + p] * buf[q];
-      ehs += buf[p] * f;
+      float f[kG];
+#pragma unroll
+      for (int m = 0; m < kG; ++m) f[m] = 0.f;
+      if (PM1) {
+        int fi = 0, fs = 0;
+#pragma unroll 4
+        for (int q = 0; q < N; ++q) {
+          const int j = J8[(size_t)q * N + p];
+          const float4 v = reinterpret_cast<const float4*>(sig)[q];
+          const float jf = (float)j;
+          f[0] += jf * v.x;
+          f[1] += jf * v.y;
+          f[2] += jf * v.z;
+          f[3] += jf * v.w;
+          if (m0 == 0) {
+            fi += j * s[q];
+            fs += j * ss[q];
+          }
+        }
+        if (m0 == 0) {
+          ea += (long long)s[p] * fi;
+          eb += (long long)ss[p] * fs;
+        }
+      } else {
+        double fi = 0.0, fs = 0.0;
+        for (int q = 0; q < N; ++q) {
+          const double j = J64[(size_t)q * N + p];
+          const float4 v = reinterpret_cast<const float4*>(sig)[q];
+          const float jf = (float)j;
+          f[0] += jf * v.x;
+          f[1] += jf * v.y;
+          f[2] += jf * v.z;
+          f[3] += jf * v.w;
+          if (m0 == 0) {
+            fi += j * s[q];
+            fs += j * ss[q];
+          }
+        }
+        if (m0 == 0) {
+          da += s[p] * fi;
+          db += ss[p] * fs;
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < kG; ++m) ehs += sig[(size_t)p * kG + m] * f[m];
     }
   }
+  E = PM1 ? -(double)block_sum<long long>(ea, red_i) : -block_sum<double>(da, red_d);
+  Es = PM1 ? -(double)block_sum<long long>(eb, red_i) : -block_sum<double>(db, red_d);
   ehs = -block_sum<float>(ehs, red_f);
   if (tid == 0) {
     float* o = F + (size_t)run * kF;
@@ -401,18 +425,19 @@ template <typename T>
 cudaError_t launch_features_typed(chym_ctx* c, const void* snap, double k_frac, float* F, cudaStream_t st) {
   int P2 = 1;
   while (P2 < c->N) P2 <<= 1;
-  const size_t smem = sizeof(float) * ((size_t)P2 + c->N) + 2 * (size_t)c->N + 16;
+  const size_t smem = sizeof(float) * ((size_t)std::max(P2, 4 * c->N) + c->N) + 2 * (size_t)c->N + 16;
+  const int threads = c->N <= 128 ? 128 : kFeatThreads;
   if (c->kind == CHYM_J_PM1) {
     auto kern = features_kernel<T, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<c->n_runs, kFeatThreads, smem, st>>>((const T*)c->d_X, (const T*)snap, c->N, c->D, P2,
+    kern<<<c->n_runs, threads, smem, st>>>((const T*)c->d_X, (const T*)snap, c->N, c->D, P2,
                                                 c->d_J8, c->d_J64, c->d_h, c->d_hidx, (float)k_frac, F);
   } else {
     auto kern = features_kernel<T, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<c->n_runs, kFeatThreads, smem, st>>>((const T*)c->d_X, (const T*)snap, c->N, c->D, P2,
+    kern<<<c->n_runs, threads, smem, st>>>((const T*)c->d_X, (const T*)snap, c->N, c->D, P2,
                                                 c->d_J8, c->d_J64, c->d_h, c->d_hidx, (float)k_frac, F);
   }
   return cudaGetLastError();
@@ -638,7 +663,7 @@ CHYM_API chym_status chym_mlp_forward_device(chym_mlp* n, const float* d_F, int 
   if (B == 0) return CHYM_OK;
   const size_t smem = sizeof(SmemNet) + 8 * sizeof(WarpAct);
   CHYM_CUDA_TRY(cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int grid = std::min((B + 7) / 8, 152 * 4);
+  const int grid = std::min((B + 7) / 8, 152);  // every CTA stages the network first
   mlp_forward_kernel<<<grid, 256, smem, (cudaStream_t)stream>>>(view(n), d_F, B, d_logits);
   CHYM_CUDA_TRY(cudaGetLastError());
   return CHYM_OK;
