@@ -93,6 +93,7 @@ static_assert(128 * kHelperRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * kLaunc
 constexpr int kAccCols = 256;                  // TMEM columns of one accumulator
 constexpr size_t kRingBudget = 192 * 1024;     // shared memory for the stage ring
 constexpr int kLaunchSteps = 1024;             // most steps of one launch
+constexpr int kMaxGridY = 65535;
 constexpr int kPhaseTiles = 2;                 // tiles per CTA of a phase (at least)
 constexpr int kPhaseSteps = 32;                // fewest steps of a call that is split into phases
 constexpr uint32_t kA8Block = 128 * kKc;       // bytes of an e4m3 A block (4 KB)
@@ -916,7 +917,6 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           ok = mbar_wait(smem_addr(&stored), it & 1u, L.wait_ns) && !s_abort;
           if (!ok) break;
           fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
-          __threadfence();
           asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
         }
         if (!ok) give_up();
@@ -962,50 +962,51 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
   }
 }
 
-// X[run][p][mu] (float) -> Xm[c][p] and the hi/lo blocks of buffer 0 (the
-// buffer is zeroed beforehand, so padding spins and runs stay zero).
-__global__ void k2_pack_kernel(const float* __restrict__ X, float* __restrict__ Xm,
-                               uint8_t* __restrict__ Xt, int N, int D, int KP, int KC, int CT,
-                               int RT, int n_runs, int lo8) {
-  const int n = D * RT;
+// X[run][p][mu] (float) -> Xm[c][p] and the hi/lo blocks of buffer 0, padding spins and runs
+// (up to the column tiles' last) included; buffer 1 is written whole by the first step.
+// Thread = (spin, component) of one unit of 8 runs, unit0 + blockIdx.y: coalesced reads, one
+// 16-byte row of each block.  (Per element, with 2-byte stores after a memset of both
+// buffers: 201 us for 8192 runs of N = 1000, D = 4.)
+template <int D>
+__global__ void __launch_bounds__(256) k2_pack_kernel(const float* __restrict__ X, float* __restrict__ Xm,
+                                                      uint8_t* __restrict__ Xt, int N, int KP, int KC, int CT, int RT,
+                                                      int n_runs, int lo8, int unit0) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= KP * D) return;
+  const int p = e / D, mu = e % D, run0 = (unit0 + blockIdx.y) * kUnit;
+  const int n = D * RT, ct = run0 / RT, col = mu * RT + run0 % RT;
   const size_t BB = b_block_bytes(n), BL = b_lo_bytes(n, lo8);
-  const size_t lo_off = (size_t)CT * KC * BB;
-  const size_t total = (size_t)n_runs * D * KP;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const int p = (int)(e % KP);
-    const size_t c = e / KP;
-    const int run = (int)(c / D), mu = (int)(c % D);
-    const float v = p < N ? X[((size_t)run * N + p) * D + mu] : 0.f;
-    Xm[c * KP + p] = v;
-    const int ct = run / RT, cl = mu * RT + run % RT;
-    const size_t row_in = (size_t)((p % kKc) >> 3) * kCoreK + (size_t)(p & 7) * 16;
-    const size_t off = ((size_t)ct * KC + p / kKc) * BB + (size_t)(cl >> 3) * kCoreMN + row_in + (size_t)(cl & 7) * 2;
-    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-    const float hf = __bfloat162float(hi);
-    if (lo8) {  // both halves scaled by 2^kLoScaleLog2, lo in e4m3 (see store_hilo8)
-      constexpr float S = (float)(1u << kLoScaleLog2);
-      *reinterpret_cast<__nv_bfloat16*>(Xt + off) = __float2bfloat16_rn(hf * S);
-      const size_t off8 = ((size_t)ct * KC + p / kKc) * BL + (size_t)(cl >> 4) * kCoreMN + row_in + (size_t)(cl & 15);
-      Xt[lo_off + off8] = (uint8_t)__nv_cvt_float_to_fp8((v - hf) * S, __NV_SATFINITE, __NV_E4M3);
-    } else {
-      *reinterpret_cast<__nv_bfloat16*>(Xt + off) = hi;
-      *reinterpret_cast<__nv_bfloat16*>(Xt + lo_off + off) = __float2bfloat16_rn(v - hf);
-    }
+  float v[kUnit];
+#pragma unroll
+  for (int j = 0; j < kUnit; ++j) {
+    v[j] = p < N && run0 + j < n_runs ? X[((size_t)(run0 + j) * N) * D + e] : 0.f;
+    if (run0 + j < n_runs) Xm[((size_t)(run0 + j) * D + mu) * KP + p] = v[j];
   }
+  const size_t row_in = (size_t)((p % kKc) >> 3) * kCoreK + (size_t)(p & 7) * 16, blk = (size_t)ct * KC + p / kKc;
+  uint8_t* hi = Xt + blk * BB + (size_t)(col >> 3) * kCoreMN + row_in;
+  uint8_t* lo = Xt + (size_t)CT * KC * BB + blk * BL + row_in;
+  const float (&v0)[kPiece] = *reinterpret_cast<const float (*)[kPiece]>(v);
+  const float (&v1)[kPiece] = *reinterpret_cast<const float (*)[kPiece]>(v + kPiece);
+  uint32_t h0[2], l0[2], h1[2], l1[2];
+  if (lo8) {  // both halves scaled by 2^kLoScaleLog2, lo in e4m3
+    split_piece8<kPiece>(v0, h0, l0);
+    split_piece8<kPiece>(v1, h1, l1);
+    *reinterpret_cast<uint2*>(lo + (size_t)(col >> 4) * kCoreMN + (size_t)(col & 15)) = make_uint2(l0[0], l1[0]);
+  } else {
+    split_piece<kPiece>(v0, h0, l0);
+    split_piece<kPiece>(v1, h1, l1);
+    *reinterpret_cast<uint4*>(lo + (size_t)(col >> 3) * kCoreMN) = make_uint4(l0[0], l0[1], l1[0], l1[1]);
+  }
+  *reinterpret_cast<uint4*>(hi) = make_uint4(h0[0], h0[1], h1[0], h1[1]);
 }
 
-__global__ void k2_unpack_kernel(const float* __restrict__ Xm, float* __restrict__ X, int N, int D,
-                                 int KP, int n_runs) {
-  const size_t total = (size_t)n_runs * N * D;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const int mu = (int)(e % D);
-    const size_t rp = e / D;
-    const int p = (int)(rp % N);
-    const size_t run = rp / N;
-    X[e] = Xm[(run * D + mu) * KP + p];
-  }
+// Xm[c][p] -> X[run][p][mu]; blockIdx.y = run.
+template <int D>
+__global__ void __launch_bounds__(256) k2_unpack_kernel(const float* __restrict__ Xm, float* __restrict__ X, int N,
+                                                        int KP) {
+  const size_t run = blockIdx.y;
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e < N * D) X[run * N * D + e] = Xm[(run * D + e % D) * KP + e / D];
 }
 
 // per-run constant 1 + dt (h - 1)
@@ -1051,12 +1052,13 @@ int k2_rt(int D, int n_runs, int want = 0) {
 }
 
 // Time of a tile in the planner's units (ns): the ring's feed against the epilogue, which
-// overlap.  95 bytes a ns of feed and 42 ns per run and component (two passes of the eight
-// warps over 128 spins) were measured with one side of the tile loop emptied (N = 800,
-// D = 4, FP8 mode); the constant is the hand-over between them.
+// overlap.  95 bytes a ns of feed were measured with the epilogue emptied, and per run and D
+// the epilogue's share of full steps (N = 1000; D = 2 costs as much noise as D = 4, its blocks
+// serving two spins); the constant is the hand-over between them.
 double k2_tile_ns(int N, int D, int RT, int a_terms, int lo8) {
+  constexpr double run_ns[9] = {0, 150, 160, 240, 250, 400, 450, 560, 620};
   const int KC = (N + 127) / 128 * 128 / kKc;
-  const double feed = KC * (double)stage_bytes(D * RT, a_terms, lo8) / 95.0, epi = 42.0 * D * RT;
+  const double feed = KC * (double)stage_bytes(D * RT, a_terms, lo8) / 95.0, epi = run_ns[D] * RT;
   return std::max(feed, epi) + 0.3 * std::min(feed, epi) + 1000.0;
 }
 
@@ -1133,6 +1135,21 @@ cudaError_t prepare_k2_operand(chym_ctx* c) {
 // ---------------------------------------------------------------------------
 // Runner: a set of large-N contexts integrated together for `steps` steps.
 // ---------------------------------------------------------------------------
+// f(std::integral_constant<int, D>()) for the D of a context.
+template <typename F>
+void with_dim(int D, F f) {
+  switch (D) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 7: f(std::integral_constant<int, 7>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+  }
+}
+
 // Workspace, per-run constants and buffer 0 of one context; fills its descriptor.
 cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void* desc_out, int RT) {
   cudaError_t e = prepare_k2_operand(c);
@@ -1160,11 +1177,15 @@ cudaError_t k2_prepare(chym_ctx* c, const StepConsts& sc, cudaStream_t st, void*
   float* Xm = (float*)ws;
   uint8_t* Xt = ws + xm_bytes;
   float* ar = (float*)(Xt + xt_bytes);
-  e = cudaMemsetAsync(Xt, 0, xt_bytes, st);
-  if (e != cudaSuccess) return e;
   k2_runconst_kernel<<<(sc.n_runs + 255) / 256, 256, 0, st>>>(c->d_h, c->d_hidx, sc.n_runs, sc.dt, ar);
-  k2_pack_kernel<<<152 * 8, 256, 0, st>>>((const float*)c->d_X, Xm, Xt, N, D, KP, KC, CT, RT,
-                                           sc.n_runs, lo8);
+  with_dim(D, [&](auto dim) {
+    constexpr int kD = decltype(dim)::value;
+    const int units = CT * RT / kUnit;
+    for (int u0 = 0; u0 < units; u0 += kMaxGridY) {
+      const dim3 grid((unsigned)((KP * kD + 255) / 256), (unsigned)std::min(kMaxGridY, units - u0));
+      k2_pack_kernel<kD><<<grid, 256, 0, st>>>((const float*)c->d_X, Xm, Xt, N, KP, KC, CT, RT, sc.n_runs, lo8, u0);
+    }
+  });
   d.D = D;
   d.flag0 = 0;  // set by k2_integrate
   d.Aimg = (const uint8_t*)c->d_Ak2;
@@ -1202,7 +1223,14 @@ size_t k2_desc_bytes() { return sizeof(K2Desc); }
 
 cudaError_t k2_finish(chym_ctx* c, const void* desc, cudaStream_t st) {
   const K2Desc& d = *reinterpret_cast<const K2Desc*>(desc);
-  k2_unpack_kernel<<<152 * 8, 256, 0, st>>>(d.Xm, (float*)c->d_X, c->N, c->D, d.KP, d.n_runs);
+  with_dim(c->D, [&](auto dim) {
+    constexpr int kD = decltype(dim)::value;
+    for (int r0 = 0; r0 < d.n_runs; r0 += kMaxGridY) {
+      const dim3 grid((unsigned)((c->N * kD + 255) / 256), (unsigned)std::min(kMaxGridY, d.n_runs - r0));
+      k2_unpack_kernel<kD><<<grid, 256, 0, st>>>(d.Xm + (size_t)r0 * kD * d.KP,
+                                                 (float*)c->d_X + (size_t)r0 * c->N * kD, c->N, d.KP);
+    }
+  });
   return cudaGetLastError();
 }
 
