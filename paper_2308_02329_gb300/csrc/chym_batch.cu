@@ -145,11 +145,14 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
   // work in SM-microseconds per step: the small-N dimensions and the large-N group.  The SMs
   // are split in proportion, so that all parts finish together; the large-N launches take the
   // SMs that the persistent small-N CTAs leave free.
-  long long runs_of[9] = {0};
+  long long runs_of[9] = {0}, chunks_of[9] = {0};  // runs, and chunks of the smallest size (4 runs)
   double small_total = 0.0, total = 0.0;
   int dims = 0;
   for (int D = 1; D <= 8; ++D) {
-    for (int i : by_dim[D]) runs_of[D] += b->ctxs[i]->n_runs;
+    for (int i : by_dim[D]) {
+      runs_of[D] += b->ctxs[i]->n_runs;
+      chunks_of[D] += (b->ctxs[i]->n_runs + 3) / 4;
+    }
     if (runs_of[D]) small_total += b->chunk_cost[D] * (double)runs_of[D] / tc_chunk_runs(D);
     dims += runs_of[D] ? 1 : 0;
   }
@@ -171,13 +174,14 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     int next = 0;
     double longest = -1.0;
     for (int D = 1; D <= 8; ++D) {
-      if (!runs_of[D]) continue;
+      if (ctas_of[D] >= chunks_of[D]) continue;  // a chunk each: more SMs cannot help
       const double t = ctas_of[D] ? b->chunk_cost[D] * tc_step_chunks(D, runs_of[D], ctas_of[D]) : INFINITY;
       if (t > longest) {
         longest = t;
         next = D;
       }
     }
+    if (next == 0) break;
     ++ctas_of[next];
   }
   // plan: descriptors of all small-N contexts, then per dimension its items and CTA ranges
