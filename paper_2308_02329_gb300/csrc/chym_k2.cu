@@ -409,17 +409,19 @@ __device__ __forceinline__ void split_piece(const float (&v)[n], uint32_t (&hi)[
 }
 
 // FP8 mode: S bf16(v) and, in lo[0], the n bytes e4m3(S (v - bf16(v))), S = 2^kLoScaleLog2.
+// The product by S and the difference are exact, so the pair is scaled as BF16 (one
+// instruction for two) and the remainder is one FMA.
 template <int n>
 __device__ __forceinline__ void split_piece8(const float (&v)[n], uint32_t (&hi)[n / 2], uint32_t (&lo)[n / 2]) {
   constexpr float S = (float)(1u << kLoScaleLog2);
+  const __nv_bfloat162 S2 = __floats2bfloat162_rn(S, S);
   uint32_t l = 0;
 #pragma unroll
   for (int j = 0; j < n / 2; ++j) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 hs = __floats2bfloat162_rn(hf.x * S, hf.y * S);  // exact
+    const __nv_bfloat162 hs = __hmul2_rn(__floats2bfloat162_rn(v[2 * j], v[2 * j + 1]), S2);
+    const float2 hf = __bfloat1622float2(hs);
     hi[j] = *reinterpret_cast<const uint32_t*>(&hs);
-    l |= (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2((v[2 * j] - hf.x) * S, (v[2 * j + 1] - hf.y) * S),
+    l |= (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(fmaf(v[2 * j], S, -hf.x), fmaf(v[2 * j + 1], S, -hf.y)),
                                             __NV_SATFINITE, __NV_E4M3)
          << (16 * j);
   }
