@@ -801,6 +801,31 @@ cudaError_t launch_csr(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Runs per CTA with which the FP64 per-spin form (step_simt_kernel) fills the SMs in one wave,
+// or 0 where step_f64_kernel is the better one.  A thread with all D components of a spin loads
+// J once for D products and shares the drift's factors, so it wins where its warps are full:
+// one CTA an SM, four warps of (run, spin) slots, three quarters of its passes of 512 threads.
+// us a step, step_f64_kernel -> per spin: ladder N = 100, D = 3, 4000 runs 176 -> 143 (281 with
+// uneven waves of per-spin CTAs); SK N = 1000, D = 3, 64 runs 1200 -> 800; N = 20, D = 3,
+// 1520 runs 25.0 -> 15.8; below the line N = 20, D = 3, 912 runs (120 slots) 10.0 / 10.0 and
+// 304 runs 4.2 / 9.2.  Fewer slots will do where step_f64_kernel would cut an SM's runs into
+// several CTAs (N = 20, D = 8, 608 runs 22.5 -> 20.5).  D = 1 has nothing to share and draws a
+// pair of normals for one: only long dense rows outweigh that (N = 500, 64 runs 106 -> 78).
+int per_spin_f64_runs(const chym_ctx* c, int D, int n_runs) {
+  const int N = c->N;
+  if (D == 1 && (c->sparse || N < 256)) return 0;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  if (sms <= 0) return 0;
+  const long long RC = ((long long)n_runs + sms - 1) / sms, slots = RC * N;
+  const size_t j_bytes = (size_t)N * N * sizeof(double);
+  const size_t avail = kSimtSmemBudget - (!c->sparse && j_bytes <= kSimtSmemBudget / 2 ? j_bytes : 0);
+  if (RC > 64 || RC * 2 * N * D * sizeof(double) > avail) return 0;
+  if (slots < 128 && (RC == 1 || slots * D <= 512)) return 0;
+  const long long passes = (slots + 511) / 512;
+  return passes == 1 || RC == 1 || 4 * slots >= 3 * 512 * passes ? (int)RC : 0;
+}
+
 template <typename T, int D>
 cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   const bool csr = c->sparse;  // the SIMT kernels use the compressed rows whenever they exist
@@ -808,9 +833,14 @@ cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st
     const cudaError_t e = csr ? launch_simt_tiled<D, true>(c, sc, st) : launch_simt_tiled<D, false>(c, sc, st);
     if (e != cudaErrorInvalidConfiguration) return e;
     if (csr) return launch_csr<D>(c, sc, st);
-  } else {
-    const cudaError_t e = launch_f64<D>(c, sc, st);
-    if (e != cudaErrorInvalidConfiguration) return e;
+  }
+  int full = 0;  // runs per CTA of per_spin_f64_runs
+  if constexpr (sizeof(T) == 8) {
+    full = per_spin_f64_runs(c, D, sc.n_runs);
+    if (full == 0) {
+      const cudaError_t e = launch_f64<D>(c, sc, st);
+      if (e != cudaErrorInvalidConfiguration) return e;
+    }
   }
   const int RB = csr ? 1 : SimtTraits<T>::RB;
   const int N = c->N;
@@ -826,6 +856,7 @@ cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   while (RC > RB && (int64_t)((sc.n_runs + RC - 1) / RC) < sms) RC -= RB;
+  if (full > 0) RC = full;
   const size_t smem = (j_smem ? j_bytes : 0) + (size_t)RC * per_run;
   const int threads = std::min(512, std::max(64, ((N * (RC / RB) + 31) / 32) * 32));
   const int grid = (sc.n_runs + RC - 1) / RC;

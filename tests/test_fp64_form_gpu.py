@@ -29,3 +29,14 @@ def test_state_matches_oracle(N, D, n_h, reps, graph):
     Xo = O.run(J, D, inputs.h_per_run(h, reps), seeds, oracle_params(prm), oracle_schedule(sch), steps)
     assert rel_err(X, Xo) <= 1e-10   # FP64 mode, as in the other parity tests
     ctx.close()
+
+
+@pytest.mark.parametrize("N,D,n_h,reps,graph", [
+    (160, 3, 2, 15, "sk"), (20, 3, 7, 200, "sk"), (100, 2, 1, 1201, "mobius"), (300, 1, 1, 41, "gauss"),
+    (130, 8, 3, 7, "sk"), (40, 6, 2, 401, "gauss"), (200, 3, 1, 305, "gauss"), (128, 5, 1, 153, "mobius"),
+    (64, 4, 1, 153, "sk"), (600, 2, 1, 3, "mobius"), (1100, 4, 1, 2, "sk"), (21, 7, 1, 1000, "sk"), (20, 8, 1, 607, "sk")])
+def test_full_warps_one_cta_an_sm(N, D, n_h, reps, graph):
+    """Sizes whose (run, spin) slots fill the warps of one block per SM: several runs per block
+    with a ragged last one, slots from 80 (D = 8), just above 128 and above 512, J in and beyond shared memory,
+    sparse rows, one component."""
+    test_state_matches_oracle(N, D, n_h, reps, graph)
