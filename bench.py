@@ -281,14 +281,12 @@ def step_roofline(jobs, prec, steps_total, dur, clock_info, peaks, peak_src, pre
                          "integer multiply counts 2 (half-rate pipe), frac_unweighted counts it 1"}
 
 
-# DRAM bytes (read + write) of the dominant kernel per launch, from ncu captures of these
-# kernels as they stand (dram__bytes_read.sum + dram__bytes_write.sum), by workload and
-# precision: None where no capture of the current kernel exists.
+# DRAM bytes (read + write) of the dominant kernel, from ncu captures of these kernels as they
+# stand (dram__bytes_read.sum + dram__bytes_write.sum), by workload and precision; a workload
+# without a capture of its current kernel has no entry.
 TRAFFIC = {
-    ("n100", "bf16x2"): (3.25e7, "the three step_tc_kernel launches of one bench step (D = 2, 3, 4; "
-                                 "7.5 + 10.8 + 14.2 MB read, writes stay in L2)"),
-    ("sk800", "fp8"): (2.972e9, "one step_k2_kernel launch (one integration step): 1486 MB captured "
-                                "on 32768 runs, doubled for 65536 (traffic grows with the columns)"),
+    ("sk800", "fp8"): (2.326e9, "step_k2_kernel per integration step: 37.2 GB captured for 64 steps of "
+                                "16384 runs, 4 times that for 65536 (traffic grows with the columns)"),
 }
 
 REPLAY_RUNS, REPLAY_STEPS = 64, 400
