@@ -217,7 +217,7 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     std::vector<unsigned char> items;
     std::vector<int> cta;
     const int chunk = b->shapes.ch[D] ? b->shapes.ch[D] : tc_pick_chunk(D, runs_of[D], P);
-    tc_plan_items(jobs, chunk, tc_runs_per_item(D), P, items, cta);
+    tc_plan_items(D, jobs, chunk, P, items, cta);
     DimLaunch L{D, (int)cta.size() - 1, kp_max, terms_max, chunk, 0, 0, stall};
     b->part_ctas[D] = L.P;
     b->part_units[D] = tc_step_chunks(D, runs_of[D], L.P) * L.P;

@@ -280,11 +280,11 @@ struct TcJob {
 int tc_pick_chunk(int D, long long runs, int P);
 // cost of one step of `runs` runs of dimension D on P CTAs, in chunks of tc_chunk_runs(D) runs
 double tc_step_chunks(int D, long long runs, int P);
-// Split the runs of `jobs` (all of one dimension) over at most P CTAs in near-equal
-// numbers of `chunk`-run chunks; items never cross a context and hold at most `per_item`
-// runs.  items: packed TcItem records; cta_begin: first item of each CTA, and the end.
-void tc_plan_items(const std::vector<TcJob>& jobs, int chunk, int per_item, int P,
-                   std::vector<unsigned char>& items, std::vector<int>& cta_begin);
+// Split the runs of `jobs` (all of dimension D) over at most P CTAs in near-equal numbers
+// of `chunk`-run chunks; items never cross a context.  items: packed TcItem records;
+// cta_begin: first item of each CTA, and the end.
+void tc_plan_items(int D, const std::vector<TcJob>& jobs, int chunk, int P, std::vector<unsigned char>& items,
+                   std::vector<int>& cta_begin);
 cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, const int* d_cta_begin,
                             int n_cta, int64_t steps, int kp_max, int terms_max, unsigned* status,
                             cudaStream_t st, bool test_stall = false, int chunk = 0);

@@ -828,57 +828,113 @@ int tc_pick_chunk(int D, long long runs, int P) {
   return D <= 3 && runs > 4LL * tc_groups(D) * P ? 8 : 4;
 }
 
+namespace {
 // One step of an item with c chunks takes fixed + round ceil(c / groups) + chunk c microseconds:
 // its products, waits and barriers, the longest group's chunks one after the other, and the
 // chunks' share of the arithmetic units.  Fitted at N = 100 to within 5 % (D = 3: 3.23 us with 4
-// chunks, 4.45 with 5, 5.62 with 8).  In chunks of the cost of a full item's.
-double tc_step_chunks(int D, long long runs, int P) {
+// chunks, 4.45 with 5, 5.62 with 8).  Chunks of tc_unit(D) runs, or shorter ones (runs).
+int tc_unit(int D) { return D <= 3 ? 8 : 4; }
+
+double tc_item_us(int D, long long c, int runs) {
   struct Fit {
     double fixed, round, chunk;
   };
   constexpr Fit fits[9] = {{},           {1.00, 0.06, 0.21}, {0.97, 0.60, 0.21}, {0.82, 0.93, 0.37}, {0.90, 0.58, 0.20},
                            {1.50, 0.40, 0.40}, {0.90, 0.87, 0.37}, {1.25, 0.05, 0.75}, {1.75, 0.35, 0.60}};
-  const int unit = D <= 3 ? 8 : 4, full = tc_runs_per_item(D) / unit, G = tc_groups(D);
-  auto item = [&](long long c) {
-    return c ? fits[D].fixed + fits[D].round * (double)((c + G - 1) / G) + fits[D].chunk * (double)c : 0.0;
-  };
-  const long long k = ((runs + unit - 1) / unit + P - 1) / P;  // chunks of the longest list
-  const double t = (double)(k / full) * item(full) + item(k % full);
-  return t * full * unit / (item(full) * tc_chunk_runs(D));
+  const int G = tc_groups(D);
+  const Fit& f = fits[D];
+  return c ? f.fixed + (f.round * (double)((c + G - 1) / G) + f.chunk * (double)c) * runs / tc_unit(D) : 0.0;
 }
 
-void tc_plan_items(const std::vector<TcJob>& jobs, int chunk, int per_item, int P,
-                   std::vector<unsigned char>& items, std::vector<int>& cta_begin) {
+// Chunks [begin, begin + count) of one job on a CTA; the spans of every CTA.
+struct TcSpan {
+  int job;
+  long long begin, count;
+};
+using TcSpread = std::vector<std::vector<TcSpan>>;
+}  // namespace
+
+// In chunks of the cost of a full item's.
+double tc_step_chunks(int D, long long runs, int P) {
+  const int unit = tc_unit(D), full = tc_runs_per_item(D) / unit;
+  const long long k = ((runs + unit - 1) / unit + P - 1) / P;  // chunks of the longest list
+  const double full_us = tc_item_us(D, full, unit), t = (double)(k / full) * full_us + tc_item_us(D, k % full, unit);
+  return t * full * unit / (full_us * tc_chunk_runs(D));
+}
+
+// Two ways to spread the chunks, and the one whose longest CTA is shorter: equal numbers of
+// chunks whatever their context, where a CTA on the border of two contexts runs an item of
+// each, one after the other; or whole CTAs for each context.  An item of one chunk costs
+// nearly as much as one of four, so the second way is the shorter one where a CTA has a chunk
+// or two (five contexts of N = 18, D = 3, 228 runs, 271 steps: 866 us a call the first way, 594
+// the second; 13 packed contexts of D = 2, 672 runs, 500 steps: 3371 and 2674), the first where
+// a CTA has several items anyway or the contexts outnumber the CTAs.
+void tc_plan_items(int D, const std::vector<TcJob>& jobs, int chunk, int P, std::vector<unsigned char>& items,
+                   std::vector<int>& cta_begin) {
+  const int n = (int)jobs.size(), full = tc_runs_per_item(D) / chunk;
+  std::vector<long long> chunks;
   long long C = 0;
-  for (const auto& j : jobs) C += (j.n_runs + chunk - 1) / chunk;
-  if (P > C) P = (int)std::max(1LL, C);
-  const size_t ib = tc_item_bytes();
-  cta_begin.assign(1, 0);
-  int cta = 0;
-  long long acc = 0;
-  auto bound = [&](int b) { return ((long long)(b + 1) * C + P / 2) / P; };
-  int n_items = 0;
   for (const auto& j : jobs) {
-    int run = 0;
-    while (run < j.n_runs) {
-      long long cap = bound(cta) - acc;
-      if (cap <= 0 && cta + 1 < P) {
-        cta_begin.push_back(n_items);
-        ++cta;
+    chunks.push_back((j.n_runs + chunk - 1) / chunk);
+    C += chunks.back();
+  }
+  if (P > C) P = (int)std::max(1LL, C);
+  auto list_us = [&](long long c) {  // items of one context, one after the other
+    return (double)(c / full) * tc_item_us(D, full, chunk) + tc_item_us(D, c % full, chunk);
+  };
+  auto longest = [&](const TcSpread& spread) {
+    double t = 0.0;
+    for (const auto& cta : spread) {
+      double us = 0.0;
+      for (const TcSpan& s : cta) us += list_us(s.count);
+      t = std::max(t, us);
+    }
+    return t;
+  };
+  TcSpread spread(P);
+  long long at = 0;  // chunks placed
+  for (int j = 0, b = 0; j < n; ++j)
+    for (long long done = 0; done < chunks[j];) {
+      const long long cap = ((long long)(b + 1) * C + P / 2) / P - at;  // of CTA b
+      if (cap <= 0) {
+        ++b;
         continue;
       }
-      if (cap <= 0) cap = (j.n_runs - run + chunk - 1) / chunk;  // last CTA takes the rest
-      const int left_chunks = (j.n_runs - run + chunk - 1) / chunk;
-      const int take = (int)std::min<long long>({cap, (long long)(per_item / chunk), (long long)left_chunks});
-      const int runs = std::min(take * chunk, j.n_runs - run);
-      items.resize(items.size() + ib);
-      tc_fill_item(items.data() + items.size() - ib, j.desc, run, runs);
-      ++n_items;
-      run += runs;
-      acc += take;
+      const long long take = std::min(cap, chunks[j] - done);
+      spread[b].push_back(TcSpan{j, done, take});
+      done += take;
+      at += take;
     }
+  if (n > 1 && n <= P) {
+    std::vector<int> of(n, 1);  // CTAs of each job, each next one to the job with the longest list
+    for (int left = P - n; left > 0; --left) {
+      int next = 0;
+      for (int j = 1; j < n; ++j)
+        if (chunks[j] * of[next] > chunks[next] * of[j]) next = j;
+      if (of[next] >= chunks[next]) break;  // a chunk each
+      ++of[next];
+    }
+    TcSpread apart;
+    for (int j = 0; j < n; ++j)
+      for (int b = 0; b < of[j]; ++b) {
+        const long long begin = chunks[j] * b / of[j];
+        apart.push_back({TcSpan{j, begin, chunks[j] * (b + 1) / of[j] - begin}});
+      }
+    if (longest(apart) < longest(spread)) spread.swap(apart);
   }
-  while ((int)cta_begin.size() < P + 1) cta_begin.push_back(n_items);
+  const size_t ib = tc_item_bytes();
+  int n_items = 0;
+  cta_begin.assign(1, 0);
+  for (const auto& cta : spread) {
+    for (const TcSpan& s : cta)
+      for (long long c = 0; c < s.count; c += full, ++n_items) {
+        const int run = (int)(s.begin + c) * chunk;
+        const int runs = std::min((int)std::min<long long>(full, s.count - c) * chunk, jobs[s.job].n_runs - run);
+        items.resize(items.size() + ib);
+        tc_fill_item(items.data() + items.size() - ib, jobs[s.job].desc, run, runs);
+      }
+    cta_begin.push_back(n_items);
+  }
 }
 
 // Launch the small-N tensor-core kernel of dimension D on a prepared plan in
@@ -948,7 +1004,7 @@ cudaError_t launch_step_tc(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   const int chunk = tc_pick_chunk(c->D, sc.n_runs, sms);
   std::vector<unsigned char> items;
   std::vector<int> cta;
-  tc_plan_items({TcJob{0, sc.n_runs}}, chunk, tc_runs_per_item(c->D), sms, items, cta);
+  tc_plan_items(c->D, {TcJob{0, sc.n_runs}}, chunk, sms, items, cta);
   const size_t cta_off = sizeof(TcDesc) + items.size();
   const size_t bytes = cta_off + sizeof(int) * cta.size();
   std::vector<unsigned char> plan(bytes);

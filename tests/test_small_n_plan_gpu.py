@@ -32,3 +32,27 @@ def test_spread_of_the_runs_leaves_states_unchanged(N, D, R):
     assert np.array_equal(ctx.get_state()[0], X)
     b.close()
     ctx.close()
+
+
+# runs per context: CTAs shared between contexts, whole CTAs for each, one run, more contexts than SMs
+@pytest.mark.parametrize("D,runs", [(3, [228] * 5), (2, [105, 105, 105]), (4, [1, 300, 7]), (3, [4096, 5]),
+                                    (1, [3] * 160), (8, [45, 999, 2])])
+def test_spread_of_several_contexts_leaves_states_unchanged(D, runs):
+    sched = chym.Schedule(1, 3, 9)
+    prm = chym.Params(eps=0.06, prec=chym.PREC_BF16X2)
+    ctxs, alone = [], []
+    for i, R in enumerate(runs):
+        ctx = chym.Context(inputs.sk_pm1(18 + i % 7, 3 + i), D, chym.J_PM1)
+        seeds = inputs.run_seeds(50 + i, R)
+        ctx.run(prm, np.array([0.8]), seeds, 7, sched)
+        alone.append(ctx.get_state()[0])
+        ctx.run(prm, np.array([0.8]), seeds, 0, sched)
+        ctxs.append(ctx)
+    b = chym.Batch(ctxs)
+    b.run([prm] * len(runs), [sched] * len(runs), 7)
+    b.status()
+    for ctx, X in zip(ctxs, alone):
+        assert np.array_equal(ctx.get_state()[0], X)
+    b.close()
+    for ctx in ctxs:
+        ctx.close()
