@@ -701,7 +701,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
-  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], drain_bar, stored;
+  __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], stored[2], drain_bar;
   __shared__ uint32_t s_tmem, s_cleared;
   __shared__ int s_rank, s_P;
   __shared__ volatile int s_abort;
@@ -727,9 +727,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&acc_full[b])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&acc_empty[b])),
                    "r"(kEpiWarps));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&stored[b])), "r"(kEpiWarps));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&drain_bar)));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&stored)), "r"(kEpiWarps));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid == 64) {  // count this CTA in; the first one closes the count
@@ -916,7 +916,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           const int i = at.i;
           const K2Tile tile = W.tile(i);
           unsigned* done = L.flags + W.desc(i, tile).flag0 + tile.ct;
-          ok = mbar_wait(smem_addr(&stored), it & 1u, L.wait_ns) && !s_abort;
+          ok = mbar_wait(smem_addr(&stored[it & 1u]), (it >> 1) & 1u, L.wait_ns) && !s_abort;
           if (!ok) break;
           fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
           asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
@@ -946,12 +946,14 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const bool ok = epilogue<D>(W, L, s_runc[warp - kEpiWarp0], acc_full, &s_abort, lane_base, (warp - kEpiWarp0) >> 2, [&](uint32_t it) {
-      // this accumulator may be overwritten now, and the tile's stores published
+      // The tile's stores may be published and its accumulator overwritten.  A warp may be a
+      // tile ahead of another, so each accumulator has its own `stored`; it arrives there first,
+      // so that two tiles ahead, behind acc_empty, every warp has.
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&stored[it & 1u])) : "memory");
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&stored)) : "memory");
       }
     });
     if (!ok && lane == 0) give_up();

@@ -84,3 +84,30 @@ def test_fewer_free_sms_leave_states_unchanged(busy_runs):
     assert np.array_equal(small.get_state(a.cuda_stream)[0], S)
     small.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("D,wide,narrow", [(4, 64, 32), (2, 128, 32), (1, 256, 32)])
+def test_wide_and_narrow_tiles_in_one_list(D, wide, narrow):
+    """Tiles of wide and of narrow columns in turn, M tiles with two live rows, several a CTA:
+    the epilogue's warps finish far apart, and a tile counts as finished only when all have."""
+    # a launch has at least 152 tiles, so a CTA's list holds wide and narrow ones
+    sizes = [(130, 160 * wide), (130, 16), (200, 9), (130, 33), (257, 5), (130, narrow), (140, 1), (385, 16)]
+    prm, sched = [], chym.Schedule(1, 40, 200)
+    ctxs, alone, seeds = [], [], []
+    for i, (N, R) in enumerate(sizes):
+        ctx, eps = _ctx(N, D, "sk" if i % 2 else "gauss")
+        ctxs.append(ctx)
+        prm.append(chym.Params(eps=eps, prec=chym.PREC_BF16X2))
+        seeds.append(inputs.run_seeds(20 + i, R))
+        alone.append(_states(ctx, prm[-1], sched, seeds[-1], 200))
+    batch = chym.Batch(ctxs)
+    batch.set_shapes({"rt": [wide if d == D else 0 for d in range(1, 9)]})
+    for i, ctx in enumerate(ctxs):
+        ctx.run(prm[i], np.array([0.8]), seeds[i], 0, sched)
+    batch.run(prm, [sched] * len(ctxs), 200)
+    batch.status()
+    for ctx, X in zip(ctxs, alone):
+        assert np.array_equal(ctx.get_state()[0], X)
+    batch.close()
+    for ctx in ctxs:
+        ctx.close()
