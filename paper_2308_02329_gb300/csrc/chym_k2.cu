@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&acc_full[b])));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&acc_empty[b])),
-                   "r"(kEpiWarps));
+                   "r"(kEpiWarps + 1));  // and the publisher
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&stored[b])), "r"(kEpiWarps));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&drain_bar)));
@@ -918,6 +918,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           unsigned* done = L.flags + W.desc(i, tile).flag0 + tile.ct;
           ok = mbar_wait(smem_addr(&stored[it & 1u]), (it >> 1) & 1u, L.wait_ns) && !s_abort;
           if (!ok) break;
+          // seen: only now may the tile after next take this accumulator and complete its
+          // `stored` once more (a parity tells the last phase from the one under way, no more;
+          // a publisher two tiles late would wait for a phase that never comes)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
           fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
           asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
         }

@@ -111,3 +111,25 @@ def test_wide_and_narrow_tiles_in_one_list(D, wide, narrow):
     batch.close()
     for ctx in ctxs:
         ctx.close()
+
+
+def test_short_tiles_in_long_walks():
+    """Thousands of the shortest tiles a CTA: the publisher stays within two tiles of the
+    epilogue whatever their times, and no wait runs out."""
+    sched, n, steps = chym.Schedule(1, 400, 1100), 220, 1100
+    ctxs, prm, seeds = [], [], []
+    for i in range(n):
+        ctx, eps = _ctx(129 + i % 3, 1, "sk")
+        ctxs.append(ctx)
+        prm.append(chym.Params(eps=eps, prec=chym.PREC_FP8))
+        seeds.append(inputs.run_seeds(50 + i, 1 + i % 9))
+        ctx.run(prm[i], np.array([0.8]), seeds[i], 0, sched)
+    batch = chym.Batch(ctxs)
+    batch.run(prm, [sched] * n, steps)
+    batch.status()
+    got = {i: ctxs[i].get_state()[0] for i in (0, 1, 100, 219)}
+    for i, X in got.items():
+        assert np.array_equal(X, _states(ctxs[i], prm[i], sched, seeds[i], steps))
+    batch.close()
+    for ctx in ctxs:
+        ctx.close()
