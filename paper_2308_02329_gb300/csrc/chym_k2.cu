@@ -867,7 +867,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
         const uint64_t o_bhi = (kABlock + a2) >> 4, o_blo = o_bhi + (BB >> 4), o_alo = kABlock >> 4;
         constexpr uint64_t kStep = 2u * kCoreK >> 4;
         const int KC = d.KC;
-        if (use > 0 && !mbar_wait(smem_addr(&acc_empty[b]), (use - 1u) & 1u, L.wait_ns)) {
+        // (voted on, like every wait of a warp that goes on together)
+        if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_addr(&acc_empty[b]), (use - 1u) & 1u, L.wait_ns) && !s_abort)) {
           ok = false;
           break;
         }

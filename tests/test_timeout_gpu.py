@@ -98,3 +98,21 @@ def test_stalled_batch_reports_the_timeout_and_recovers():
         assert np.array_equal(c.get_state()[0], ca.get_state()[0])
         c.close()
         ca.close()
+
+
+@pytest.mark.parametrize("D,prec,runs", [(3, chym.PREC_BF16X2, 9728), (8, chym.PREC_FP8, 4864)])
+def test_stall_behind_a_held_accumulator(D, prec, runs):
+    """Three tiles a CTA: the issuer's own wait, for an accumulator that nobody gives back, runs
+    out too, and its warp leaves together."""
+    J, eps, h, seeds = make_case(300, D, 2, runs // 2, 9)
+    sch = chym.Schedule(1, 10, 20)
+    ctx = chym.Context(J, D)
+    ctx.run(_params(eps, prec, False), h, seeds, 4, sch)
+    X, _ = ctx.get_state()
+    ctx.run(_params(eps, prec, True), h, seeds, 4, sch)
+    with pytest.raises(chym.ChymError) as e:
+        ctx.energy()
+    assert e.value.status == chym.ETIMEOUT
+    ctx.run(_params(eps, prec, False), h, seeds, 4, sch)
+    assert np.array_equal(ctx.get_state()[0], X)
+    ctx.close()
