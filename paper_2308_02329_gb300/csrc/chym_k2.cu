@@ -61,8 +61,6 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
-#include <functional>
-#include <queue>
 #include <type_traits>
 #include <utility>
 #include <vector>
@@ -94,8 +92,21 @@ constexpr int kAccCols = 256;                  // TMEM columns of one accumulato
 constexpr size_t kRingBudget = 192 * 1024;     // shared memory for the stage ring
 constexpr int kLaunchSteps = 1024;             // most steps of one launch
 constexpr int kMaxGridY = 65535;
-constexpr int kPhaseTiles = 2;                 // tiles per CTA of a phase (at least)
-constexpr int kPhaseSteps = 32;                // fewest steps of a call that is split into phases
+// Phases.  The CTAs of a phase stay within its tiles of one another, so that those that share a
+// column tile read it while it is in L2; walking their whole lists they drift apart by up to a
+// step.  Two tiles a CTA are the fewest that cover a tile's hand-over: us a step for 1 / 2 / 3 /
+// 4 / all, N = 800, D = 4, 65536 runs 1179 / 766 / 792 / 809 / 943; N = 600, D = 3, 16384 runs
+// 172 / 110 / 112 / 114 / 120; 125 instances of N = 130..2000, D = 4, 64 runs 278 / 207 / 214 /
+// 215 / 218.  A phase costs the filling of the CTAs' pipelines once, not worth it for few steps.
+constexpr int kPhaseTiles = 2;
+constexpr int kPhaseSteps = 32;
+// Several D.  Side by side, on shares of the SMs, they hold each other's data out of L2 and end
+// apart (the 512 instances of the uneven workload: 1064 us a step, 821 one after the other; their
+// D = 4 and 8 alone 601 and 558; 8 instances of 2048 runs 317 and 307), so each has to gain
+// kBesideLoss by the tiles' times: few tiles of each D, which would leave SMs idle.
+constexpr double kBesideLoss = 1.2;
+constexpr double kHandOverNs = 4000.0;         // a step's, with one tile a CTA: store, publish, fetch
+constexpr double kLaunchNs = 10000.0;          // start and end of a launch
 constexpr uint32_t kA8Block = 128 * kKc;       // bytes of an e4m3 A block (4 KB)
 constexpr int kLoScaleLog2 = 16;               // FP8 mode: B operands carry 2^16
 
@@ -1265,22 +1276,82 @@ cudaError_t k2_launch(int D, const K2Launch& L, int grid, size_t smem, cudaStrea
   return cudaErrorInvalidValue;
 }
 
+// Column tiles [ct, ct + n) of a context.
+struct K2Cols {
+  int desc, ct, n;
+};
+using K2Phase = std::vector<K2Cols>;
+
 // The contexts of one D: their tiles in lists per CTA, and where these sit in the device block.
 struct K2Group {
   int D = 0, grid = 0, phases = 1;
   double cost = 0.0;
   size_t n_tiles = 0, o_sync = 0, n_sync = 0, o_tile = 0, o_cta = 0;
-  std::vector<int> descs;
+  std::vector<int> descs;  // the costliest tiles first
   std::vector<std::vector<K2Tile>> lists;
   std::vector<std::vector<int>> phase_end;  // per CTA
 };
+
+// The column tiles of a group in phases of at most `rounds` tiles a CTA, each column tile in
+// the first phase with room for it; the last takes up to a round more rather than leave it to
+// one of its own.
+template <typename Desc>
+std::vector<K2Phase> k2_phases(const K2Group& g, Desc desc, int grid, size_t rounds) {
+  std::vector<K2Phase> out;
+  std::vector<size_t> room;
+  size_t left = g.n_tiles;
+  for (int i : g.descs) {
+    const size_t MT = (size_t)desc(i).MT;
+    size_t f = 0;
+    for (int ct = 0; ct < desc(i).CT;) {
+      while (f < room.size() && room[f] < MT) ++f;
+      if (f == room.size()) {
+        out.emplace_back();
+        room.push_back(left <= (rounds + 1) * grid ? left : std::max(rounds * grid, MT));
+      }
+      const int n = (int)std::min<size_t>(desc(i).CT - ct, room[f] / MT);
+      out[f].push_back(K2Cols{i, ct, n});
+      room[f] -= n * MT;
+      left -= n * MT;
+      ct += n;
+    }
+  }
+  return out;
+}
+
+// Deals a phase's tiles out to `grid` CTAs, each next one to the CTA with the least work so
+// far (the lowest of equals, mt fastest); lists may be null.  Returns the longest load.
+template <typename Desc>
+double k2_deal(const K2Phase& phase, Desc desc, const std::vector<double>& tile_ns, int grid,
+               std::vector<std::vector<K2Tile>>* lists) {
+  std::vector<std::pair<double, int>> load(grid);
+  for (int b = 0; b < grid; ++b) load[b] = {0.0, b};
+  for (const K2Cols& c : phase) {
+    const double ns = tile_ns[c.desc];
+    const int MT = desc(c.desc).MT;
+    for (long long t = 0, n = (long long)c.n * MT; t < n;) {
+      // one tile each to the CTAs that stay below the least loaded one's next tile
+      int m = 1;
+      while (m < grid && load[m].first < load[0].first + ns) ++m;
+      const long long rounds = !lists && m == grid ? std::max(1LL, (n - t) / grid) : 1;
+      m = (int)std::min<long long>(m, n - t);
+      for (int j = 0; j < m; ++j, ++t) {
+        if (lists) (*lists)[load[j].second].push_back(K2Tile{c.desc, (int)(t % MT), c.ct + (int)(t / MT), 0});
+        load[j].first += ns * rounds;
+      }
+      t += m * (rounds - 1);
+      std::sort(load.begin(), load.end());
+    }
+  }
+  return load.back().first;
+}
 
 }  // namespace
 
 // Integrate the contexts whose descriptors are in `descs` (host copies, dims[i] =
 // their D) for `steps` steps on stream st: one persistent launch per D and kLaunchSteps
-// steps.  With several D the CTAs are split in proportion to their work and the launches
-// run side by side on the runner's streams.
+// steps.  Several D take all CTAs one after the other, or shares of them in proportion to
+// their work, side by side on the runner's streams (see kBesideLoss).
 cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const std::vector<int>& dims,
                          int64_t steps, unsigned* status, cudaStream_t st, int ctas, const int* stage_choice) {
   const size_t db = sizeof(K2Desc);
@@ -1310,48 +1381,58 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
     total += g.cost;
     groups.push_back(g);
   }
-  // side by side, each on its share of the CTAs; one after the other where they are too few
-  const bool beside = groups.size() > 1 && ctas >= 2 * (int)groups.size();
-  int left = ctas;
+  for (K2Group& g : groups)
+    std::stable_sort(g.descs.begin(), g.descs.end(), [&](int x, int y) { return tile_ns[x] > tile_ns[y]; });
+  // The phases of a group on n CTAs, and the time of a step over all of them.  Each is dealt out
+  // by itself: what counts is the longest load of every phase, not of the lists (dealt over the
+  // lists, CTAs had 1 to 3 tiles of a phase: N = 800 above 877, N = 600 130, the uneven workload 1275).
+  auto plan = [&](const K2Group& g, int n, double* ns) {
+    const int grid = (int)std::min<size_t>(g.n_tiles, (size_t)n);
+    const size_t rounds = (g.n_tiles + grid - 1) / grid;
+    std::vector<K2Phase> p = k2_phases(g, desc, grid, steps >= kPhaseSteps ? std::min<size_t>(rounds, kPhaseTiles) : rounds);
+    *ns = rounds == 1 ? kHandOverNs : 0.0;
+    for (const K2Phase& c : p) *ns += k2_deal(c, desc, tile_ns, grid, nullptr);
+    return p;
+  };
+  std::vector<int> share(groups.size(), ctas);
+  std::vector<std::vector<K2Phase>> phases(groups.size());
+  double in_turn = 0.0;
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    double ns = 0.0;
+    phases[gi] = plan(groups[gi], ctas, &ns);
+    in_turn += ns + kLaunchNs / (double)std::min<int64_t>(steps, kLaunchSteps);
+  }
+  bool beside = false;
+  if (groups.size() > 1 && ctas >= 2 * (int)groups.size()) {
+    std::vector<int> part(groups.size());
+    std::vector<std::vector<K2Phase>> p(groups.size());
+    int left = ctas;
+    double longest = 0.0;
+    for (size_t gi = 0; gi < groups.size(); ++gi) {
+      const int others = (int)(groups.size() - gi) - 1;
+      part[gi] = std::min(left - others, std::max(1, (int)(left * groups[gi].cost / total + 0.5)));
+      left -= part[gi];
+      total -= groups[gi].cost;
+      double ns = 0.0;
+      p[gi] = plan(groups[gi], part[gi], &ns);
+      longest = std::max(longest, ns);
+    }
+    if (longest * kBesideLoss < in_turn) {
+      beside = true;
+      share.swap(part);
+      phases.swap(p);
+    }
+  }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     K2Group& g = groups[gi];
-    const int others = (int)(groups.size() - gi) - 1;
-    int share = ctas;
-    if (beside) {
-      share = std::min(left - others, std::max(1, (int)(left * g.cost / total + 0.5)));
-      left -= share;
-      total -= g.cost;
-    }
-    g.grid = (int)std::min<size_t>(g.n_tiles, (size_t)share);
-    // the costliest tiles first, each to the CTA with the least work so far (the lowest of
-    // equals: tiles of one cost go round), so the lists end close together
-    std::stable_sort(g.descs.begin(), g.descs.end(), [&](int x, int y) { return tile_ns[x] > tile_ns[y]; });
+    g.grid = (int)std::min<size_t>(g.n_tiles, (size_t)share[gi]);
+    g.phases = (int)phases[gi].size();
     g.lists.resize(g.grid);
     g.phase_end.resize(g.grid);
-    g.phases = steps >= kPhaseSteps ? std::max(1, (int)(g.n_tiles / ((size_t)g.grid * kPhaseTiles))) : 1;
-    using Load = std::pair<double, int>;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int b = 0; b < g.grid; ++b) heap.push({0.0, b});
-    // phases of whole rounds of the grid, as far as the column tiles allow, so that no phase
-    // but the last leaves CTAs idle
-    const size_t rounds = (g.n_tiles + g.grid - 1) / g.grid;
-    size_t dealt = 0;
-    int ph = 0;
-    auto close_phase = [&]() {
+    for (const K2Phase& p : phases[gi]) {
+      k2_deal(p, desc, tile_ns, g.grid, &g.lists);
       for (int b = 0; b < g.grid; ++b) g.phase_end[b].push_back((int)g.lists[b].size());
-      ++ph;
-    };
-    for (int i : g.descs)
-      for (int ct = 0; ct < desc(i).CT; ++ct) {
-        if (ph + 1 < g.phases && dealt + desc(i).MT > rounds * (size_t)(ph + 1) / g.phases * (size_t)g.grid) close_phase();
-        for (int mt = 0; mt < desc(i).MT; ++mt, ++dealt) {  // mt fastest
-          const Load l = heap.top();
-          heap.pop();
-          g.lists[l.second].push_back(K2Tile{i, mt, ct, 0});
-          heap.push({l.first + tile_ns[i], l.second});
-        }
-      }
-    while (ph < g.phases) close_phase();
+    }
   }
   // device block: [join words | column-tile counters] of every group (zeroed per launch), then
   // descriptors, tiles and lists

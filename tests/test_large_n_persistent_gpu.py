@@ -133,3 +133,64 @@ def test_short_tiles_in_long_walks():
     batch.close()
     for ctx in ctxs:
         ctx.close()
+
+
+def _dims_batch(specs, steps, sched):
+    """Contexts (N, D, R) with a state each, and the batch over them."""
+    ctxs, prm, seeds = [], [], []
+    for i, (N, D, R) in enumerate(specs):
+        ctx, eps = _ctx(N, D, "gauss" if i % 3 == 2 else "sk")
+        ctxs.append(ctx)
+        prm.append(chym.Params(eps=eps, prec=chym.PREC_FP8 if i % 2 else chym.PREC_BF16X2))
+        seeds.append(inputs.run_seeds(70 + i, R))
+        ctx.run(prm[i], np.array([0.8]), seeds[i], 0, sched)
+    return ctxs, prm, seeds, chym.Batch(ctxs)
+
+
+@pytest.mark.parametrize("specs", [
+    [(130, 4, 9800), (300, 4, 700), (520, 4, 33), (200, 4, 2500)],                       # one D, phases
+    [(260, 2, 9000), (260, 3, 6000), (200, 2, 40), (390, 8, 3000), (150, 3, 5), (640, 8, 100)],  # in turn
+    [(260, 1, 500), (390, 4, 300), (640, 6, 64), (520, 4, 16), (130, 7, 9)]])              # side by side
+def test_phases_of_several_contexts_and_dims(specs):
+    sched = chym.Schedule(1, 30, 70)
+    ctxs, prm, seeds, batch = _dims_batch(specs, 70, sched)
+    batch.run(prm, [sched] * len(ctxs), 70)
+    batch.status()
+    got = [ctx.get_state()[0] for ctx in ctxs]
+    for ctx, p, sd, X in zip(ctxs, prm, seeds, got):
+        assert np.array_equal(X, _states(ctx, p, sched, sd, 70))
+    batch.close()
+    for ctx in ctxs:
+        ctx.close()
+
+
+def test_several_dims_take_no_longer_than_one_after_the_other():
+    """Many uneven instances of four D in one batch against the four batches of one D each."""
+    torch = pytest.importorskip("torch")
+    sched, steps = chym.Schedule(1, 1000, 2000), 200
+    rng = np.random.default_rng(4)
+    specs = [(int(rng.integers(250, 1100)), (2, 3, 4, 8)[i % 4], 64) for i in range(200)]
+    ctxs, prm, _, batch = _dims_batch(specs, 0, sched)
+    parts = [(batch, list(range(len(specs))))]
+    for D in (2, 3, 4, 8):
+        of = [i for i, s in enumerate(specs) if s[1] == D]
+        parts.append((chym.Batch([ctxs[i] for i in of]), of))
+
+    def ms(b, of):
+        best = np.inf
+        for rep in range(4):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            b.run([prm[i] for i in of], [sched] * len(of), steps, torch.cuda.current_stream().cuda_stream)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1)) if rep else best
+        b.status()
+        return best
+
+    t = [ms(*p) for p in parts]
+    assert t[0] < 1.15 * sum(t[1:]), t
+    for b, _ in parts:
+        b.close()
+    for ctx in ctxs:
+        ctx.close()
