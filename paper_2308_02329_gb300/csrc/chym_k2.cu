@@ -54,7 +54,8 @@
 // tile's epilogue, and one D after the other left most SMs idle.)
 // The CTAs wait for one another, so only CTAs known to be resident take part: each counts
 // itself in; once all have, or 100 us after the first, the first one freezes the count P,
-// CTAs that start later exit, and the P present ones share the lists of the absent ones.
+// CTAs that start later exit, and the P present ones share the lists of the absent ones; such a
+// launch stops early once enough have come late, and the next one counts again (go_on).
 // All waits are bounded; on a timeout the CTA raises the status word, drains its own
 // tensor-core and copy work with bounded waits, frees TMEM and returns.
 #include <cuda_bf16.h>
@@ -91,6 +92,7 @@ static_assert(128 * kHelperRegs + 32 * kEpiWarps * kEpiRegs <= kThreads * kLaunc
 constexpr int kAccCols = 256;                  // TMEM columns of one accumulator
 constexpr size_t kRingBudget = 192 * 1024;     // shared memory for the stage ring
 constexpr int kLaunchSteps = 1024;             // most steps of one launch
+constexpr int kCheckSteps = 2;                 // with CTAs missing: steps between looks for late ones
 constexpr int kMaxGridY = 65535;
 // Phases.  The CTAs of a phase stay within its tiles of one another, so that those that share a
 // column tile read it while it is in L2; walking their whole lists they drift apart by up to a
@@ -150,6 +152,12 @@ struct __align__(16) RunC {
 };
 constexpr int kTileCache = 24;  // tiles of a CTA's list whose descriptors are kept in shared memory
 
+// Where a launch begins: steps taken in this call, and launches that stopped early so far.
+struct K2Progress {
+  int64_t step;
+  int stops, pad;
+};
+
 struct K2Launch {
   const K2Desc* descs;
   const K2Tile* tiles;
@@ -157,10 +165,13 @@ struct K2Launch {
   const int* cta_begin;   // list of CTA b: tiles [cta_begin[b], cta_begin[b + 1])
   const int* phase_end;   // [CTA][phase]: ends of the phases in its list
   int phases;
-  unsigned* sync;         // [0] CTAs present (kFrozen: count closed), [1] their number once closed
+  unsigned* sync;         // [0] CTAs arrived (kFrozen: count closed), [1] their number when it was
+                          // closed, [2] 2 x checks passed + 1 if stopped at the next (go_on)
   unsigned* flags;        // per column tile: M tiles finished, over all steps of the launch
-  int64_t step0;          // steps taken in this call before this launch
-  int steps;
+  K2Progress* progress;   // of this launch and the next, by launch parity
+  int launch;             // parity of its index in the call
+  int max_stops;          // launches of the call that may stop early
+  int64_t total;          // steps of the call
   int stages;             // depth of the ring
   uint32_t stage_stride;  // bytes per stage
   unsigned* status;
@@ -509,10 +520,17 @@ __device__ __forceinline__ void advance_piece(const EpiTile& w, const RunC<D>* r
   if constexpr (D > 4) block(std::integral_constant<int, 1>());
 }
 
+// What a launch does: steps from `step0`, on P CTAs.
+struct K2Span {
+  int64_t step0;
+  int steps, stops, P;
+};
+
 // A CTA's list of tiles: entry i is table entry base + i stride.  The list falls into phases,
 // each advanced by all steps before the next begins.
 struct TileWalk {
   int base, stride, count, phases;
+  const K2Span* span;
   const int* phase_end;  // ends of the phases in the list (one phase: count)
   const K2Launch* L;
   const K2Desc* cache;   // descriptors of the first kTileCache tiles
@@ -524,6 +542,27 @@ struct TileWalk {
   __device__ __forceinline__ int end_of(int ph) const { return phases > 1 ? phase_end[ph] : count; }
 };
 
+// A launch that found SMs busy goes on past step s (a multiple of kCheckSteps) unless CTAs have
+// come late since, a quarter as many as it has or more: then it stops there, and the next
+// launch counts anew (kept to the first SMs for the whole launch, a call of 1000 steps of N = 1000,
+// D = 4, 2048 runs took 334 ms where a run of 2.3 ms held 140 SMs at its start; 34 now, 32 alone).
+// Whoever gets there first decides, so nobody waits: every CTA passes its steps in order, so a
+// check is open only while all before it are passed.
+__device__ __forceinline__ bool go_on(const K2Launch& L, const K2Span& span, int s) {
+  const unsigned e = (unsigned)(s / kCheckSteps);
+  for (;;) {
+    const unsigned v = ld_acquire(L.sync + 2);
+    if (v >> 1 >= e) return true;
+    if (v & 1u) return false;
+    const unsigned late = (ld_acquire(L.sync) & ~kFrozen) - (unsigned)span.P;
+    const bool stop = span.stops < L.max_stops && 4u * late >= (unsigned)span.P;
+    if (atomicCAS(L.sync + 2, v, stop ? v | 1u : 2u * e) != v) continue;  // decided by another
+    if (!stop) return true;
+    L.progress[L.launch ^ 1] = K2Progress{span.step0 + s, span.stops + 1, 0};
+    return false;
+  }
+}
+
 // A place in that walk, in the order in which all roles go: phase, step of the launch, tile.
 struct WalkPos {
   int i, s, i0, i1, ph;
@@ -534,7 +573,7 @@ struct WalkPos {
   __device__ __forceinline__ void next(const TileWalk& W) {
     if (++i < i1) return;
     i = i0;
-    if (++s < W.L->steps) return;
+    if (++s < W.span->steps && (W.span->P == (int)gridDim.x || s % kCheckSteps != 0 || go_on(*W.L, *W.span, s))) return;
     s = 0;
     enter(W, i1);
     skip_empty(W);
@@ -583,7 +622,7 @@ __device__ __forceinline__ bool epilogue(const TileWalk& W, const K2Launch& L, R
   uint32_t it = 0;
   for (WalkPos at(W); !at.done(W); ++it) {
     const int i = at.i;
-    const int64_t step = L.step0 + at.s;
+    const int64_t step = W.span->step0 + at.s;
     at.next(W);  // the tile after this one
     const K2Tile tile = W.tile(i);
     const K2Desc& d = W.desc(i, tile);
@@ -714,7 +753,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
   __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages];
   __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], stored[2], drain_bar;
   __shared__ uint32_t s_tmem, s_cleared;
-  __shared__ int s_rank, s_P;
+  __shared__ int s_rank;
+  __shared__ K2Span s_span;
   __shared__ volatile int s_abort;
   __shared__ RunC<D> s_runc[kEpiWarps][RunC<D>::kSlots];
   __shared__ K2Desc s_desc[kTileCache];
@@ -744,12 +784,17 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid == 64) {  // count this CTA in; the first one closes the count
+    const K2Progress begin = L.progress[L.launch];
     const unsigned old = atomicAdd(L.sync, 1u);
     int P = 0;
-    if (!(old & kFrozen)) {
+    if (begin.step >= L.total) {  // earlier launches have taken all steps
+      if (old == 0) L.progress[L.launch ^ 1] = begin;
+    } else if (!(old & kFrozen)) {
       if (old == 0) {
         counter_wait(L.sync, gridDim.x, kJoinNs);
         P = (int)(atomicOr(L.sync, kFrozen) & ~kFrozen);
+        L.progress[L.launch ^ 1] =
+            K2Progress{begin.step + min((int64_t)kLaunchSteps, L.total - begin.step), begin.stops, 0};
         __threadfence();
         atomicExch(L.sync + 1, (unsigned)P);
       } else if (counter_wait(L.sync + 1, 1u, L.wait_ns)) {
@@ -759,12 +804,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
       }
     }
     s_rank = (int)old;
-    s_P = P;  // 0: too late (or timed out), nothing to do
+    // P = 0: too late (or timed out), nothing to do
+    s_span = K2Span{begin.step, (int)min((int64_t)kLaunchSteps, L.total - begin.step), begin.stops, P};
   }
   __syncthreads();
-  const int P = s_P, rank = s_rank;
+  const int P = s_span.P, rank = s_rank;
   // all present: this CTA's own list; else the table is dealt out round the present ones
-  TileWalk W{0, 1, 0, 1, nullptr, &L, s_desc};
+  TileWalk W{0, 1, 0, 1, &s_span, nullptr, &L, s_desc};
   if (P == (int)gridDim.x) {
     W.base = L.cta_begin[rank];
     W.count = L.cta_begin[rank + 1] - W.base;
@@ -812,7 +858,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           const uint8_t* a_src = d.Aimg + (size_t)tile.mt * KC * kABlock;       // term 0, K chunk 0
           const size_t a_term = (size_t)d.MT * KC * kABlock;                    // to the second term
           const uint8_t* a2_src = d.Aimg + a_term + (size_t)tile.mt * KC * a2;
-          const uint8_t* bx = d.Xt + (size_t)((L.step0 + st) & 1) * d.buf_bytes;
+          const uint8_t* bx = d.Xt + (size_t)((W.span->step0 + st) & 1) * d.buf_bytes;
           const uint8_t* b_src = bx + (size_t)tile.ct * KC * BB;
           const uint8_t* bl_src = bx + (size_t)d.CT * KC * BB + (size_t)tile.ct * KC * BL;
           // the scout has cleared this tile
@@ -1286,7 +1332,8 @@ using K2Phase = std::vector<K2Cols>;
 struct K2Group {
   int D = 0, grid = 0, phases = 1;
   double cost = 0.0;
-  size_t n_tiles = 0, o_sync = 0, n_sync = 0, o_tile = 0, o_cta = 0;
+  size_t n_tiles = 0, o_sync = 0, n_sync = 0, o_progress = 0, o_tile = 0, o_cta = 0;
+  int max_stops = 0;
   std::vector<int> descs;  // the costliest tiles first
   std::vector<std::vector<K2Tile>> lists;
   std::vector<std::vector<int>> phase_end;  // per CTA
@@ -1396,16 +1443,17 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
   };
   std::vector<int> share(groups.size(), ctas);
   std::vector<std::vector<K2Phase>> phases(groups.size());
+  std::vector<double> step_ns(groups.size());
   double in_turn = 0.0;
   for (size_t gi = 0; gi < groups.size(); ++gi) {
-    double ns = 0.0;
-    phases[gi] = plan(groups[gi], ctas, &ns);
-    in_turn += ns + kLaunchNs / (double)std::min<int64_t>(steps, kLaunchSteps);
+    phases[gi] = plan(groups[gi], ctas, &step_ns[gi]);
+    in_turn += step_ns[gi] + kLaunchNs / (double)std::min<int64_t>(steps, kLaunchSteps);
   }
   bool beside = false;
   if (groups.size() > 1 && ctas >= 2 * (int)groups.size()) {
     std::vector<int> part(groups.size());
     std::vector<std::vector<K2Phase>> p(groups.size());
+    std::vector<double> part_ns(groups.size());
     int left = ctas;
     double longest = 0.0;
     for (size_t gi = 0; gi < groups.size(); ++gi) {
@@ -1413,19 +1461,22 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
       part[gi] = std::min(left - others, std::max(1, (int)(left * groups[gi].cost / total + 0.5)));
       left -= part[gi];
       total -= groups[gi].cost;
-      double ns = 0.0;
-      p[gi] = plan(groups[gi], part[gi], &ns);
-      longest = std::max(longest, ns);
+      p[gi] = plan(groups[gi], part[gi], &part_ns[gi]);
+      longest = std::max(longest, part_ns[gi]);
     }
     if (longest * kBesideLoss < in_turn) {
       beside = true;
       share.swap(part);
       phases.swap(p);
+      step_ns.swap(part_ns);
     }
   }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     K2Group& g = groups[gi];
     g.grid = (int)std::min<size_t>(g.n_tiles, (size_t)share[gi]);
+    // a launch for each stop; one that finds nothing left to do takes 3 us
+    const double call_ms = 1e-6 * step_ns[gi] * (double)steps;
+    g.max_stops = (call_ms > 1.0) + (call_ms > 2.0) + (call_ms > 6.0) + (call_ms > 20.0);
     g.phases = (int)phases[gi].size();
     g.lists.resize(g.grid);
     g.phase_end.resize(g.grid);
@@ -1441,6 +1492,10 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
   for (K2Group& g : groups) {
     g.o_sync = at;
     at = up16(at + sizeof(unsigned) * g.n_sync);
+  }
+  for (K2Group& g : groups) {  // zero: the first launch begins at step 0
+    g.o_progress = at;
+    at = up16(at + 2 * sizeof(K2Progress));
   }
   const size_t o_desc = at;
   at = up16(at + descs.size());
@@ -1498,8 +1553,9 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
     const bool side = beside && gi > 0;
     cudaStream_t s = side ? R.streams[gi] : st;
     if (side && (e = cudaStreamWaitEvent(s, R.fork, 0)) != cudaSuccess) return e;
-    for (int64_t s0 = 0; s0 < steps; s0 += kLaunchSteps) {
-      if (s0 > 0 && (e = cudaMemsetAsync(base + g.o_sync, 0, sizeof(unsigned) * g.n_sync, s)) != cudaSuccess) return e;
+    const int64_t launches = (steps + kLaunchSteps - 1) / kLaunchSteps + g.max_stops;
+    for (int64_t i = 0; i < launches; ++i) {
+      if (i > 0 && (e = cudaMemsetAsync(base + g.o_sync, 0, sizeof(unsigned) * g.n_sync, s)) != cudaSuccess) return e;
       K2Launch L;
       L.descs = (const K2Desc*)(base + o_desc);
       L.tiles = (const K2Tile*)(base + g.o_tile);
@@ -1509,8 +1565,10 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
       L.phases = g.phases;
       L.sync = (unsigned*)(base + g.o_sync);
       L.flags = L.sync + 4;
-      L.step0 = s0;
-      L.steps = (int)std::min<int64_t>(kLaunchSteps, steps - s0);
+      L.progress = (K2Progress*)(base + g.o_progress);
+      L.launch = (int)(i & 1);
+      L.max_stops = g.max_stops;
+      L.total = steps;
       L.stages = stages;
       L.stage_stride = stride;
       L.status = status;

@@ -194,3 +194,48 @@ def test_several_dims_take_no_longer_than_one_after_the_other():
         b.close()
     for ctx in ctxs:
         ctx.close()
+
+
+@pytest.mark.parametrize("busy_steps", [(1500,), (600, 1200, 2400, 4800)])
+def test_sms_that_become_free_are_taken(busy_steps):
+    """Small-N runs of other streams hold most SMs for the first few ms of a large-N call: it
+    stops and goes on where it stopped, on all SMs, and takes little longer than they do."""
+    torch = pytest.importorskip("torch")
+    import time
+    ctx, eps = _ctx(520, 4, "sk")
+    prm = chym.Params(eps=eps, prec=chym.PREC_FP8)
+    steps, sched = 1501, chym.Schedule(1, 700, 1400)
+    seeds = inputs.run_seeds(8, 4096)
+    X = _states(ctx, prm, sched, seeds, steps)
+    small, ssched = [], chym.Schedule(1, 10000, 20000)
+    for i, n in enumerate(busy_steps):   # 140 CTAs of four runs in all
+        c, seps = _ctx(100, 4, "sk")
+        small.append((c, chym.Params(eps=seps, prec=chym.PREC_BF16X2), inputs.run_seeds(9 + i, 560 // len(busy_steps)), n,
+                      torch.cuda.Stream()))
+        c.run(small[-1][1], np.array([0.8]), small[-1][2], 10, ssched)
+    own = torch.cuda.Stream()
+
+    def seconds(beside):
+        ctx.run(prm, np.array([0.8]), seeds, 0, sched, own.cuda_stream)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        if beside:
+            for c, p, _, n, stream in small:
+                c.run(p, None, None, n, ssched, stream.cuda_stream)
+            time.sleep(2e-4)
+        if beside != "only":
+            ctx.run(prm, None, None, steps, sched, own.cuda_stream)
+        torch.cuda.synchronize()
+        return time.perf_counter() - t0
+
+    alone = min(seconds(False) for _ in range(3))
+    assert np.array_equal(ctx.get_state()[0], X)
+    busy = min(seconds("only") for _ in range(3))
+    t = []
+    for _ in range(3):
+        t.append(seconds(True))
+        assert np.array_equal(ctx.get_state()[0], X)
+    assert min(t) < 2.0 * alone + busy, (t, alone, busy)
+    for c in small:
+        c[0].close()
+    ctx.close()
