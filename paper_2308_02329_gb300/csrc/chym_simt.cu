@@ -801,29 +801,48 @@ cudaError_t launch_csr(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Runs per CTA with which the FP64 per-spin form (step_simt_kernel) fills the SMs in one wave,
-// or 0 where step_f64_kernel is the better one.  A thread with all D components of a spin loads
-// J once for D products and shares the drift's factors, so it wins where its warps are full:
-// one CTA an SM, four warps of (run, spin) slots, three quarters of its passes of 512 threads.
-// us a step, step_f64_kernel -> per spin: ladder N = 100, D = 3, 4000 runs 176 -> 143 (281 with
-// uneven waves of per-spin CTAs); SK N = 1000, D = 3, 64 runs 1200 -> 800; N = 20, D = 3,
-// 1520 runs 25.0 -> 15.8; below the line N = 20, D = 3, 912 runs (120 slots) 10.0 / 10.0 and
-// 304 runs 4.2 / 9.2.  Fewer slots will do where step_f64_kernel would cut an SM's runs into
-// several CTAs (N = 20, D = 8, 608 runs 22.5 -> 20.5).  D = 1 has nothing to share and draws a
-// pair of normals for one: only long dense rows outweigh that (N = 500, 64 runs 106 -> 78).
+// Runs per CTA with which the FP64 per-spin form (step_simt_kernel) fills the SMs in equal
+// waves, or 0 where step_f64_kernel is the better one.  A thread with all D components of a spin
+// loads J once for D products and shares the drift's factors, so it wins where its warps are
+// full: four warps of (run, spin) slots an SM.  us a step, step_f64_kernel -> per spin:
+//   one CTA an SM: ladder N = 100, D = 3, 4096 runs 174 -> 142; SK N = 500, D = 3, 64 runs 343 ->
+//   213; N = 20, D = 3, 1520 runs 24.4 -> 15.3; below the line, 304 runs 4.2 / 9.2;
+//   several: SK N = 100, D = 3, 4096 runs 385 -> 345, 7904 runs 741 -> 663; ladder, 32768 runs 1384
+//   -> 1155; N = 64, D = 5, 9728 runs 692 -> 629.
+// Fewer slots will do where step_f64_kernel would cut an SM's runs into several CTAs (N = 20,
+// D = 8, 608 runs 21.7 -> 20.1).  The waves are those that waste the least, a CTA whose last
+// pass of 512 threads leaves most idle counted a tenth longer (SK N = 300, D = 3, 256 runs: 187 in
+// CTAs of two runs, 172 of one; N = 20, 4096 runs: 42 of 27, 38 of 14); where a twelfth is wasted
+// all the same, step_f64_kernel's smaller CTAs win (SK N = 1000, D = 2, 1024 runs 3687 / 4115).
+// D = 1 has nothing to share and draws a pair of normals for one: only long dense rows in one
+// full wave outweigh that (N = 500, 64 runs 104 -> 76; N = 300, 7904 runs 1461 / 1532).
 int per_spin_f64_runs(const chym_ctx* c, int D, int n_runs) {
   const int N = c->N;
   if (D == 1 && (c->sparse || N < 256)) return 0;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (sms <= 0) return 0;
-  const long long RC = ((long long)n_runs + sms - 1) / sms, slots = RC * N;
+  const long long share = ((long long)n_runs + sms - 1) / sms, slots = share * N;
+  if (slots < 128 && (share == 1 || slots * D <= 512)) return 0;
   const size_t j_bytes = (size_t)N * N * sizeof(double);
   const size_t avail = kSimtSmemBudget - (!c->sparse && j_bytes <= kSimtSmemBudget / 2 ? j_bytes : 0);
-  if (RC > 64 || RC * 2 * N * D * sizeof(double) > avail) return 0;
-  if (slots < 128 && (RC == 1 || slots * D <= 512)) return 0;
-  const long long passes = (slots + 511) / 512;
-  return passes == 1 || RC == 1 || 4 * slots >= 3 * 512 * passes ? (int)RC : 0;
+  const long long fit = std::min<long long>(64, avail / ((size_t)2 * N * D * sizeof(double)));
+  if (fit < 1) return 0;
+  const long long fewest = (share + fit - 1) / fit;
+  if (D == 1 && fewest > 1) return 0;
+  long long RC = 0, least = 0;  // in tenths of a run
+  for (long long waves = fewest; waves <= (D == 1 ? 1 : 2 * fewest); ++waves) {
+    const long long runs = (share + waves - 1) / waves, passes = (runs * N + 511) / 512;
+    const bool full = passes == 1 || runs == 1 || 4 * runs * N >= 3 * 512 * passes;
+    if (D == 1 && !full) return 0;
+    const long long cost = waves * runs * (full ? 10 : 11);
+    if (RC == 0 || cost < least) {
+      RC = runs;
+      least = cost;
+    }
+  }
+  const long long used = (share + RC - 1) / RC * RC;
+  return 12 * used <= 13 * share ? (int)RC : 0;
 }
 
 template <typename T, int D>

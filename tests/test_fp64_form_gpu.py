@@ -40,3 +40,34 @@ def test_full_warps_one_cta_an_sm(N, D, n_h, reps, graph):
     with a ragged last one, slots from 80 (D = 8), just above 128 and above 512, J in and beyond shared memory,
     sparse rows, one component."""
     test_state_matches_oracle(N, D, n_h, reps, graph)
+
+
+@pytest.mark.parametrize("N,D,n_h,reps,graph", [
+    (10, 3, 1, 9800, "sk"), (20, 3, 1, 4096, "sk"), (100, 2, 1, 4097, "sk"), (48, 4, 1, 9733, "mobius"),
+    (101, 8, 1, 1530, "gauss"), (300, 3, 1, 256, "sk"), (500, 3, 1, 1369, "mobius"), (300, 1, 1, 7904, "mobius")])
+def test_several_waves(N, D, n_h, reps, graph):
+    """More runs than one block per SM holds, and blocks of half the runs where one would leave
+    most of a pass idle: equal waves, the last one ragged."""
+    test_state_matches_oracle(N, D, n_h, reps, graph)
+
+
+def test_two_waves_take_no_longer_than_twice_one():
+    torch = pytest.importorskip("torch")
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ctx = chym.Context(inputs.sk_pm1(100, 3), 3)
+    prm, sch = chym.Params(eps=0.025, prec=chym.PREC_FP64), chym.Schedule(1, 100, 200)
+
+    def ms(R):
+        ctx.run(prm, np.array([0.8]), inputs.run_seeds(4, R), 0, sch)
+        best = np.inf
+        for _ in range(4):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            ctx.run(prm, None, None, 20, sch, torch.cuda.current_stream().cuda_stream)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1))
+        return best
+
+    assert ms(52 * sms) < 2.1 * ms(26 * sms)   # 26 runs fill a block's shared memory
+    ctx.close()
