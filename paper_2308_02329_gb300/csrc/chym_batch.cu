@@ -437,9 +437,11 @@ CHYM_API chym_status chym_batch_tune(chym_batch* b, const chym_params* params,
   }
   // ---- tile shapes: coordinate search, one part at a time, at the tuned split ----
   // Each candidate runs the whole batch for probe_steps steps (timed per part); a part
-  // keeps the candidate under which its own time was shortest.  Large-N parts (one per
-  // dimension, timed together): runs per column tile, then ring depth; small-N parts:
-  // the epilogue chunk.  Changing one part's shape leaves the others' work unchanged.
+  // keeps the candidate under which its own time was shortest, 0 (the choice made for each
+  // call: k2_pick_rt, tc_pick_chunk) the first of them.  Large-N parts (one per dimension,
+  // timed together): runs per column tile, then ring depth; small-N parts: the epilogue
+  // chunk, which D >= 4 has no choice of.  Changing one part's shape leaves the others' work
+  // unchanged.
   if (status == CHYM_OK) {
     for (int D = 0; D <= 8; ++D) b->chunk_cost[D] = best_chunk[D];
     b->k2_cost = best_k2;
@@ -478,9 +480,11 @@ CHYM_API chym_status chym_batch_tune(chym_batch* b, const chym_params* params,
     for (int D = 1; D <= 8 && status == CHYM_OK; ++D) {
       if (!large[D]) continue;
       double best = INFINITY;
-      int best_rt = b->shapes.rt[D];
-      for (int rt = 32; rt <= 256 && status == CHYM_OK; rt *= 2) {
-        if (!k2_rt_valid(D, rt) || (rt > 32 && rt / 2 >= runs[D])) continue;
+      int best_rt = 0;
+      // 0 may be narrower than 32 (N = 250, D = 3, 1024 runs: 16 runs, 9.1 us a step; 32 runs 11.2)
+      for (int rt : {0, 32, 64, 128, 256}) {
+        if (status != CHYM_OK) break;
+        if (rt && (!k2_rt_valid(D, rt) || (rt > 32 && rt / 2 >= runs[D]))) continue;
         b->shapes.rt[D] = rt;
         double t = 0.0;
         status = probe(0, &t);
@@ -503,15 +507,21 @@ CHYM_API chym_status chym_batch_tune(chym_batch* b, const chym_params* params,
       }
       b->shapes.stages[D] = best_s;
     }
-    for (int D = 1; D <= 4 && status == CHYM_OK; ++D) {
+    for (int D = 1; D <= 3 && status == CHYM_OK; ++D) {
       if (!small[D]) continue;
-      double t8 = 0.0, t4 = 0.0;
-      b->shapes.ch[D] = 8;
-      status = probe(D, &t8);
-      if (status != CHYM_OK) break;
-      b->shapes.ch[D] = 4;
-      status = probe(D, &t4);
-      b->shapes.ch[D] = t4 < t8 ? 4 : 8;
+      double best = INFINITY;
+      int best_ch = 0;
+      for (int ch : {0, 8, 4}) {
+        if (status != CHYM_OK) break;
+        b->shapes.ch[D] = ch;
+        double t = 0.0;
+        status = probe(D, &t);
+        if (status == CHYM_OK && t < best) {
+          best = t;
+          best_ch = ch;
+        }
+      }
+      b->shapes.ch[D] = best_ch;
     }
   }
   b->timing = false;
