@@ -409,6 +409,11 @@ class MLP:
             pass
 
 
+# Version of the planner's cost model, part of a tuning cache's keys: the unit of the costs and
+# what the shapes choose from.  2: a chunk's cost is that of a full item's (1: of any chunk).
+COST_MODEL = 2
+
+
 class Batch:
     """Several contexts integrated together (see chym_batch_* in include/chym.h)."""
 
@@ -463,11 +468,12 @@ class Batch:
 
     def tune(self, params, schedules, probe_steps=64, stream=0, cache_path=None, device_key=""):
         """Measure the cost model (chym_batch_tune).  With cache_path, a JSON file of
-        earlier tunings keyed by device_key and the batch's composition: a hit sets
-        the cached costs without measuring, a miss measures and adds the entry."""
+        earlier tunings keyed by device_key, the batch's composition and the version of the
+        cost model: a hit sets the cached costs without measuring, a miss measures and adds
+        the entry."""
         import json
         import os
-        key = self.signature(device_key)
+        key = "%s-%d" % (self.signature(device_key), COST_MODEL)
         cache = {}
         if cache_path and os.path.exists(cache_path):
             with open(cache_path) as f:

@@ -49,3 +49,21 @@ def test_tuned_is_not_slower_than_untuned(specs):
     batch.close()
     for c in ctxs:
         c.close()
+
+
+def test_cached_tuning_of_another_cost_model_is_not_taken(tmp_path):
+    """An entry without the version (written before there was one) is measured anew and kept."""
+    ctxs, batch, prm, sched = _batch([(100, 3, 64), (200, 2, 40)], 20)
+    path = tmp_path / "tuning.json"
+    old = {"chunk": [123.0] * 8, "k2": 456.0, "shapes": {"rt": [32] * 8, "stages": [2] * 8, "ch": [0] * 8}}
+    path.write_text(json.dumps({batch.signature("gpu"): old}))
+    t = batch.tune(prm, sched, probe_steps=4, cache_path=str(path), device_key="gpu")
+    assert t["chunk"] != old["chunk"] and t["k2"] != old["k2"]
+    cache = json.loads(path.read_text())
+    assert cache.pop(batch.signature("gpu")) == old and len(cache) == 1
+    other = chym.Batch(ctxs)
+    assert other.tune(prm, sched, probe_steps=4, cache_path=str(path), device_key="gpu")["chunk"] == t["chunk"]
+    other.close()
+    batch.close()
+    for c in ctxs:
+        c.close()
