@@ -139,6 +139,11 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_pm1_kernel(
 // run a block, and 2.53 ms with 64-bit integer adds.
 constexpr int kDigits = 6, kDigitBits = 11;
 
+// Place of tile (i, j), i <= j, among those on and above the diagonal, row by row.
+__host__ __device__ inline size_t digit_tile(int i, int j, int tiles) {
+  return (size_t)i * tiles - (size_t)i * (i - 1) / 2 + (j - i);
+}
+
 __device__ __forceinline__ void mma_f16(float (&c)[4], const uint4& a, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_real_kernel(
 #pragma unroll
   for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = 0.0;
   for (int i = warp; i < tiles; i += kWarps) {
-    const uint4* a = Jd + ((size_t)i * tiles + i) * (kDigits * 32) + lane;
+    const uint4* a = Jd + digit_tile(i, i, tiles) * (kDigits * 32) + lane;
     float c[NT][kDigits][4];
     auto clear = [&]() {
 #pragma unroll
@@ -253,8 +258,8 @@ __global__ void row_exponents_kernel(const double* __restrict__ J, int N, int32_
   }
 }
 
-// Digit planes as A fragments: Jd[row tile][column tile][digit][lane], four FP16 pairs of
-// columns (2t, 2t+1): rows g, g + 8 at columns 2t, then at 2t + 8.  Zero past N.
+// Digit planes as A fragments: Jd[digit_tile][digit][lane], four FP16 pairs of columns
+// (2t, 2t+1): rows g, g + 8 at columns 2t, then at 2t + 8.  Zero past N.
 __global__ void digits_kernel(const double* __restrict__ J, int N, const int32_t* __restrict__ e_row,
                               uint4* __restrict__ Jd) {
   const int tiles = (N + 15) / 16;
@@ -262,6 +267,7 @@ __global__ void digits_kernel(const double* __restrict__ J, int N, const int32_t
   for (size_t s = blockIdx.x * (size_t)blockDim.x + threadIdx.x; s < total; s += (size_t)gridDim.x * blockDim.x) {
     const int lane = (int)(s & 31), g = lane >> 2, t2 = 2 * (lane & 3);
     const int i = (int)(s / 32 / tiles), j = (int)(s / 32 % tiles);
+    if (j < i) continue;
     uint32_t out[kDigits][4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
@@ -281,7 +287,7 @@ __global__ void digits_kernel(const double* __restrict__ J, int N, const int32_t
     }
 #pragma unroll
     for (int d = 0; d < kDigits; ++d)
-      Jd[((size_t)i * tiles + j) * (kDigits * 32) + d * 32 + lane] = make_uint4(out[d][0], out[d][1], out[d][2], out[d][3]);
+      Jd[digit_tile(i, j, tiles) * (kDigits * 32) + d * 32 + lane] = make_uint4(out[d][0], out[d][1], out[d][2], out[d][3]);
   }
 }
 
@@ -512,9 +518,9 @@ cudaError_t launch_segments_typed(chym_ctx* c, const SegTable& t, double* d_E, c
 
 // Digit planes and row exponents of a context with real couplings, from its FP64 copy.
 cudaError_t prepare_energy_digits(chym_ctx* c) {
-  const size_t tiles = (c->N + 15) / 16;
+  const int tiles = (c->N + 15) / 16;
   cudaError_t e = cudaMalloc((void**)&c->d_Jexp, sizeof(int32_t) * c->N);
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_Jdig, tiles * tiles * kDigits * 32 * sizeof(uint4));
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_Jdig, digit_tile(tiles, tiles, tiles) * kDigits * 32 * sizeof(uint4));
   if (e != cudaSuccess) return e;
   row_exponents_kernel<<<152 * 2, 256>>>(c->d_J64, c->N, c->d_Jexp);
   digits_kernel<<<152 * 8, 256>>>(c->d_J64, c->N, c->d_Jexp, (uint4*)c->d_Jdig);

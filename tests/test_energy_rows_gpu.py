@@ -92,3 +92,17 @@ def test_rows_shared_between_blocks(N, R, prec):
     assert np.array_equal(chym.unpack_spins(S, N)[ok], s[ok])
     assert np.array_equal(E[ok], _field_energy(J, s)[ok])
     ctx.close()
+
+
+def test_real_couplings_device_memory():
+    """A context with real couplings holds them in FP64, FP32 (twice, one with padded rows) and
+    the digit planes of the tiles on and above the diagonal: 23 bytes an entry."""
+    torch = pytest.importorskip("torch")
+    N = 2048
+    J = inputs.gaussian(N, 5)
+    chym.Context(inputs.gaussian(16, 5), 1, chym.J_REAL).close()   # the module's own memory
+    free = torch.cuda.mem_get_info()[0]
+    ctx = chym.Context(J, 1, chym.J_REAL)
+    used = free - torch.cuda.mem_get_info()[0]
+    assert used <= 25 * N * N
+    ctx.close()
