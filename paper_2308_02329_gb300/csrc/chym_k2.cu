@@ -99,9 +99,14 @@ constexpr int kMaxGridY = 65535;
 // step.  Two tiles a CTA are the fewest that cover a tile's hand-over: us a step for 1 / 2 / 3 /
 // 4 / all, N = 800, D = 4, 65536 runs 1179 / 766 / 792 / 809 / 943; N = 600, D = 3, 16384 runs
 // 172 / 110 / 112 / 114 / 120; 125 instances of N = 130..2000, D = 4, 64 runs 278 / 207 / 214 /
-// 215 / 218.  A phase costs the filling of the CTAs' pipelines once, not worth it for few steps.
-constexpr int kPhaseTiles = 2;
+// 215 / 218.  Lists shorter than kPhaseMin keep together by themselves, and in phases a context
+// whose tiles lie first in some lists and last in others has no slack for its hand-over (30
+// instances of N = 176..2000, D = 2..8, 64 runs, D = 2 in two phases: 86, else 74).  A phase costs the
+// filling of the CTAs' pipelines once, not worth it for few steps, and leaves CTAs idle where tiles
+// are uneven: by the tiles' times phases may be longer than whole lists by kDriftLoss.
+constexpr int kPhaseTiles = 2, kPhaseMin = 4;
 constexpr int kPhaseSteps = 32;
+constexpr double kDriftLoss = 1.1;
 // Several D.  Side by side, on shares of the SMs, they hold each other's data out of L2 and end
 // apart (the 512 instances of the uneven workload: 1064 us a step, 821 one after the other; their
 // D = 4 and 8 alone 601 and 558; 8 instances of 2048 runs 317 and 307), so each has to gain
@@ -976,12 +981,12 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           unsigned* done = L.flags + W.desc(i, tile).flag0 + tile.ct;
           ok = mbar_wait(smem_addr(&stored[it & 1u]), (it >> 1) & 1u, L.wait_ns) && !s_abort;
           if (!ok) break;
-          // seen: only now may the tile after next take this accumulator and complete its
-          // `stored` once more (a parity tells the last phase from the one under way, no more;
-          // a publisher two tiles late would wait for a phase that never comes)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
           fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
           asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
+          // only now may the tile after next take this accumulator and complete its `stored`
+          // once more (a parity tells the last phase from the one under way, no more; a
+          // publisher two tiles late would wait for a phase that never comes)
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
         }
         if (!ok) give_up();
       }
@@ -1436,9 +1441,21 @@ cudaError_t k2_integrate(K2Runner& R, std::vector<unsigned char>& descs, const s
   auto plan = [&](const K2Group& g, int n, double* ns) {
     const int grid = (int)std::min<size_t>(g.n_tiles, (size_t)n);
     const size_t rounds = (g.n_tiles + grid - 1) / grid;
-    std::vector<K2Phase> p = k2_phases(g, desc, grid, steps >= kPhaseSteps ? std::min<size_t>(rounds, kPhaseTiles) : rounds);
-    *ns = rounds == 1 ? kHandOverNs : 0.0;
-    for (const K2Phase& c : p) *ns += k2_deal(c, desc, tile_ns, grid, nullptr);
+    auto step = [&](const std::vector<K2Phase>& p) {
+      double t = rounds == 1 ? kHandOverNs : 0.0;
+      for (const K2Phase& c : p) t += k2_deal(c, desc, tile_ns, grid, nullptr);
+      return t;
+    };
+    std::vector<K2Phase> p = k2_phases(g, desc, grid, rounds);
+    *ns = step(p);
+    if (steps >= kPhaseSteps && g.n_tiles >= kPhaseMin * (size_t)grid) {
+      std::vector<K2Phase> q = k2_phases(g, desc, grid, kPhaseTiles);
+      const double t = step(q);
+      if (t < *ns * kDriftLoss) {
+        p.swap(q);
+        *ns = t;
+      }
+    }
     return p;
   };
   std::vector<int> share(groups.size(), ctas);

@@ -239,3 +239,26 @@ def test_sms_that_become_free_are_taken(busy_steps):
     for c in small:
         c[0].close()
     ctx.close()
+
+
+@pytest.mark.parametrize("N,D,R,kind", [(250, 3, 1024, "gauss"), (260, 4, 1200, "sk"), (130, 8, 1000, "sk"), (520, 4, 8192, "sk")])
+@pytest.mark.parametrize("busy_runs", [304, 600])
+def test_late_ctas_and_narrow_tiles_or_phases(N, D, R, kind, busy_runs):
+    """16- and 24-run tiles, several a CTA while SMs are held elsewhere, and phases once they are free."""
+    torch = pytest.importorskip("torch")
+    ctx, eps = _ctx(N, D, kind)
+    prm = chym.Params(eps=eps, prec=chym.PREC_BF16X2)
+    steps, sched = 450, chym.Schedule(1, 200, 400)
+    seeds = inputs.run_seeds(8, R)
+    X = _states(ctx, prm, sched, seeds, steps)
+    small, seps = _ctx(100, 4, "sk")
+    sprm, ssched = chym.Params(eps=seps, prec=chym.PREC_BF16X2), chym.Schedule(1, 10000, 20000)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    ctx.run(prm, np.array([0.8]), seeds, 0, sched, b.cuda_stream)
+    small.run(sprm, np.array([0.8]), inputs.run_seeds(9, busy_runs), 0, ssched, a.cuda_stream)
+    torch.cuda.synchronize()
+    small.run(sprm, None, None, 700, ssched, a.cuda_stream)   # about a millisecond
+    ctx.run(prm, None, None, steps, sched, b.cuda_stream)
+    assert np.array_equal(ctx.get_state(b.cuda_stream)[0], X)
+    small.close()
+    ctx.close()
