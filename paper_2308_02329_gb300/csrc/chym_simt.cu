@@ -845,6 +845,8 @@ int per_spin_f64_runs(const chym_ctx* c, int D, int n_runs) {
   return 12 * used <= 13 * share ? (int)RC : 0;
 }
 
+constexpr size_t kSmSharedBytes = 228 * 1024;  // of an SM
+
 template <typename T, int D>
 cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   const bool csr = c->sparse;  // the SIMT kernels use the compressed rows whenever they exist
@@ -875,8 +877,16 @@ cudaError_t launch_simt_typed(chym_ctx* c, const StepConsts& sc, cudaStream_t st
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   while (RC > RB && (int64_t)((sc.n_runs + RC - 1) / RC) < sms) RC -= RB;
-  if (full > 0) RC = full;
-  const size_t smem = (j_smem ? j_bytes : 0) + (size_t)RC * per_run;
+  size_t smem_least = 0;
+  if (full > 0) {
+    RC = full;
+    // No more CTAs on an SM than the waves: SMs that come free before others (behind another
+    // kernel) would take two where one each was meant (N = 100, D = 3, 1024 runs behind the
+    // large-N launch of a batch: 173 us a step on half the SMs, 87 on all)
+    const int waves = ((sc.n_runs + sms - 1) / sms + RC - 1) / RC;
+    smem_least = kSmSharedBytes / (waves + 1);
+  }
+  const size_t smem = std::max((j_smem ? j_bytes : 0) + (size_t)RC * per_run, smem_least);
   const int threads = std::min(512, std::max(64, ((N * (RC / RB) + 31) / 32) * 32));
   const int grid = (sc.n_runs + RC - 1) / RC;
   const T* J = sizeof(T) == 8 ? (const T*)c->d_J64 : (const T*)c->d_J32;

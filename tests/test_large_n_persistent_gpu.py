@@ -262,3 +262,35 @@ def test_late_ctas_and_narrow_tiles_or_phases(N, D, R, kind, busy_runs):
     assert np.array_equal(ctx.get_state(b.cuda_stream)[0], X)
     small.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("other", [(100, 3, 1024, "sk", chym.PREC_FP64), (100, 4, 4096, "sk", chym.PREC_FP32),
+                                   (2048, 3, 1024, "ladder", chym.PREC_BF16X2)])
+def test_batch_with_other_kernels_takes_no_longer_than_its_parts(other):
+    """A large-N context beside one that runs in FP64, plain FP32 or over sparse rows."""
+    torch = pytest.importorskip("torch")
+    steps, sched = 400, chym.Schedule(1, 1000, 2000)
+    N, D, R, kind, prec = other
+    ctxs = [chym.Context(inputs.mobius_ladder(N) if kind == "ladder" else inputs.sk_pm1(N, 3), D),
+            chym.Context(inputs.sk_pm1(1000, 3), 4)]
+    prm = [chym.Params(eps=0.02, prec=prec), chym.Params(eps=0.008, prec=chym.PREC_BF16X2)]
+    for c, p, runs in zip(ctxs, prm, (R, 2048)):
+        c.run(p, np.array([0.8]), inputs.run_seeds(4, runs), 0, sched)
+
+    def ms(of):
+        b, t = chym.Batch([ctxs[i] for i in of]), []
+        for _ in range(5):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            b.run([prm[i] for i in of], [sched] * len(of), steps, torch.cuda.current_stream().cuda_stream)
+            t1.record()
+            torch.cuda.synchronize()
+            t.append(t0.elapsed_time(t1))
+        b.status()
+        b.close()
+        return sorted(t)[2]
+
+    both, small, large = ms([0, 1]), ms([0]), ms([1])
+    assert both < 1.15 * (large + small), (both, large, small)
+    for c in ctxs:
+        c.close()
