@@ -981,12 +981,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_k2_kernel(K2Launch L) {
           unsigned* done = L.flags + W.desc(i, tile).flag0 + tile.ct;
           ok = mbar_wait(smem_addr(&stored[it & 1u]), (it >> 1) & 1u, L.wait_ns) && !s_abort;
           if (!ok) break;
+          // seen: only now may the tile after next take this accumulator and complete its
+          // `stored` once more (a parity tells the last phase from the one under way, no more;
+          // a publisher two tiles late would wait for a phase that never comes).  Behind the
+          // publication, 2 us later, it costs 1 % where a CTA has few short tiles
+          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
           fence_proxy_async();  // the epilogue's stores (generic proxy) before other SMs' TMA reads
           asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(1u) : "memory");
-          // only now may the tile after next take this accumulator and complete its `stored`
-          // once more (a parity tells the last phase from the one under way, no more; a
-          // publisher two tiles late would wait for a phase that never comes)
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&acc_empty[it & 1u])) : "memory");
         }
         if (!ok) give_up();
       }
@@ -1376,7 +1377,7 @@ std::vector<K2Phase> k2_phases(const K2Group& g, Desc desc, int grid, size_t rou
 template <typename Desc>
 double k2_deal(const K2Phase& phase, Desc desc, const std::vector<double>& tile_ns, int grid,
                std::vector<std::vector<K2Tile>>* lists) {
-  std::vector<std::pair<double, int>> load(grid);
+  std::vector<std::pair<double, int>> load(grid), merged(grid);
   for (int b = 0; b < grid; ++b) load[b] = {0.0, b};
   for (const K2Cols& c : phase) {
     const double ns = tile_ns[c.desc];
@@ -1392,7 +1393,8 @@ double k2_deal(const K2Phase& phase, Desc desc, const std::vector<double>& tile_
         load[j].first += ns * rounds;
       }
       t += m * (rounds - 1);
-      std::sort(load.begin(), load.end());
+      std::merge(load.begin(), load.begin() + m, load.begin() + m, load.end(), merged.begin());  // both sorted
+      load.swap(merged);
     }
   }
   return load.back().first;
