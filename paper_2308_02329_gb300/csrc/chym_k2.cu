@@ -109,9 +109,11 @@ constexpr int kPhaseSteps = 32;
 constexpr double kDriftLoss = 1.1;
 // Several D.  Side by side, on shares of the SMs, they hold each other's data out of L2 and end
 // apart (the 512 instances of the uneven workload: 1064 us a step, 821 one after the other; their
-// D = 4 and 8 alone 601 and 558; 8 instances of 2048 runs 317 and 307), so each has to gain
-// kBesideLoss by the tiles' times: few tiles of each D, which would leave SMs idle.
-constexpr double kBesideLoss = 1.2;
+// D = 4 and 8 alone 601 and 558; 8 instances of 2048 runs 317 and 307, 0.90 by the tiles' times), so
+// it has to gain kBesideLoss by those: few tiles of each D, which would leave SMs idle (28
+// instances of N = 61..1707, D = 3 and 4, 72 runs, 0.86: 42 steps take 9.44 ms side by side, 9.85 in
+// turn; the 30 uneven ones of kPhaseMin, 0.55: 72 and 137 us a step).
+constexpr double kBesideLoss = 1.14;
 constexpr double kHandOverNs = 4000.0;         // a step's, with one tile a CTA: store, publish, fetch
 constexpr double kLaunchNs = 10000.0;          // start and end of a launch
 constexpr uint32_t kA8Block = 128 * kKc;       // bytes of an e4m3 A block (4 KB)
