@@ -285,7 +285,9 @@ def step_roofline(jobs, prec, steps_total, dur, clock_info, peaks, peak_src, pre
 # stand (dram__bytes_read.sum + dram__bytes_write.sum), by workload and precision; a workload
 # without a capture of its current kernel has no entry.
 TRAFFIC = {
-    ("sk800", "fp8"): (2.326e9, "step_k2_kernel per integration step: 37.2 GB captured for 64 steps of "
+    ("n100", "bf16x2"): (3.06e7, "the three step_tc_kernel launches of one bench step (D = 2, 3, 4; "
+                                 "6.8 + 10.2 + 13.5 MB read, writes stay in L2)"),
+    ("sk800", "fp8"): (2.001e9, "step_k2_kernel per integration step: 32.0 GB captured for 64 steps of "
                                 "16384 runs, 4 times that for 65536 (traffic grows with the columns)"),
 }
 
@@ -1005,8 +1007,9 @@ def measure(args, w, sim_steps, rank, world, local, warm_steps=None, replay=Fals
         # statistics per context (a pack of graphs: pump indices, init and one segment
         # energy launch, its statistics are host-side); one persistent launch per
         # dimension for the small-N contexts; the large-N path adds 3 layout kernels per
-        # context and one persistent launch per dimension and 1024 integration steps; FP32/FP64
-        # contexts and sparse ones take one persistent SIMT launch each
+        # context and one persistent launch per dimension and 1024 integration steps (the up to
+        # four more that find no step left to take are not counted); FP32/FP64 contexts and
+        # sparse ones take one persistent SIMT launch each
         bf16 = prec in (chym.PREC_BF16X2, chym.PREC_FP8)
         small = [j for j in jobs if j["N"] <= 128 and bf16]
         large = [j for j in jobs if j["N"] > 128 and bf16 and not j["ctx"].uses_csr(prec)]

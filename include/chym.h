@@ -321,9 +321,9 @@ CHYM_API chym_status chym_batch_status(chym_batch* b);
 /* Autotuner of the batch planner.  The planner splits the SMs between the
  * small-N dimensions and the large-N launches in proportion to their estimated
  * work, from a cost model in SM-microseconds: per dimension D, one chunk of runs
- * (8 runs for D <= 4, 4 above) advanced one step on the small-N path; and one
- * unit of the large-N path (a 128-row output tile x one 64-wide K chunk) advanced
- * one step.  chym_batch_tune measures these costs on the current device for the
+ * (8 runs for D <= 4, 4 above) of a full item advanced one step on the small-N path;
+ * and one unit of the large-N path (a 128-row output tile x one 64-wide K chunk)
+ * advanced one step.  chym_batch_tune measures these costs on the current device for the
  * batch's own contexts at the split they run with: the whole batch is integrated
  * for probe_steps steps (once to warm up, then a few rounds timed per part with CUDA
  * events, each part's time the shorter of two runs); after each round every part's

@@ -3,11 +3,12 @@
 // Contexts on the small-N tensor-core path (N <= 128) are integrated by one
 // persistent launch per hyperspin dimension D.  Every CTA of such a launch walks a
 // host-built list of items (a run range of one context).  The planner spreads each
-// dimension's runs over its CTAs in near-equal numbers of 8-run chunks, so no SM
-// idles while another finishes a whole extra item.  The SMs are shared between the
-// dimensions in proportion to their estimated cost.  Contexts on the large-N path
-// run in one persistent launch of their own on the remaining SMs, whatever their D.  Contexts in FP32/FP64 run the SIMT kernels on
-// forked streams.
+// dimension's runs over its CTAs in near-equal numbers of 4- or 8-run chunks, so no SM
+// idles while another finishes a whole extra item.  The small-N contexts get SMs in
+// proportion to their estimated cost, and each dimension its share of them one SM at a
+// time, the next to the one whose step takes longest.  Contexts on the large-N path run
+// in persistent launches, one per D, on the remaining SMs (k2_integrate).  Contexts in
+// FP32/FP64 and over sparse rows run the SIMT kernels on forked streams.
 #include <math.h>
 
 #include <algorithm>
@@ -33,9 +34,10 @@ struct chym_batch {
   int sms = 0;
   chym::K2Runner k2;
   // Cost model of the planner, in SM-microseconds: one 8- or 4-run chunk advanced
-  // one step on the small-N path, per dimension D (of a full item, see tc_step_chunks); and one (128-row tile x K chunk
-  // of 64) advanced one step on the large-N path.  The defaults were measured on a
-  // GB300; chym_batch_tune re-measures them for the batch's own contexts.
+  // one step on the small-N path, per dimension D (a full item's, see tc_step_chunks);
+  // and one (128-row tile x K chunk of 64) advanced one step on the large-N path.  The
+  // defaults were measured on a GB300; chym_batch_tune re-measures them for the batch's
+  // own contexts.
   double chunk_cost[9] = {0, 0.27, 0.44, 0.70, 0.84, 0.66, 0.70, 0.94, 0.91};
   double k2_cost = 0.65;
   bool tuned = false;
@@ -259,7 +261,7 @@ CHYM_API chym_status chym_batch_run(chym_batch* b, const chym_params* params,
     CHYM_CUDA_TRY(cudaEventRecord(b->joins[si], s));
     used[si++] = true;
   }
-  // ---- large-N tensor-core contexts: one persistent launch over all of them ----
+  // ---- large-N tensor-core contexts: their persistent launches ----
   {
     std::vector<unsigned char> descs;
     std::vector<int> dims, idx;

@@ -1,5 +1,5 @@
-// chym_k2.cu -- large-N step: tcgen05 GEMM Y = J X with the CHYM update fused
-// into its epilogue, one persistent launch per Euler-Maruyama step (N > 128).
+// chym_k2.cu -- large-N step (N > 128): tcgen05 GEMM Y = J X with the CHYM update fused
+// into its epilogue, one persistent launch per D and kLaunchSteps Euler-Maruyama steps.
 //
 // Layouts (device, internal to this path), per context:
 //   Xm[c][p]   FP32 master state, column c = r * D + mu, spin p contiguous,
@@ -26,27 +26,29 @@
 // that x_lo S sits in the normal range of e4m3 (|x_lo| <= 2^-9 |x|); the hi and lo
 // products add into one FP32 accumulator holding S y, and the epilogue folds 1/S
 // into dt eps.  x_lo then keeps 4 significant bits: x = hi + lo within 2^-13 |x|.
-// One launch advances every context of a call (any mix of D) by all its steps.  Work is a
-// table of tiles (context, M tile mt, column tile ct), given to the CTAs once per call in
-// lists of near-equal cost (longest tile first, mt fastest so that the CTAs that run at the
-// same time share their column tile's B blocks in L2); a CTA, one per SM, walks its list
-// once per step, and its three roles walk it independently:
-//   warp 0  producer: waits until all MT tiles of the column tile have finished the previous
-//           step (a counter per column tile in global memory), then fills a ring of up to
-//           8 stages with TMA bulk copies of the A / B_hi / B_lo blocks of each K chunk
-//           (mbarrier expect_tx);
+// A launch advances every context of its D in the call.  Work is a table of tiles (context,
+// M tile mt, column tile ct), dealt to the CTAs once per call: in phases of a few tiles a CTA,
+// each advanced by all steps of the launch before the next, the tiles of a phase in lists of
+// near-equal cost (costliest first, mt fastest so that the CTAs that run at the same time
+// share their column tile's B blocks in L2).  A CTA, one per SM, walks its list of the phase
+// once per step; its five roles walk it independently:
+//   warp 3  scout: waits until all MT tiles of the column tile have finished the previous
+//           step (a counter per column tile in global memory) and clears the tile;
+//   warp 0  producer: fills a ring of up to 8 stages with TMA bulk copies of the A / B_hi /
+//           B_lo blocks of each K chunk of a cleared tile (mbarrier expect_tx);
 //   warp 1  MMA issuer: tcgen05.mma (M = 128, N = n, K = 16), J_hi X_hi +
 //           J_hi X_lo (+ J_lo X_hi), FP32 accumulators in TMEM, two of them so
 //           that the next tile's products run while the epilogue drains the last;
-//   warps 2-17 epilogue: thread = spin (TMEM lane) x a quarter of the tile's runs; it
+//   warps 4-11 epilogue: thread = spin (TMEM lane) x half of the tile's runs; it
 //           loads its runs' x (global) before the accumulator is ready, then reads
 //           Y (tcgen05.ld), applies drift, loss, annealing and Philox noise (text
 //           after Eq. 1 and after Fig. 2), writes x back and the new BF16 hi/lo
 //           straight into the other buffer (the next step's B blocks).  Per-run
 //           quantities (round keys, the rounds of Philox that depend on the run and step
 //           only, annealing scale) are staged per warp in shared memory;
-//   warp 18 publisher: once the tile's stores (generic proxy) are issued, fences towards the
-//           async proxy of the other SMs' TMA and adds 1 to the column tile's counter.
+//   warp 2  publisher: once every epilogue warp has stored the tile (generic proxy), fences
+//           towards the async proxy of the other SMs' TMA and adds 1 to the column tile's
+//           counter.
 // A column tile depends on its own tiles of the previous step only, so there is no barrier
 // over a step: tiles of other column tiles and contexts fill the time of its hand-over.
 // (One launch per step and D, graph-replayed, measured: 32 uneven instances 187 us a step,
@@ -119,8 +121,8 @@ constexpr double kLaunchNs = 10000.0;          // start and end of a launch
 constexpr uint32_t kA8Block = 128 * kKc;       // bytes of an e4m3 A block (4 KB)
 constexpr int kLoScaleLog2 = 16;               // FP8 mode: B operands carry 2^16
 
-// Runs per column tile: a multiple of 32 (whole 4-run blocks for each of the four
-// warps of a TMEM lane quarter, and n = D * RT a multiple of 16), n <= 256.
+// Most runs per column tile (n = D * RT <= 256).  Any RT is a multiple of 8 (the epilogue's
+// units) with n a multiple of 16: 32 and its multiples, or 16 and 24 from k2_pick_rt.
 __host__ __device__ constexpr int k2_rt_max(int D) {
   return D == 1 ? 256 : D == 2 ? 128 : D <= 4 ? 64 : 32;
 }

@@ -62,8 +62,8 @@ struct TcLaunch {
   unsigned long long wait_ns;  // limit of every bounded wait
 };
 
-// CH_ = 0: the default runs per epilogue chunk (8 for D <= 4, else 4); the batch
-// autotuner may choose 4 for D <= 4.
+// CH_: runs per epilogue chunk, 4 or (0) 8, for D <= 3 (tc_pick_chunk, or the batch
+// autotuner's choice); above D = 3 chunks have 4 runs.
 // kATmem: J sits in TMEM beside the accumulators and masters instead of shared memory.  A
 // product of N = 48 columns reads 4 KB of J against 1.5 KB of X, which keeps shared memory
 // busy for its whole 44 cycles (24 from TMEM) and stalls the other groups' epilogues: at
@@ -737,7 +737,7 @@ cudaError_t launch_tc_plan(TcLaunch L, int n_cta, cudaStream_t st) {
   using Cfg = TcCfg<D, CH_>;
   const size_t b_bytes = (size_t)L.kp_max * Cfg::CG * 2u;
   // at least 128 KB: one CTA owns all 512 TMEM columns of its SM, so neither a
-  // second CTA of this kernel nor a large-N step CTA (>= 104 KB) may be placed
+  // second CTA of this kernel nor a large-N step CTA (>= 120 KB) may be placed
   // beside it (it would wait in tcgen05.alloc until this CTA exits)
   if (Cfg::kATmem) L.a_region = 0;
   const size_t smem = std::max<size_t>(L.a_region + (size_t)Cfg::G * 2 * b_bytes, 128 * 1024);
