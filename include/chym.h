@@ -156,7 +156,9 @@ CHYM_API chym_status chym_lambda_max(chym_ctx* ctx, double* lambda_out);
  * step (checkpoint/resume: the noise is counter based, so two calls of K/2
  * steps equal one call of K) and n_runs must match.  The schedule refers to
  * absolute steps.  The call is asynchronous with respect to the host except
- * for the upload of h and seeds.
+ * for the upload of h and seeds.  It spreads its runs over every SM for the shortest
+ * call; several contexts at once are integrated fastest as a batch (below), not by
+ * calls on streams of their own, which take the SMs one after the other.
  * EINVAL: steps < 0, n_h < 1, n_runs not a multiple of n_h, bad params. */
 CHYM_API chym_status chym_run(chym_ctx* ctx, const chym_params* params, const double* h, int n_h,
                      const uint64_t* seeds, int n_runs, int64_t steps,
@@ -296,9 +298,10 @@ CHYM_API chym_status chym_ground_state_search(chym_ctx* ctx, int restarts, int s
  * Fig. 4 are averages over replicas, pump values and graphs), so a batch spreads
  * them over the whole GPU: contexts on the small-N tensor-core path (BF16X2,
  * N <= 128) are integrated by one persistent launch per dimension D whose CTAs walk
- * a host-planned list of run ranges, balanced in whole 8-run chunks across the SMs;
- * the other contexts run their own launches concurrently on forked streams.  The
- * batch keeps the contexts (not owned) and its streams, events and plan buffer. */
+ * a host-planned list of run ranges, balanced in whole chunks of 4 or 8 runs across the
+ * SMs; contexts on the large-N path (N > 128) by one persistent launch per dimension and
+ * 1024 steps; the other contexts run their own launches concurrently on forked streams.
+ * The batch keeps the contexts (not owned) and its streams, events and plan buffer. */
 typedef struct chym_batch chym_batch;
 
 /* ctxs: n_ctx contexts (pointers copied; the contexts must outlive the batch). */
