@@ -158,7 +158,7 @@ CHYM_API chym_status chym_lambda_max(chym_ctx* ctx, double* lambda_out);
  * absolute steps.  The call is asynchronous with respect to the host except
  * for the upload of h and seeds.  It spreads its runs over every SM for the shortest
  * call; several contexts at once are integrated fastest as a batch (below), not by
- * calls on streams of their own, which take the SMs one after the other.
+ * calls on streams of their own, of which at most two share an SM.
  * EINVAL: steps < 0, n_h < 1, n_runs not a multiple of n_h, bad params. */
 CHYM_API chym_status chym_run(chym_ctx* ctx, const chym_params* params, const double* h, int n_h,
                      const uint64_t* seeds, int n_runs, int64_t steps,

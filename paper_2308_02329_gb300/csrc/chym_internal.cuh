@@ -287,7 +287,7 @@ void tc_plan_items(int D, const std::vector<TcJob>& jobs, int chunk, int P, std:
                    std::vector<int>& cta_begin);
 cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, const int* d_cta_begin,
                             int n_cta, int64_t steps, int kp_max, int terms_max, unsigned* status,
-                            cudaStream_t st, bool test_stall = false, int chunk = 0);
+                            cudaStream_t st, bool test_stall = false, int chunk = 0, int groups = 0);
 // Tile shapes the batch autotuner may choose (0: the kernels' defaults).
 struct TileShapes {
   int rt[9] = {};      // large-N path: runs per column tile, per D

@@ -58,6 +58,7 @@ struct TcLaunch {
   int64_t steps;
   uint32_t a_region;     // bytes reserved for the largest J image of the launch
   int kp_max;            // largest K (rows of B) of the launch
+  uint32_t tmem_cols;
   unsigned* status;
   unsigned long long wait_ns;  // limit of every bounded wait
 };
@@ -70,13 +71,15 @@ struct TcLaunch {
 // N = 100 the products of four groups added 1.2 us to a step of 4.8 to 7.2 us, overlapped
 // with nothing.  Groups are as wide as that leaves room for (CG = 48; J takes up to 128
 // columns); at D = 5, 7 and 8 it would cost whole groups, and J stays in shared memory.
-template <int D, int CH_ = 0>
+// G_: warpgroups of a CTA, 0 for the most; 1 and 2 leave room for a second CTA on the SM.
+template <int D, int CH_ = 0, int G_ = 0>
 struct TcCfg {
   static constexpr bool kATmem = D <= 4 || D == 6;
   static constexpr int RG = D == 1 ? 48 : D == 2 ? 24 : D == 4 ? 12 : (D == 6 || D == 8) ? 8 : 16;
   static constexpr int CG = D * RG;        // MMA N: columns of one group
   static constexpr int CH = D <= 3 ? (CH_ ? CH_ : 8) : 4;  // runs per epilogue chunk
-  static constexpr int G = std::min(4, (kATmem ? 384 : 512) / (2 * CG));
+  static constexpr int kMostG = std::min(4, (kATmem ? 384 : 512) / (2 * CG));
+  static constexpr int G = G_ ? G_ : kMostG;
   static constexpr int kACol = 2 * G * CG;  // J's first TMEM column
   static_assert(CG % 16 == 0 && CG <= 256, "MMA N must be a multiple of 16 in [16, 256]");
   static_assert(RG % CH == 0, "chunk must divide the group");
@@ -354,9 +357,9 @@ __device__ __forceinline__ void quad_transpose(float v0, float v1, float v2, flo
   b[3] = high ? ko : ro;
 }
 
-template <int D, int CH_>
-__global__ void __launch_bounds__(128 * TcCfg<D, CH_>::G, 1) step_tc_kernel(TcLaunch L) {
-  using Cfg = TcCfg<D, CH_>;
+template <int D, int CH_, int G_>
+__global__ void __launch_bounds__(128 * TcCfg<D, CH_, G_>::G, G_ ? 2 : 1) step_tc_kernel(TcLaunch L) {
+  using Cfg = TcCfg<D, CH_, G_>;
   constexpr int RG = Cfg::RG, CG = Cfg::CG, CH = Cfg::CH, G = Cfg::G;
   constexpr bool kATmem = Cfg::kATmem;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(128 * TcCfg<D, CH_>::G, 1) step_tc_kernel(TcLa
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_addr(&s_tmem)),
-                 "r"(512));
+                 "r"(L.tmem_cols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
@@ -712,7 +715,7 @@ __global__ void __launch_bounds__(128 * TcCfg<D, CH_>::G, 1) step_tc_kernel(TcLa
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L.tmem_cols));
   }
 }
 
@@ -732,16 +735,25 @@ float bf16_value(uint16_t b) {
   return f;
 }
 
-template <int D, int CH_>
-cudaError_t launch_tc_plan(TcLaunch L, int n_cta, cudaStream_t st) {
-  using Cfg = TcCfg<D, CH_>;
+template <int D, int CH_, int G_ = 0>
+cudaError_t launch_tc_plan(TcLaunch L, int n_cta, int groups, cudaStream_t st) {
+  using Cfg = TcCfg<D, CH_, G_>;
+  if constexpr (G_ == 0) {
+    if (groups == 1) return launch_tc_plan<D, CH_, 1>(L, n_cta, groups, st);
+    if constexpr (Cfg::kMostG > 2 && TcCfg<D, CH_, 2>::kACol <= 256)
+      if (groups == 2) return launch_tc_plan<D, CH_, 2>(L, n_cta, groups, st);
+  }
   const size_t b_bytes = (size_t)L.kp_max * Cfg::CG * 2u;
-  // at least 128 KB: one CTA owns all 512 TMEM columns of its SM, so neither a
-  // second CTA of this kernel nor a large-N step CTA (>= 120 KB) may be placed
-  // beside it (it would wait in tcgen05.alloc until this CTA exits)
+  // all columns, or of few groups those of accumulators, masters and J (two couplings a column)
+  const uint32_t need = (uint32_t)Cfg::kACol + (Cfg::kATmem ? L.a_region / 512u : 0u);
+  L.tmem_cols = G_ == 0 || need > 256 ? 512 : 256;
+  // Shared memory so that no more CTAs fit an SM than its 512 TMEM columns hold (the last would
+  // wait in tcgen05.alloc until one exits): two of 256 columns, 78 KB each, or one, 156 KB,
+  // with neither a small one nor a large-N step CTA (the whole register file) beside it.
+  const size_t least = (L.tmem_cols == 256 ? 78 : 156) * 1024;
   if (Cfg::kATmem) L.a_region = 0;
-  const size_t smem = std::max<size_t>(L.a_region + (size_t)Cfg::G * 2 * b_bytes, 128 * 1024);
-  auto kern = step_tc_kernel<D, CH_>;
+  const size_t smem = std::max<size_t>(L.a_region + (size_t)Cfg::G * 2 * b_bytes, least);
+  auto kern = step_tc_kernel<D, CH_, G_>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<n_cta, 128 * Cfg::G, smem, st>>>(L);
@@ -941,7 +953,7 @@ void tc_plan_items(int D, const std::vector<TcJob>& jobs, int chunk, int P, std:
 // device memory: descs, items and the per-CTA item ranges.
 cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, const int* d_cta_begin,
                             int n_cta, int64_t steps, int kp_max, int terms_max, unsigned* status,
-                            cudaStream_t st, bool test_stall, int chunk) {
+                            cudaStream_t st, bool test_stall, int chunk, int groups) {
   TcLaunch L;
   L.wait_ns = test_stall ? kTestWaitLimitNs : kWaitLimitNs;
   L.descs = (const TcDesc*)d_descs;
@@ -952,14 +964,14 @@ cudaError_t launch_tc_items(int D, const void* d_descs, const void* d_items, con
   L.a_region = (uint32_t)(terms_max * 128 * kp_max * 2);
   L.status = status;
   switch (D) {
-    case 1: return chunk == 4 ? launch_tc_plan<1, 4>(L, n_cta, st) : launch_tc_plan<1, 0>(L, n_cta, st);
-    case 2: return chunk == 4 ? launch_tc_plan<2, 4>(L, n_cta, st) : launch_tc_plan<2, 0>(L, n_cta, st);
-    case 3: return chunk == 4 ? launch_tc_plan<3, 4>(L, n_cta, st) : launch_tc_plan<3, 0>(L, n_cta, st);
-    case 4: return launch_tc_plan<4, 0>(L, n_cta, st);
-    case 5: return launch_tc_plan<5, 0>(L, n_cta, st);
-    case 6: return launch_tc_plan<6, 0>(L, n_cta, st);
-    case 7: return launch_tc_plan<7, 0>(L, n_cta, st);
-    case 8: return launch_tc_plan<8, 0>(L, n_cta, st);
+    case 1: return chunk == 4 ? launch_tc_plan<1, 4>(L, n_cta, groups, st) : launch_tc_plan<1, 0>(L, n_cta, groups, st);
+    case 2: return chunk == 4 ? launch_tc_plan<2, 4>(L, n_cta, groups, st) : launch_tc_plan<2, 0>(L, n_cta, groups, st);
+    case 3: return chunk == 4 ? launch_tc_plan<3, 4>(L, n_cta, groups, st) : launch_tc_plan<3, 0>(L, n_cta, groups, st);
+    case 4: return launch_tc_plan<4, 0>(L, n_cta, groups, st);
+    case 5: return launch_tc_plan<5, 0>(L, n_cta, groups, st);
+    case 6: return launch_tc_plan<6, 0>(L, n_cta, groups, st);
+    case 7: return launch_tc_plan<7, 0>(L, n_cta, groups, st);
+    case 8: return launch_tc_plan<8, 0>(L, n_cta, groups, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -1005,6 +1017,14 @@ cudaError_t launch_step_tc(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   std::vector<unsigned char> items;
   std::vector<int> cta;
   tc_plan_items(c->D, {TcJob{0, sc.n_runs}}, chunk, sms, items, cta);
+  // No more warpgroups than the items have chunks, so that calls on other streams may share the
+  // SMs.  N = 100, D = 3, us a step: eight contexts on streams of their own, 512 runs each 9.9 -> 5.7,
+  // 1216 runs 13.1 -> 8.3; one of 512 runs alone 1.51 -> 1.31, its barriers and registers being
+  // those of one group.  (A batch has the SMs to itself, and its CTAs one each.)
+  int most = 0;
+  for (size_t i = 0; i < items.size(); i += sizeof(TcItem))
+    most = std::max(most, reinterpret_cast<const TcItem*>(items.data() + i)->run_count);
+  const int groups = (most + chunk - 1) / chunk;
   const size_t cta_off = sizeof(TcDesc) + items.size();
   const size_t bytes = cta_off + sizeof(int) * cta.size();
   std::vector<unsigned char> plan(bytes);
@@ -1024,7 +1044,7 @@ cudaError_t launch_step_tc(chym_ctx* c, const StepConsts& sc, cudaStream_t st) {
   const unsigned char* base = (const unsigned char*)c->d_plan;
   return launch_tc_items(c->D, base, base + sizeof(TcDesc), (const int*)(base + cta_off),
                          (int)cta.size() - 1, sc.steps, (c->N + 15) / 16 * 16,
-                         c->kind == CHYM_J_PM1 ? 1 : 2, c->d_status, st, sc.test_stall != 0, chunk);
+                         c->kind == CHYM_J_PM1 ? 1 : 2, c->d_status, st, sc.test_stall != 0, chunk, groups);
 }
 
 }  // namespace chym

@@ -56,3 +56,43 @@ def test_spread_of_several_contexts_leaves_states_unchanged(D, runs):
     b.close()
     for ctx in ctxs:
         ctx.close()
+
+
+@pytest.mark.parametrize("D,R", [(1, 300), (2, 700), (3, 512), (3, 1216), (4, 512), (5, 512), (6, 500), (8, 600)])
+def test_calls_on_several_streams_share_the_sms(D, R):
+    """Eight contexts on streams of their own, few runs an SM each: states as alone, and where
+    two CTAs fit an SM the calls do not queue for whole SMs."""
+    torch = pytest.importorskip("torch")
+    import time
+    n, steps = 8, 800
+    sched = chym.Schedule(1, 300, 600)
+    ctxs, prm, seeds, alone, streams = [], [], [], [], []
+    for i in range(n):
+        real = i % 3 == 2
+        J = inputs.gaussian(100, 3 + i) if real else inputs.sk_pm1(100 - 7 * i, 3 + i)
+        ctx = chym.Context(J, D, chym.J_REAL if real else chym.J_PM1)
+        ctxs.append(ctx)
+        prm.append(chym.Params(eps=0.25 if real else 0.025, prec=chym.PREC_BF16X2))
+        seeds.append(inputs.run_seeds(60 + i, R))
+        ctx.run(prm[i], np.array([0.8]), seeds[i], steps, sched)
+        alone.append(ctx.get_state()[0])
+        streams.append(torch.cuda.Stream())
+
+    def seconds(which):
+        for i in which:
+            ctxs[i].run(prm[i], np.array([0.8]), seeds[i], 0, sched)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        for i in which:
+            ctxs[i].run(prm[i], None, None, steps, sched, streams[i].cuda_stream)
+        torch.cuda.synchronize()
+        return time.perf_counter() - t0
+
+    one = min(max(seconds([i]) for i in (0, 2)) for _ in range(3))
+    t = min(seconds(range(n)) for _ in range(3))
+    for ctx, X in zip(ctxs, alone):
+        assert np.array_equal(ctx.get_state()[0], X)
+    if D == 3 and R == 512:
+        assert t < 5.5 * one, (t, one)
+    for ctx in ctxs:
+        ctx.close()
